@@ -6,7 +6,8 @@
 //   (inference)     8 -> 128 -> 128 -> 1 on the tcgen05 tensor cores: mlp_tc.cu
 //   k_topk_*        per group: keep the `top` best-scored candidates, in list order
 //   training        FP32 forward/backward (strided tiled GEMM, split over K with a
-//                   fixed-order reduction), weighted BCE with logits, AdamW
+//                   fixed-order reduction), weighted BCE with logits, AdamW; with BF16
+//                   operands: train_tc.cu
 //
 // Feature definitions (R = distance from the last, i.e. farthest, candidate of the list to
 // its nearest member -- the group's candidate radius -- or 1 if zero; a* the nearest
@@ -429,28 +430,14 @@ __global__ void k_sum_splits(const float* __restrict__ part, int nz, long long l
     out[i] = s;
 }
 
-__device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
-// W_used = round_bf16(master) (or a copy when bf16 is off)
-__global__ void k_round_params(const float* __restrict__ p, float* __restrict__ q, int n, int bf16) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) q[i] = bf16 ? bf16_round(p[i]) : p[i];
-}
-
-__global__ void k_round_rows(const float* __restrict__ x, float* __restrict__ y, long long n, int bf16) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < n) y[i] = bf16 ? bf16_round(x[i]) : x[i];
-}
-
-// Z += bias (row-broadcast); H = gelu(Z) (H optionally rounded to bf16)
+// Z += bias (row-broadcast); H = gelu(Z)
 __global__ void k_bias_gelu(float* __restrict__ Z, float* __restrict__ H, const float* __restrict__ bias,
-                            long long rows, int bf16) {
+                            long long rows) {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= rows * HID) return;
     float z = Z[i] + bias[i % HID];
     Z[i] = z;
-    float h = gelu_f(z);
-    H[i] = bf16 ? bf16_round(h) : h;
+    H[i] = gelu_f(z);
 }
 
 // s = H2 w3 + b3; per-row loss and dS = (pw y (sigma - 1) + (1 - y) sigma) / B
@@ -526,20 +513,22 @@ __global__ void k_adamw(float* __restrict__ p, float* __restrict__ m, float* __r
     p[i] = p[i] - lr * (mh / (sqrtf(vh) + eps) + wd * p[i]);
 }
 
-// scratch layout of one training step on B rows (floats)
+// scratch layout of one FP32 training step on B rows (floats); the BF16 step has its own over the same
+// buffer (train_tc_floats, and 16-byte alignment)
 struct TrainWs {
     long long B;
     int nz;  // K-splits of the weight-gradient GEMMs
-    long long q() const { return 0; }                        // rounded params, NPARAM
-    long long xr() const { return NPARAM + 15; }             // rounded features B x 8
-    long long z1() const { return xr() + B * NF; }           // B x 128
+    long long z1() const { return 0; }                       // B x 128
     long long h1() const { return z1() + B * HID; }
     long long z2() const { return h1() + B * HID; }
     long long h2() const { return z2() + B * HID; }
     long long ds() const { return h2() + B * HID; }          // B
     long long lrow() const { return ds() + B; }              // B
     long long part() const { return lrow() + B; }            // nz x 128 x 128
-    long long size() const { return part() + (long long)nz * HID * HID; }
+    long long size() const {
+        const long long f32 = part() + (long long)nz * HID * HID, tc = train_tc_floats(B) + 4;
+        return f32 > tc ? f32 : tc;
+    }
 };
 
 TrainWs train_ws(long long B) {
@@ -550,19 +539,9 @@ TrainWs train_ws(long long B) {
     return w;
 }
 
-// the training GEMMs: 128-wide products in BF16 on the tensor cores (gemm_tc) when `tc`, the
-// rest (and everything in the FP32 mode) in the CUDA-core tiled GEMM; K-splits summed in a
-// fixed order either way
+// the FP32 mode's GEMMs, K-splits summed in a fixed order (BF16 steps: train_tc.cu)
 void gemm(cudaStream_t s, int M, int N, int K, const float* A, long long sam, long long sak, const float* B,
-          long long sbk, long long sbn, float* C, int nz, float* part, sic_handle* tc = nullptr) {
-    if (tc && N == HID) {
-        gemm_tc(tc, s, M, K, A, sam, sak, B, sbk, sbn, nz == 1 ? C : part, nz);
-        if (nz > 1) {
-            long long len = (long long)M * N;
-            k_sum_splits<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(part, nz, len, C);
-        }
-        return;
-    }
+          long long sbk, long long sbn, float* C, int nz, float* part) {
     int kchunk = (K + nz - 1) / nz;
     kchunk = (kchunk + 15) / 16 * 16;
     dim3 grid((N + 63) / 64, (M + 63) / 64, nz);
@@ -648,9 +627,11 @@ extern "C" sic_status sic_mlp_grads(sic_handle* h, const float* params, const fl
     if (ws_bytes < sizeof(float) * (size_t)L.size()) return SIC_ERR_INVALID;
     SIC_CUDA_TRY(cudaSetDevice(h->device));
     cudaStream_t s = (cudaStream_t)stream;
+    if (bf16) {
+        float* w = (float*)(((uintptr_t)ws + 15) / 16 * 16);
+        return train_tc(h, params, feat, label, batch, pos_weight, grads, loss, score, w, s);
+    }
     float* W = (float*)ws;
-    float* q = W + L.q();
-    float* xr = W + L.xr();
     float* Z1 = W + L.z1();
     float* H1 = W + L.h1();
     float* Z2 = W + L.z2();
@@ -660,30 +641,26 @@ extern "C" sic_status sic_mlp_grads(sic_handle* h, const float* params, const fl
     float* part = W + L.part();
     const long long B = batch;
     const unsigned ew = (unsigned)((B * HID + 255) / 256);
-    k_round_params<<<(NPARAM + 255) / 256, 256, 0, s>>>(params, q, NPARAM, bf16);
-    k_round_rows<<<(unsigned)((B * NF + 255) / 256), 256, 0, s>>>(feat, xr, B * NF, bf16);
-    // forward (with bf16: the 128-wide products on the tensor cores, operands in BF16)
-    sic_handle* tc = bf16 ? h : nullptr;
-    gemm(s, (int)B, HID, NF, xr, NF, 1, q + OFF_W1, HID, 1, Z1, 1, part, tc);
-    k_bias_gelu<<<ew, 256, 0, s>>>(Z1, H1, q + OFF_B1, B, bf16);
-    gemm(s, (int)B, HID, HID, H1, HID, 1, q + OFF_W2, HID, 1, Z2, 1, part, tc);
-    k_bias_gelu<<<ew, 256, 0, s>>>(Z2, H2, q + OFF_B2, B, 0);
-    k_head<<<(unsigned)((B + 3) / 4), 128, 0, s>>>(H2, q + OFF_W3, q + OFF_B3, label, B, pos_weight, score, dS,
-                                                   lrow);
+    gemm(s, (int)B, HID, NF, feat, NF, 1, params + OFF_W1, HID, 1, Z1, 1, part);
+    k_bias_gelu<<<ew, 256, 0, s>>>(Z1, H1, params + OFF_B1, B);
+    gemm(s, (int)B, HID, HID, H1, HID, 1, params + OFF_W2, HID, 1, Z2, 1, part);
+    k_bias_gelu<<<ew, 256, 0, s>>>(Z2, H2, params + OFF_B2, B);
+    k_head<<<(unsigned)((B + 3) / 4), 128, 0, s>>>(H2, params + OFF_W3, params + OFF_B3, label, B, pos_weight, score,
+                                                   dS, lrow);
     k_sum_loss<<<1, 256, 0, s>>>(lrow, B, loss);
     // backward: w3, b3
     gemm(s, HID, 1, (int)B, H2, 1, HID, dS, 1, 1, grads + OFF_W3, L.nz, part);
     k_colsum<<<1, 32, 0, s>>>(dS, B, 1, grads + OFF_B3);
     // dZ2 into H2's storage (H2 is no longer needed)
-    k_dz2<<<ew, 256, 0, s>>>(dS, q + OFF_W3, Z2, H2, B);
+    k_dz2<<<ew, 256, 0, s>>>(dS, params + OFF_W3, Z2, H2, B);
     float* dZ2 = H2;
-    gemm(s, HID, HID, (int)B, H1, 1, HID, dZ2, HID, 1, grads + OFF_W2, L.nz, part, tc);
+    gemm(s, HID, HID, (int)B, H1, 1, HID, dZ2, HID, 1, grads + OFF_W2, L.nz, part);
     k_colsum<<<1, 128, 0, s>>>(dZ2, B, HID, grads + OFF_B2);
     // dH1 = dZ2 W2^T  -> into Z2's storage, then dZ1 = dH1 .* gelu'(Z1)
-    gemm(s, (int)B, HID, HID, dZ2, HID, 1, q + OFF_W2, 1, HID, Z2, 1, part, tc);
+    gemm(s, (int)B, HID, HID, dZ2, HID, 1, params + OFF_W2, 1, HID, Z2, 1, part);
     float* dZ1 = Z2;
     k_mul_dgelu<<<ew, 256, 0, s>>>(dZ1, Z1, B * HID);
-    gemm(s, NF, HID, (int)B, xr, 1, NF, dZ1, HID, 1, grads + OFF_W1, L.nz, part, tc);
+    gemm(s, NF, HID, (int)B, feat, 1, NF, dZ1, HID, 1, grads + OFF_W1, L.nz, part);
     k_colsum<<<1, 128, 0, s>>>(dZ1, B, HID, grads + OFF_B1);
     SIC_CUDA_TRY(cudaGetLastError());
     return SIC_OK;
