@@ -1,11 +1,11 @@
-// Supernodal greedy selection (Section 5.2, multiple targets sharing one selection).
-// (FP32 with at most 256 candidates, m <= 64 and k <= 64 goes to the register-resident
-// kernel of select_agg_reg.cu.)
+// Supernodal greedy selection (Section 5.2, multiple targets sharing one selection)
+// in FP32: supernodes beyond the register-resident kernel of select_agg_reg.cu (at most 256
+// candidates and k <= 64); double precision is select_fx.cu.
 //
 // One CTA owns one group at a time over a persistent grid.  The two partial Cholesky
 // factors of the paper's Cholesky approach (Appendix C.2) live in shared memory when
 // they fit (e.g. 256 candidates in FP32) and otherwise in a per-CTA slab of the
-// caller's workspace.  Layout (elements of T), column-major so that thread r touches
+// caller's workspace.  Layout (floats), column-major so that thread r touches
 // row r of every column:
 //   F1  [k][Cm]       columns of the picks, conditioned on earlier picks only;
 //   F2c [mm+k][Cm]    candidate rows of F2: first the m target columns (left-looking
@@ -26,17 +26,15 @@
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ bool better(T s, int i, T bs, int bi) {
+__device__ __forceinline__ bool better(float s, int i, float bs, int bi) {
     return s > bs || (s == bs && i < bi);
 }
 
 // acc - sum_{tau < len} col[tau * ld] * piv[tau], with four independent partial sums so
 // that the loads of consecutive terms are in flight together
-template <typename T>
-__device__ __forceinline__ T dot_down(T acc, const T* __restrict__ col, long long ld, const T* __restrict__ piv,
+__device__ __forceinline__ float dot_down(float acc, const float* __restrict__ col, long long ld, const float* __restrict__ piv,
                                       int len) {
-    T a1 = (T)0, a2 = (T)0, a3 = (T)0;
+    float a1 = 0.f, a2 = 0.f, a3 = 0.f;
     int tau = 0;
     for (; tau + 4 <= len; tau += 4) {
         acc = fma(-col[(long long)tau * ld], piv[tau], acc);
@@ -80,45 +78,35 @@ inline AggLayout agg_layout(int max_cand, int max_m, int k, bool rowmajor) {
 }
 
 // acc - sum_{tau < len} row[tau] * piv[tau] over a contiguous row (shared memory)
-template <typename T>
-__device__ __forceinline__ T dot_row(T acc, const T* __restrict__ row, const T* __restrict__ piv, int len) {
-    T a1 = (T)0, a2 = (T)0, a3 = (T)0;
+__device__ __forceinline__ float dot_row(float acc, const float* __restrict__ row, const float* __restrict__ piv, int len) {
+    float a1 = 0.f, a2 = 0.f, a3 = 0.f;
     int tau = 0;
-    if constexpr (sizeof(T) == 4) {
-        const float4* r4 = reinterpret_cast<const float4*>(row);
-        const float4* p4 = reinterpret_cast<const float4*>(piv);
-        for (; tau + 4 <= len; tau += 4) {
-            const float4 a = r4[tau >> 2], b = p4[tau >> 2];
-            acc = fmaf(-a.x, b.x, acc);
-            a1 = fmaf(-a.y, b.y, a1);
-            a2 = fmaf(-a.z, b.z, a2);
-            a3 = fmaf(-a.w, b.w, a3);
-        }
-    } else {
-        for (; tau + 4 <= len; tau += 4) {
-            acc = fma(-row[tau], piv[tau], acc);
-            a1 = fma(-row[tau + 1], piv[tau + 1], a1);
-            a2 = fma(-row[tau + 2], piv[tau + 2], a2);
-            a3 = fma(-row[tau + 3], piv[tau + 3], a3);
-        }
+    const float4* r4 = reinterpret_cast<const float4*>(row);
+    const float4* p4 = reinterpret_cast<const float4*>(piv);
+    for (; tau + 4 <= len; tau += 4) {
+        const float4 a = r4[tau >> 2], b = p4[tau >> 2];
+        acc = fmaf(-a.x, b.x, acc);
+        a1 = fmaf(-a.y, b.y, a1);
+        a2 = fmaf(-a.z, b.z, a2);
+        a3 = fmaf(-a.w, b.w, a3);
     }
     for (; tau < len; ++tau) acc = fma(-row[tau], piv[tau], acc);
     return (acc + a1) + (a2 + a3);
 }
 
-template <typename T, int NT, bool SMEM>
+template <int NT, bool SMEM>
 __global__ void __launch_bounds__(NT, 1) k_select_agg(
-    const double* __restrict__ pts, long long n, int dim, KP<T> kp, T floor_, const long long* __restrict__ grp_ptr,
+    const double* __restrict__ pts, long long n, int dim, KP<float> kp, float floor_, const long long* __restrict__ grp_ptr,
     long long n_grp, const long long* __restrict__ cand_ptr, const int32_t* __restrict__ cand_idx, int max_cand,
-    int max_m, int k, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_count, T* __restrict__ ws,
+    int max_m, int k, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_count, float* __restrict__ ws,
     AggLayout L, double* __restrict__ gain, DevStatus* st) {
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sm = reinterpret_cast<T*>(smem_raw);
-    T* base = SMEM ? sm : ws + (long long)blockIdx.x * L.size();
-    T* p1 = SMEM ? sm + L.size() : sm;       // k (16-byte aligned: L.size() is a multiple of 4)
-    T* p2 = p1 + (k + 3) / 4 * 4;             // max_m + k
-    __shared__ T wsc[NW];
+    float* sm = reinterpret_cast<float*>(smem_raw);
+    float* base = SMEM ? sm : ws + (long long)blockIdx.x * L.size();
+    float* p1 = SMEM ? sm + L.size() : sm;       // k (16-byte aligned: L.size() is a multiple of 4)
+    float* p2 = p1 + (k + 3) / 4 * 4;             // max_m + k
+    __shared__ float wsc[NW];
     __shared__ int wix[NW];
     __shared__ int s_fail;
     __shared__ double gv1[128], gv2[128];  // the picks' two conditional variances (gains only)
@@ -130,35 +118,18 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
 #define E1(r, c) (SMEM ? F1[(long long)(r) * P1 + (c)] : F1[(long long)(c) * Cm + (r)])
 #define E2(r, c) (SMEM ? F2c[(long long)(r) * P2 + (c)] : F2c[(long long)(c) * Cm + (r)])
 #define E2T(a, c) (SMEM ? F2t[(long long)(a) * P2t + (c)] : F2t[(long long)(c) * mm + (a)])
-    T* F1 = base + L.f1();
-    T* F2c = base + L.f2c();
-    T* F2t = base + L.f2t();
-    T* X = base + L.x();
-    T* V1 = base + L.v1();
-    T* V2 = base + L.v2();
+    float* F1 = base + L.f1();
+    float* F2c = base + L.f2c();
+    float* F2t = base + L.f2t();
+    float* X = base + L.x();
+    float* V1 = base + L.v1();
+    float* V2 = base + L.v2();
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const T NEG = -INFINITY;
-    const T diag = kp.s2 + kp.nugget;
-    // FP64: Theta by the fill's table-driven exp and Newton square root (about 2 ulp); the
-    // table s2 2^(j/256) follows the pivot rows
-    double* tab = reinterpret_cast<double*>(p2 + (L.mm + k));
-    if constexpr (sizeof(T) == 8) {
-        exp_table_fill(tab, kp.s2);
-        __syncthreads();
-    }
-    auto theta = [&](T d2) -> T {
-        if constexpr (sizeof(T) == 8)
-            return matern_d2_fast(kp, d2, tab);
-        else
-            return matern<T>(kp, sic_sqrt(d2));
-    };
-    auto rsqrt_t = [](T v) -> T {
-        if constexpr (sizeof(T) == 8)
-            return rsqrt_newton(v);
-        else
-            return (T)1 / sic_sqrt(v);
-    };
+    const float NEG = -INFINITY;
+    const float diag = kp.s2 + kp.nugget;
+    auto theta = [&](float d2) -> float { return matern<float>(kp, sic_sqrt(d2)); };
+    auto rsqrt_t = [](float v) -> float { return (float)1 / sic_sqrt(v); };
 
     for (long long g = blockIdx.x; g < n_grp; g += gridDim.x) {
         const long long g0 = grp_ptr[g];
@@ -174,8 +145,7 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
             continue;
         }
         double org[3] = {0.0, 0.0, 0.0};
-        if constexpr (sizeof(T) == 4)
-            for (int d = 0; d < dim; ++d) org[d] = pts[g0 * dim + d];
+        for (int d = 0; d < dim; ++d) org[d] = pts[g0 * dim + d];
         for (int i = tid; i < C + m; i += NT) {
             const bool cnd = i < C;
             long long p = cnd ? (long long)cand_idx[b0 + i] : g0 + (i - C);
@@ -186,7 +156,7 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
                 p = g0;
                 ok = false;
             }
-            for (int d = 0; d < 3; ++d) X[d * ldx + xi] = (d < dim) ? (T)(pts[p * dim + d] - org[d]) : (T)0;
+            for (int d = 0; d < 3; ++d) X[d * ldx + xi] = (d < dim) ? (float)(pts[p * dim + d] - org[d]) : 0.f;
             if (cnd) {
                 V1[i] = ok ? diag : NEG;
                 V2[i] = ok ? diag : NEG;
@@ -199,38 +169,38 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
         for (int a = 0; a < m; ++a) {
             if (tid < a) p2[tid] = E2T(a, tid);
             __syncthreads();
-            T dv = diag;
+            float dv = diag;
             for (int b = 0; b < a; ++b) dv = fma(-p2[b], p2[b], dv);
-            if (!(dv > (T)0)) {
+            if (!(dv > 0.f)) {
                 if (tid == 0) {
                     record_error(st, SIC_ERR_NOT_PD, g);
                     s_fail = 1;
                 }
                 break;
             }
-            const T dsq = sic_sqrt(dv);
-            const T rs = (T)1 / dsq;
+            const float dsq = sic_sqrt(dv);
+            const float rs = (float)1 / dsq;
             const long long xa = Cm + a;
-            const T ax = X[xa], ay = X[ldx + xa], az = X[2 * ldx + xa];
+            const float ax = X[xa], ay = X[ldx + xa], az = X[2 * ldx + xa];
             for (int i = tid; i < C + m; i += NT) {
                 if (i < C) {
-                    T dx = X[i] - ax, dy = X[ldx + i] - ay, dz = X[2 * ldx + i] - az;
-                    T num = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
+                    float dx = X[i] - ax, dy = X[ldx + i] - ay, dz = X[2 * ldx + i] - az;
+                    float num = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
                     num = SMEM ? dot_row(num, F2c + (long long)i * P2, p2, a) : dot_down(num, F2c + i, Cm, p2, a);
-                    const T u = num * rs;
+                    const float u = num * rs;
                     E2(i, a) = u;
                     V2[i] = fma(-u, u, V2[i]);
                 } else {
                     const int ta = i - C;
-                    T u;
+                    float u;
                     if (ta < a) {
-                        u = (T)0;
+                        u = 0.f;
                     } else if (ta == a) {
                         u = dsq;
                     } else {
                         const long long xt = Cm + ta;
-                        T dx = X[xt] - ax, dy = X[ldx + xt] - ay, dz = X[2 * ldx + xt] - az;
-                        T num = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
+                        float dx = X[xt] - ax, dy = X[ldx + xt] - ay, dz = X[2 * ldx + xt] - az;
+                        float num = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
                         num = SMEM ? dot_row(num, F2t + (long long)ta * P2t, p2, a) : dot_down(num, F2t + ta, mm, p2, a);
                         u = num * rs;
                     }
@@ -243,18 +213,18 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
         int t = 0;
         if (!s_fail) {
             for (; t < k; ++t) {
-                T bs = NEG;
+                float bs = NEG;
                 int bi = 0x7fffffff;
                 for (int r = tid; r < C; r += NT) {
-                    T v2 = V2[r];
+                    float v2 = V2[r];
                     if (v2 >= floor_) {
-                        T s = V1[r] / v2;
+                        float s = V1[r] / v2;
                         if (better(s, r, bs, bi)) { bs = s; bi = r; }
                     }
                 }
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
-                    T os = __shfl_xor_sync(0xffffffffu, bs, off);
+                    float os = __shfl_xor_sync(0xffffffffu, bs, off);
                     int oi = __shfl_xor_sync(0xffffffffu, bi, off);
                     if (better(os, oi, bs, bi)) { bs = os; bi = oi; }
                 }
@@ -263,28 +233,28 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
                     wix[warp] = bi;
                 }
                 __syncthreads();
-                T gs = wsc[0];
+                float gs = wsc[0];
                 int q = wix[0];
 #pragma unroll
                 for (int w = 1; w < NW; ++w)
                     if (better(wsc[w], wix[w], gs, q)) { gs = wsc[w]; q = wix[w]; }
                 if (q == 0x7fffffff) break;
-                const T v1q = V1[q], v2q = V2[q];
-                const T qx = X[q], qy = X[ldx + q], qz = X[2 * ldx + q];
+                const float v1q = V1[q], v2q = V2[q];
+                const float qx = X[q], qy = X[ldx + q], qz = X[2 * ldx + q];
                 for (int tau = tid; tau < t; tau += NT) p1[tau] = E1(q, tau);
                 for (int tau = tid; tau < m + t; tau += NT) p2[tau] = E2(q, tau);
                 __syncthreads();
-                const T r1 = rsqrt_t(v1q);
-                const T r2 = rsqrt_t(v2q);
+                const float r1 = rsqrt_t(v1q);
+                const float r2 = rsqrt_t(v2q);
                 for (int r = tid; r < C; r += NT) {
                     if (V2[r] == NEG) continue;
-                    T dx = X[r] - qx, dy = X[ldx + r] - qy, dz = X[2 * ldx + r] - qz;
-                    T th = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
+                    float dx = X[r] - qx, dy = X[ldx + r] - qy, dz = X[2 * ldx + r] - qz;
+                    float th = theta(fma(dz, dz, fma(dy, dy, dx * dx)));
                     if (r == q) th += kp.nugget;
-                    const T n1 = SMEM ? dot_row(th, F1 + (long long)r * P1, p1, t) : dot_down(th, F1 + r, Cm, p1, t);
-                    const T n2 = SMEM ? dot_row(th, F2c + (long long)r * P2, p2, m + t)
+                    const float n1 = SMEM ? dot_row(th, F1 + (long long)r * P1, p1, t) : dot_down(th, F1 + r, Cm, p1, t);
+                    const float n2 = SMEM ? dot_row(th, F2c + (long long)r * P2, p2, m + t)
                                       : dot_down(th, F2c + r, Cm, p2, m + t);
-                    const T u1 = n1 * r1, u2 = n2 * r2;
+                    const float u1 = n1 * r1, u2 = n2 * r2;
                     E1(r, t) = u1;
                     E2(r, m + t) = u2;
                     if (r == q) {
@@ -323,11 +293,9 @@ __global__ void __launch_bounds__(NT, 1) k_select_agg(
 
 constexpr size_t SMEM_LIMIT = 227 * 1024 - 4096;  // dynamic part; the static arrays take < 4 KB
 
-template <typename T>
 size_t agg_smem_bytes(const AggLayout& L, bool in_smem) {
-    size_t piv = sizeof(T) * (size_t)((L.k + 3) / 4 * 4 + L.mm + L.k);
-    const size_t tab = sizeof(T) == 8 ? sizeof(double) * EXP_TAB : 0;  // the FP64 Matern's exp table
-    return (in_smem ? sizeof(T) * (size_t)L.size() + piv : piv) + tab;
+    size_t piv = sizeof(float) * (size_t)((L.k + 3) / 4 * 4 + L.mm + L.k);
+    return in_smem ? sizeof(float) * (size_t)L.size() + piv : piv;
 }
 
 // Plan of one launch: where the state lives, threads per CTA, grid, workspace.
@@ -340,9 +308,9 @@ struct AggPlan {
     size_t ws_bytes;
 };
 
-template <typename T, int NT, bool SMEM>
+template <int NT, bool SMEM>
 int agg_grid_for(sic_handle* h, size_t smem, long long n_grp) {
-    auto kern = k_select_agg<T, NT, SMEM>;
+    auto kern = k_select_agg<NT, SMEM>;
     // opt in at any size: the static arrays count against the 48 KB default as well
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int g = persistent_grid(h, kern, NT, smem, n_grp);
@@ -358,11 +326,10 @@ int agg_grid_for(sic_handle* h, size_t smem, long long n_grp) {
 // it), that plan when it is possible.  Every plan gives the same picks: each candidate row's
 // arithmetic and the argmax's tie-break do not depend on the thread count, and the shared-
 // memory and workspace dot products sum in the same order.
-template <typename T>
 AggPlan agg_plan(sic_handle* h, long long n_grp, int max_cand, int max_m, int k, int variant = 0) {
     AggPlan P;
     P.L = agg_layout(max_cand, max_m, k, true);
-    P.smem = agg_smem_bytes<T>(P.L, true) <= SMEM_LIMIT;
+    P.smem = agg_smem_bytes(P.L, true) <= SMEM_LIMIT;
     P.nt = (max_cand <= 256) ? 256 : 512;
     if (variant) {
         const int vnt = variant / 2;
@@ -370,15 +337,15 @@ AggPlan agg_plan(sic_handle* h, long long n_grp, int max_cand, int max_m, int k,
         if (!(variant & 1)) P.smem = false;
     }
     if (!P.smem) P.L = agg_layout(max_cand, max_m, k, false);
-    P.smem_bytes = agg_smem_bytes<T>(P.L, P.smem);
+    P.smem_bytes = agg_smem_bytes(P.L, P.smem);
     long long work = n_grp > 0 ? n_grp : 1;
     if (P.nt == 256)
-        P.grid = P.smem ? agg_grid_for<T, 256, true>(h, P.smem_bytes, work)
-                        : agg_grid_for<T, 256, false>(h, P.smem_bytes, work);
+        P.grid = P.smem ? agg_grid_for<256, true>(h, P.smem_bytes, work)
+                        : agg_grid_for<256, false>(h, P.smem_bytes, work);
     else
-        P.grid = P.smem ? agg_grid_for<T, 512, true>(h, P.smem_bytes, work)
-                        : agg_grid_for<T, 512, false>(h, P.smem_bytes, work);
-    P.ws_bytes = P.smem ? 0 : sizeof(T) * (size_t)P.L.size() * (size_t)P.grid;
+        P.grid = P.smem ? agg_grid_for<512, true>(h, P.smem_bytes, work)
+                        : agg_grid_for<512, false>(h, P.smem_bytes, work);
+    P.ws_bytes = P.smem ? 0 : sizeof(float) * (size_t)P.L.size() * (size_t)P.grid;
     return P;
 }
 
@@ -393,33 +360,32 @@ extern "C" sic_status sic_select_aggregated_workspace(sic_handle* h, int64_t n_g
     if (agg_reg_applies(prec, max_cand, max_m, k))
         *bytes = agg_reg_workspace(n_grp, max_m);
     else if (prec == SIC_FP64)
-        *bytes = agg_plan<double>(h, n_grp, max_cand, max_m, k).ws_bytes;
+        *bytes = fx_plan_groups(h, n_grp, max_cand, max_m, k, 0).ws_bytes;
     else if (prec == SIC_FP32_MIXED)
-        *bytes = agg_plan<float>(h, n_grp, max_cand, max_m, k).ws_bytes;
+        *bytes = agg_plan(h, n_grp, max_cand, max_m, k).ws_bytes;
     else
         return SIC_ERR_INVALID;
     return SIC_OK;
 }
 
 namespace {
-template <typename T>
 sic_status launch_agg(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, const int64_t* grp_ptr,
                       int64_t n_grp, const int64_t* cand_ptr, const int32_t* cand_idx, int max_cand, int max_m, int k,
                       int32_t* sel_idx, int32_t* sel_count, double* gain, void* ws, size_t ws_bytes,
                       cudaStream_t s) {
-    const int prec = sizeof(T) == 8 ? SIC_FP64 : SIC_FP32_MIXED;
+    const int prec = SIC_FP32_MIXED;
     const int variant = tune_get(h, TUNE_SELECT_AGG, tune_select_key_a(k, prec), tune_select_key_b(max_cand, max_m), 0);
-    AggPlan P = agg_plan<T>(h, n_grp, max_cand, max_m, k, variant);
+    AggPlan P = agg_plan(h, n_grp, max_cand, max_m, k, variant);
     if (variant && P.ws_bytes > 0 && (!ws || ws_bytes < P.ws_bytes))
-        P = agg_plan<T>(h, n_grp, max_cand, max_m, k);  // the tuned plan needs more workspace than given
+        P = agg_plan(h, n_grp, max_cand, max_m, k);  // the tuned plan needs more workspace than given
     if (P.ws_bytes > 0 && (!ws || ws_bytes < P.ws_bytes)) return SIC_ERR_INVALID;
-    KP<T> kpt = make_kp<T>(*kp);
-    T fl = (T)sic_floor_of(kp);
+    KP<float> kpt = make_kp<float>(*kp);
+    float fl = (float)sic_floor_of(kp);
     const long long* gp = (const long long*)grp_ptr;
     const long long* cp = (const long long*)cand_ptr;
 #define SIC_AGG_LAUNCH(NTV, SM)                                                                                   \
-    k_select_agg<T, NTV, SM><<<P.grid, NTV, P.smem_bytes, s>>>(pts, n, kp->dim, kpt, fl, gp, n_grp, cp, cand_idx, \
-                                                               max_cand, max_m, k, sel_idx, sel_count, (T*)ws,    \
+    k_select_agg<NTV, SM><<<P.grid, NTV, P.smem_bytes, s>>>(pts, n, kp->dim, kpt, fl, gp, n_grp, cp, cand_idx, \
+                                                               max_cand, max_m, k, sel_idx, sel_count, (float*)ws,    \
                                                                P.L, gain, h->d_status)
     if (P.nt == 256) {
         if (P.smem) SIC_AGG_LAUNCH(256, true); else SIC_AGG_LAUNCH(256, false);
@@ -449,11 +415,17 @@ extern "C" sic_status sic_select_aggregated_gain(sic_handle* h, const double* pt
     if (agg_reg_applies(prec, max_cand, max_m, k))
         return launch_agg_reg(h, pts, n, kp, grp_ptr, n_grp, cand_ptr, cand_idx, max_cand, max_m, k, sel_idx,
                               sel_count, gain, ws, ws_bytes, s);
-    if (prec == SIC_FP64)
-        return launch_agg<double>(h, pts, n, kp, grp_ptr, n_grp, cand_ptr, cand_idx, max_cand, max_m, k, sel_idx,
-                                  sel_count, gain, ws, ws_bytes, s);
+    if (prec == SIC_FP64) {
+        const int variant = tune_get(h, TUNE_SELECT_AGG, tune_select_key_a(k, prec), tune_select_key_b(max_cand, max_m), 0);
+        FxPlan P = fx_plan_groups(h, n_grp, max_cand, max_m, k, variant / 2);
+        if (variant && P.ws_bytes > 0 && (!ws || ws_bytes < P.ws_bytes))
+            P = fx_plan_groups(h, n_grp, max_cand, max_m, k, 0);  // the tuned plan needs more workspace than given
+        if (P.ws_bytes > 0 && (!ws || ws_bytes < P.ws_bytes)) return SIC_ERR_INVALID;
+        return launch_fx_groups(h, P, pts, n, kp, grp_ptr, n_grp, cand_ptr, cand_idx, max_cand, max_m, k, sel_idx,
+                                sel_count, gain, ws, s);
+    }
     if (prec == SIC_FP32_MIXED)
-        return launch_agg<float>(h, pts, n, kp, grp_ptr, n_grp, cand_ptr, cand_idx, max_cand, max_m, k, sel_idx,
+        return launch_agg(h, pts, n, kp, grp_ptr, n_grp, cand_ptr, cand_idx, max_cand, max_m, k, sel_idx,
                                  sel_count, gain, ws, ws_bytes, s);
     return SIC_ERR_INVALID;
 }
@@ -476,13 +448,12 @@ extern "C" sic_status sic_select_aggregated(sic_handle* h, const double* pts, in
 // max_m), later sic_select_aggregated calls launch it, and the outputs of a final run with it
 // are left in sel_idx / sel_count.
 namespace {
-template <typename T>
 int agg_variants(sic_handle* h, long long n_grp, int max_cand, int max_m, int k, size_t ws_bytes, int* out) {
     int nv = 0;
     for (int nt : {256, 512})
         for (int sm = 1; sm >= 0; --sm) {
             const int v = 2 * nt + sm;
-            AggPlan P = agg_plan<T>(h, n_grp, max_cand, max_m, k, v);
+            AggPlan P = agg_plan(h, n_grp, max_cand, max_m, k, v);
             if (P.nt != nt || (int)P.smem != sm || P.ws_bytes > ws_bytes) continue;  // not possible here
             out[nv++] = v;
         }
@@ -504,10 +475,14 @@ extern "C" sic_status sic_tune_select_aggregated(sic_handle* h, const double* pt
     if (agg_reg_applies(prec, max_cand, max_m, k)) {
         vars[nv++] = 256;
         if (max_cand <= 128) vars[nv++] = 128;
-    } else if (prec == SIC_FP64) {
-        nv = agg_variants<double>(h, n_grp, max_cand, max_m, k, ws ? ws_bytes : 0, vars);
+    } else if (prec == SIC_FP64) {  // threads per CTA; what does not fit in shared memory is in the workspace
+        for (int nt : {128, 256, 512, 1024}) {
+            if ((nt == 128 && max_cand > 128) || (nt == 1024 && max_cand <= 512)) continue;
+            const FxPlan P = fx_plan_groups(h, n_grp, max_cand, max_m, k, nt);
+            if (P.ws_bytes <= (ws ? ws_bytes : 0)) vars[nv++] = 2 * nt + (P.ws_bytes == 0);
+        }
     } else {
-        nv = agg_variants<float>(h, n_grp, max_cand, max_m, k, ws ? ws_bytes : 0, vars);
+        nv = agg_variants(h, n_grp, max_cand, max_m, k, ws ? ws_bytes : 0, vars);
     }
     if (nv == 0) return SIC_ERR_INVALID;  // no plan fits the given workspace
     cudaStream_t s = (cudaStream_t)stream;

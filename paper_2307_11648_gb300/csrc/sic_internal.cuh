@@ -246,6 +246,81 @@ __device__ __forceinline__ double matern_d2_fast(const KP<double>& k, double d2,
     return fma(fma(t, 1.0 / 3.0, 1.0), t * e, e);
 }
 
+// ---- exact squared distances in integer arithmetic (the fill and the FP64 selections) ----
+
+// A coordinate x in fixed point at the largest biased exponent E of its dimension in the unit:
+// x 2^(1084 - E), so that |x_fix| < 2^62; exact for every x whose exponent is within 9 of E (a
+// unit's points are near one another: their coordinates share the exponent unless they are
+// within a few length scales of zero, where the truncation below 2^(E - 1085) is far below an
+// ulp of the kernel entries).  Integer operations only.
+__device__ __forceinline__ long long fx_coord(double x, int E) {
+    const long long u = __double_as_longlong(x);
+    const int e = (int)((u >> 52) & 0x7ff);
+    if (!e) return 0LL;
+    const long long mant = (u & 0xfffffffffffffLL) | 0x10000000000000LL;
+    const int sh = E - e;  // >= 0
+    const long long f = sh <= 9 ? (mant << (9 - sh)) : (sh - 9 < 63 ? (mant >> (sh - 9)) : 0LL);
+    return u < 0 ? -f : f;
+}
+
+// dx^2 of one dimension, exact in 128 bits (h:l), for a difference |dx| < 2^63
+__device__ __forceinline__ void sq128(long long dx, unsigned long long& h, unsigned long long& l) {
+    const unsigned long long a = dx < 0 ? 0ULL - (unsigned long long)dx : (unsigned long long)dx;
+    const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+    const unsigned long long q0 = (unsigned long long)al * al;
+    const unsigned long long q1 = ((unsigned long long)ah * al) << 1;  // ah < 2^31
+    l = q0 + (q1 << 32);
+    h = (unsigned long long)ah * ah + (q1 >> 32) + (l < q0 ? 1ULL : 0ULL);
+}
+
+// The squared distance between points i and j from their fixed-point coordinates (xf[d ld + i],
+// scale 2^(1084 - E_d) in dimension d): each dimension's square exact in 128 bits, aligned to the
+// largest scale (a right shift, dropping bits below 2^-125 of the largest term), summed and
+// rounded once to FP64 (to nearest, ties away from zero).  Integer operations only.
+__device__ __forceinline__ double fx_dist2(const long long* __restrict__ xf, int ld, int dim, int i, int j, int E0,
+                                           int E1, int E2) {
+    const int Em = max(E0, max(dim > 1 ? E1 : 0, dim > 2 ? E2 : 0));
+    unsigned long long h = 0ULL, l = 0ULL;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (d >= dim) break;
+        unsigned long long sh, sl;
+        sq128(xf[d * ld + i] - xf[d * ld + j], sh, sl);
+        const int s = 2 * (Em - (d == 0 ? E0 : (d == 1 ? E1 : E2)));
+        if (s >= 128) {
+            sh = sl = 0ULL;
+        } else if (s >= 64) {
+            sl = sh >> (s - 64);
+            sh = 0ULL;
+        } else if (s > 0) {
+            sl = (sl >> s) | (sh << (64 - s));
+            sh >>= s;
+        }
+        l += sl;
+        h += sh + (l < sl ? 1ULL : 0ULL);
+    }
+    if ((h | l) == 0ULL) return 0.0;
+    int p;
+    unsigned long long t;  // the leading 64 bits, leading bit at 63
+    if (h) {
+        const int z = __clzll((long long)h);
+        p = 127 - z;
+        t = z ? ((h << z) | (l >> (64 - z))) : h;
+    } else {
+        const int z = __clzll((long long)l);
+        p = 63 - z;
+        t = l << z;
+    }
+    unsigned long long mt = ((t >> 10) + 1ULL) >> 1;  // 53 bits, rounded
+    if (mt >> 53) {
+        mt >>= 1;
+        ++p;
+    }
+    const int be = p + 2 * Em - 1145;  // |X| 2^(2 Em - 2168) = (mt 2^-52) 2^(p + 2 Em - 2168)
+    if (be <= 0) return 0.0;
+    return __longlong_as_double((long long)(((unsigned long long)be << 52) | (mt & 0xfffffffffffffULL)));
+}
+
 #define SIC_CUDA_TRY(expr)                        \
     do {                                          \
         cudaError_t _e = (expr);                  \
@@ -284,6 +359,22 @@ sic_status launch_agg_reg(sic_handle* h, const double* pts, long long n, const s
                           const int64_t* grp_ptr, int64_t n_grp, const int64_t* cand_ptr, const int32_t* cand_idx,
                           int max_cand, int max_m, int k, int32_t* sel_idx, int32_t* sel_count, double* gain,
                           void* ws, size_t ws_bytes, cudaStream_t s);
+
+// double-precision selections with fixed-point factor rows (select_fx.cu).  A launch plan: threads per
+// CTA, grid, columns of the state kept in shared memory and the workspace for the others (nt 0:
+// the default thread count).
+struct FxPlan {
+    int nt, grid, nc;
+    size_t smem, ws_bytes;
+};
+FxPlan fx_plan_groups(sic_handle* h, long long n_grp, int max_cand, int max_m, int k, int nt);
+sic_status launch_fx_groups(sic_handle* h, const FxPlan& P, const double* pts, long long n, const sic_kernel* kp,
+                            const int64_t* grp_ptr, int64_t n_grp, const int64_t* cand_ptr, const int32_t* cand_idx,
+                            int max_cand, int max_m, int k, int32_t* sel_idx, int32_t* sel_count, double* gain,
+                            void* ws, cudaStream_t s);
+sic_status launch_fx_columns(sic_handle* h, const double* pts, long long n, const sic_kernel* kp,
+                             const int32_t* targets, int64_t n_cols, const int64_t* cand_ptr, const int32_t* cand_idx,
+                             int max_cand, int k, int32_t* sel_idx, int32_t* sel_count, double* gain, cudaStream_t s);
 
 // fixed-order sum of log v (fill.cu); ws holds sic_build_factor_workspace(n) bytes
 sic_status launch_sum_logv(const double* logv, long long n, double* sum_logv, void* ws, cudaStream_t s);
