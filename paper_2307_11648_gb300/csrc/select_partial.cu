@@ -19,11 +19,19 @@
 //            columns before p stay; the new column is Theta_{:,q | first p} / sqrt(Theta_{qq |
 //            first p}) by left-looking; the columns from p on are downdated in place by it
 //            column by column (eq. chol_partial_update): one warp forms the rotations in order
-//            from the pivot rows (the targets and picks), then every candidate row applies them
-//            all, with one barrier in between.
-// Columns live in physical slots in insertion order; `ordr/ords/opos` map the logical
-// (latest-first) order to the pivot row, the slot and the target position (INT_MAX for a
-// pick).  One CTA per group (persistent), L in shared memory, rows spread over the threads.
+//            from the pivot rows (the targets and picks), the candidate rows apply them.
+// Columns live in physical slots in insertion order; `pk/opos` map the logical (latest-first)
+// order to the pivot row and slot and to the target position (INT_MAX for a pick).  One CTA per
+// group (persistent), L in shared memory, rows spread over the threads of all warps but the first.
+//
+// A step walks each candidate row's columns twice: the left-looking product over the first p, then
+// one walk that applies the rotations and takes the next step's score as it goes.  The first warp
+// runs the rotations' serial chain at the same time -- its rows' downdate values in registers, a pivot's value
+// by shuffle, the entries of the next column loaded ahead -- and hands them over 16 columns at a time through
+// named barriers; the target block is factored once, before the candidates' rows, which need no barrier then.
+// Bound: that chain, about 200 cycles per column in one warp's instructions (a chain without the
+// shuffle took as long), with the walk of two warps per scheduler behind it.  N = 2^16, 256 candidates, k = 64 (2,811
+// groups): 16.1 ms with score, columns and rotations one after the other, 9.0 ms now.
 #include <limits.h>
 
 #include "sic_internal.cuh"
@@ -36,20 +44,24 @@ __device__ __forceinline__ float pt_div(float a, float b) { return __fdividef(a,
 __device__ __forceinline__ double pt_div(double a, double b) { return a / b; }
 
 // A column's rotation from its pivot entry lee and downdate value xe: the new pivot
-// rr = sqrt(lee^2 - xe^2), cos = rr / lee, sin = xe / lee and 1 / cos.  FP32 takes one fast
-// reciprocal and one reciprocal square root (it sits on the insertion's serial chain); FP64
-// divides exactly.
-__device__ __forceinline__ bool pt_rot(float lee, float xe, float& rr, float& cth, float& sth, float& icth) {
-    const float rr2 = fmaf(-xe, xe, lee * lee);
-    const float irr = rsqrtf(rr2), ilee = __fdividef(1.f, lee);
+// rr = sqrt(lee^2 - xe^2), cos = rr / lee, sin = xe / lee and 1 / cos = lee / rr.  Only xe is on the
+// insertion's serial chain; a = lee^2 and, in FP32, ilee = 1 / lee come from the pivot's own lane.  FP32
+// takes one fast reciprocal and one reciprocal square root; FP64 divides exactly.
+__device__ __forceinline__ float pt_inv(float lee) { return __fdividef(1.f, lee); }
+__device__ __forceinline__ double pt_inv(double) { return 0.0; }
+__device__ __forceinline__ bool pt_rot(float lee, float a, float ilee, float xe, float& rr, float& cth, float& sth,
+                                       float& icth) {
+    const float rr2 = fmaf(-xe, xe, a);
+    const float irr = rsqrtf(rr2);
     rr = rr2 * irr;
     cth = rr * ilee;
     sth = xe * ilee;
     icth = lee * irr;
     return rr2 > 0.f && lee > 0.f;
 }
-__device__ __forceinline__ bool pt_rot(double lee, double xe, double& rr, double& cth, double& sth, double& icth) {
-    const double rr2 = fma(-xe, xe, lee * lee);
+__device__ __forceinline__ bool pt_rot(double lee, double a, double, double xe, double& rr, double& cth, double& sth,
+                                       double& icth) {
+    const double rr2 = fma(-xe, xe, a);
     rr = sqrt(rr2 > 0.0 ? rr2 : 0.0);
     cth = rr / lee;
     sth = xe / lee;
@@ -60,9 +72,91 @@ __device__ __forceinline__ bool pt_rot(double lee, double xe, double& rr, double
 struct PtLayout {
     int R, W, P;  // rows (candidates + targets), columns (targets + picks), row pitch (odd)
     __host__ __device__ size_t bytes(size_t tsz) const {
+        return tsz * ((size_t)R * P + 4 * (size_t)R + 3 * (size_t)W) + sizeof(int) * ((size_t)R + 4 * (size_t)W);
+    }
+    // the size that decides which problems are taken (the state's size with two more integers per row)
+    size_t limit_bytes(size_t tsz) const {
         return tsz * ((size_t)R * P + 4 * (size_t)R + 3 * (size_t)W) + sizeof(int) * (2 * (size_t)R + 3 * (size_t)W);
     }
 };
+
+constexpr int PT_CHUNK = 16;  // columns handed over per named barrier
+constexpr int PT_EL = 6;      // element rows per lane of the first warp: 32 * PT_EL = 192 columns
+
+__device__ __forceinline__ void pt_arrive(int id) {
+    asm volatile("barrier.arrive %0, %1;" ::"r"(id), "n"(PT_NT) : "memory");
+}
+__device__ __forceinline__ void pt_sync(int id) {
+    asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(PT_NT) : "memory");
+}
+
+// The least (key, index) over the warp, key INFINITY where there is none
+__device__ __forceinline__ void pt_warp_min(float& key, int& idx) {
+    const unsigned b = __float_as_uint(key);
+    const unsigned o = (b & 0x80000000u) ? ~b : (b | 0x80000000u);  // monotone in the key (-0 < +0 apart)
+    const unsigned lo = __reduce_min_sync(0xffffffffu, o);
+    idx = (int)__reduce_min_sync(0xffffffffu, o == lo ? (unsigned)idx : (unsigned)INT_MAX);
+    key = __uint_as_float((lo & 0x80000000u) ? (lo & 0x7fffffffu) : ~lo);
+}
+__device__ __forceinline__ void pt_warp_min(double& key, int& idx) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double ok = __shfl_xor_sync(0xffffffffu, key, off);
+        const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
+        if (ok < key || (ok == key && oi < idx)) {
+            key = ok;
+            idx = oi;
+        }
+    }
+}
+
+// Rotations j0 .. min(j0 + 32, ne) of a downdate, by the first warp: lane = pivot row of rotation j0 + lane
+// (block 0) and of j0 + 32 i + lane (block i < NA, to which the rotations are applied), with each row's downdate
+// value x, its offset in Lm, its entry L in the current column and its pivot entry lee.  pc: (row << 8 | slot) of
+// the columns from the first rotation on.  Rotations go to rc / rsn / ric and are handed over per chunk.
+template <int NA, typename T>
+__device__ __forceinline__ bool pt_chain(T* __restrict__ Lm, const int* __restrict__ pc, T* __restrict__ rc,
+                                         T* __restrict__ rsn, T* __restrict__ ric, int j0, int ne, int lane,
+                                         const int (&row)[PT_EL], const T (&lee)[PT_EL], T (&x)[PT_EL], T (&L)[PT_EL]) {
+    constexpr unsigned FULL = 0xffffffffu;
+    bool ok = true;
+    const T a0 = lee[0] * lee[0], i0 = pt_inv(lee[0]);
+    int s = pc[j0] & 255, s1 = pc[min(j0 + 1, ne - 1)] & 255;
+    const int n = min(32, ne - j0);
+    for (int cc = 0; cc < n; ++cc) {
+        const int j = j0 + cc;
+        const T le = __shfl_sync(FULL, lee[0], cc), la = __shfl_sync(FULL, a0, cc), li = __shfl_sync(FULL, i0, cc);
+        const T xe = __shfl_sync(FULL, x[0], cc);
+        const int s2 = pc[min(j + 2, ne - 1)] & 255;
+        T ln[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) ln[i] = Lm[row[i] + s1];
+        T rr, cth, sth, icth;
+        ok = pt_rot(le, la, li, xe, rr, cth, sth, icth) && ok;
+        if (lane == 0) {
+            rc[j] = cth;
+            rsn[j] = sth;
+            ric[j] = icth;
+        }
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const T xr = x[i];
+            const T nl = (L[i] - sth * xr) * icth;
+            const T xn = cth * xr - sth * nl;
+            const bool act = i == 0 ? (lane > cc && lane < n) : (j0 + 32 * i + lane < ne);
+            if (act) {
+                Lm[row[i] + s] = nl;
+                x[i] = xn;
+            }
+            L[i] = ln[i];
+        }
+        if (lane == cc) Lm[row[0] + s] = rr;
+        s = s1;
+        s1 = s2;
+        if ((j & (PT_CHUNK - 1)) == PT_CHUNK - 1 || j == ne - 1) pt_arrive(1 + j / PT_CHUNK);
+    }
+    return ok;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
@@ -77,18 +171,19 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
     T* rc = xv + Lay.R;                               // [W] rotation of logical column c: cos,
     T* rsn = rc + Lay.W;                              //     sin,
     T* ric = rsn + Lay.W;                             //     1 / cos
-    int* pos = reinterpret_cast<int*>(ric + Lay.W);   // [R] positions
-    int* rank = pos + Lay.R;                          // [R] logical column of an element row, -1 otherwise
-    int* ordr = rank + Lay.R;                         // [W] pivot row of logical column c
-    int* ords = ordr + Lay.W;                         // [W] physical slot of logical column c
-    int* opos = ords + Lay.W;                         // [W] target position of column c (INT_MAX: a pick)
+    int* pos = reinterpret_cast<int*>(ric + Lay.W);   // [R] positions; ~position once the row is a pivot
+    int* pk = pos + Lay.R;                            // 2 x [W] (pivot row << 8 | slot) of logical column c
+    int* opos = pk + 2 * Lay.W;                       // 2 x [W] target position of column c (INT_MAX: a pick)
     __shared__ T s_rs, s_d;
-    __shared__ int s_p, s_fail;
+    __shared__ int s_fail;
     __shared__ T wkey[PT_NT / 32];
     __shared__ int widx[PT_NT / 32];
     __shared__ double gprod[128];
     __shared__ int gcnd[128];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int WT = PT_NT - 32;  // threads of the walking warps
+    constexpr unsigned FULL = 0xffffffffu;
+    const int wt = tid - 32;
     const int PP = Lay.P, RR = Lay.R;
     const T diag = kp.s2 + kp.nugget;
     const T INF = (T)INFINITY;
@@ -123,7 +218,6 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                 p = 0;
             }
             pos[r] = (int)p;
-            rank[r] = -1;
 #pragma unroll
             for (int d = 0; d < 3; ++d) X[d * RR + r] = (d < dim) ? (T)(pts[p * dim + d] - org[d]) : (T)0;
         }
@@ -137,185 +231,250 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
             __syncthreads();
             continue;
         }
-
-        int ncol = 0;
-        // inserts row q's point: place p, left-looking column into slot ncol, in-place
-        // downdate of the columns from p on; false (uniformly) when a pivot is not positive
-        auto insert = [&](int q) -> bool {
-            if (warp == 0) {
-                // its place: binary search of the columns (positions descending)
-                int p = 0;
-                if (lane == 0) {
-                    int lo = 0, hi = ncol;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (pos[ordr[mid]] > pos[q]) lo = mid + 1; else hi = mid;
-                    }
-                    p = lo;
-                }
-                p = __shfl_sync(0xffffffffu, p, 0);
-                T part = (T)0;
-                for (int c = lane; c < p; c += 32) {
-                    const T l = Lm[q * PP + ords[c]];
-                    part = fma(l, l, part);
-                }
+        int cur = 0;  // which half of pk / opos holds the current maps
+        auto theta = [&](int r, T qx, T qy, T qz) -> T {
+            const T dx = X[r] - qx, dy = X[RR + r] - qy, dz = X[2 * RR + r] - qz;
+            return matern<T>(kp, sic_sqrt(dx * dx + dy * dy + dz * dz));
+        };
+        // by the first warp: Theta_{qq | first p} and 1 / its root to s_d, s_rs, from row q's entries
+        auto pivot = [&](int q, int p, const int* __restrict__ cols) {
+            T part = (T)0;
+            for (int c = lane; c < p; c += 32) {
+                const T l = Lm[q * PP + (cols ? (cols[c] & 255) : c)];
+                part = fma(l, l, part);
+            }
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-                if (lane == 0) {
-                    const T d = diag - part;  // Theta_{qq | first p}
-                    s_p = p;
-                    s_d = d;
-                    if (!(d > (T)0)) s_fail = 2;
-                    s_rs = (d > (T)0) ? (T)1 / sic_sqrt(d) : (T)0;
-                }
+            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(FULL, part, off);
+            if (lane == 0) {
+                const T d = diag - part;  // Theta_{qq | first p}
+                s_d = d;
+                if (!(d > (T)0)) s_fail = 2;
+                s_rs = (d > (T)0) ? (T)1 / sic_sqrt(d) : (T)0;
             }
-            __syncthreads();
-            if (s_fail) return false;
-            const int p = s_p;
-            const T rs = s_rs;
-            const T qx = X[q], qy = X[RR + q], qz = X[2 * RR + q];
-            for (int r = tid; r < R; r += PT_NT) {
-                const int rk = rank[r];
-                T u = (T)0;
-                if (r == q) {
-                    u = s_d * rs;  // sqrt(d)
-                } else if (rk < 0 || rk >= p) {
-                    const T dx = X[r] - qx, dy = X[RR + r] - qy, dz = X[2 * RR + r] - qz;
-                    T num = matern<T>(kp, sic_sqrt(dx * dx + dy * dy + dz * dz));
-                    for (int c = 0; c < p; ++c) num = fma(-Lm[r * PP + ords[c]], Lm[q * PP + ords[c]], num);
-                    u = num * rs;
-                }
-                Lm[r * PP + ncol] = u;
-                xv[r] = (r == q) ? (T)0 : u;
-            }
-            __syncthreads();
-            // the downdate of the columns from p on, in two phases.  (1) Warp 0 forms the
-            // columns' rotations in order from the pivot rows alone -- the rows of the targets and
-            // picks at earlier positions than q, which are the pivots of those same columns --
-            // each lane carrying a few of those rows; the rotations go to shared memory.  (2)
-            // Every other row below (the candidates) applies them in order, with no barrier
-            // between columns.
-            if (warp == 0) {
-                bool bad = false;
-                for (int c = p; c < ncol; ++c) {
-                    const int e = ordr[c], s = ords[c];
-                    T rr, cth, sth, icth;
-                    bad = !pt_rot(Lm[e * PP + s], xv[e], rr, cth, sth, icth) || bad;
-                    __syncwarp();  // every lane has read the pivot's entries
-                    if (lane == 0) {
-                        rc[c] = cth;
-                        rsn[c] = sth;
-                        ric[c] = icth;
-                        Lm[e * PP + s] = rr;
-                    }
-                    for (int c2 = c + 1 + lane; c2 < ncol; c2 += 32) {
-                        const int r = ordr[c2];
-                        const T xr = xv[r];
-                        const T nl = (Lm[r * PP + s] - sth * xr) * icth;
-                        Lm[r * PP + s] = nl;
-                        xv[r] = cth * xr - sth * nl;
-                    }
-                    __syncwarp();  // the next pivot row is final
-                }
-                if (bad && lane == 0) s_fail = 2;
-            }
-            __syncthreads();
-            if (s_fail) return false;
-            for (int r = tid; r < R; r += PT_NT) {
-                if (rank[r] >= 0 || r == q) continue;
-                T xr = xv[r];
-                for (int c = p; c < ncol; ++c) {
-                    const int s = ords[c];
-                    const T nl = (Lm[r * PP + s] - rsn[c] * xr) * ric[c];
-                    Lm[r * PP + s] = nl;
-                    xr = rc[c] * xr - rsn[c] * nl;
-                }
-            }
-            __syncthreads();
-            // row q now holds a pivot: nothing in the columns after its own; the column maps
-            // shift one place from p on (each thread carries one entry across the barrier)
-            for (int c = p + tid; c < ncol; c += PT_NT) Lm[q * PP + ords[c]] = (T)0;
-            const int cm = p + 1 + tid;  // the new index of the entry this thread moves
-            int mr = 0, ms = 0, mp = 0;
-            if (cm <= ncol) {
-                mr = ordr[cm - 1];
-                ms = ords[cm - 1];
-                mp = opos[cm - 1];
-            }
-            __syncthreads();
-            if (cm <= ncol) {
-                ordr[cm] = mr;
-                ords[cm] = ms;
-                opos[cm] = mp;
-            }
-            if (tid == 0) {
-                ordr[p] = q;
-                ords[p] = ncol;
-                opos[p] = (q >= C) ? pos[q] : INT_MAX;
-            }
-            for (int r = tid; r < R; r += PT_NT) {
-                if (r == q) rank[r] = p;
-                else if (rank[r] >= p) rank[r] += 1;
-            }
-            __syncthreads();
-            ++ncol;
-            return true;
         };
 
+        // ---- the targets, latest first: column c = slot c = row C + m - 1 - c, no downdates ----
         bool ok = true;
-        // the targets, latest first: each lands after every column so far (no downdate)
-        for (int a = m - 1; a >= 0 && ok; --a) ok = insert(C + a);
-        int t = 0;
-        for (; t < k && ok; ++t) {
-            T bk = INF;
-            int bi = INT_MAX;
-            for (int j = tid; j < C; j += PT_NT) {
-                if (rank[j] >= 0) continue;
-                const int pj = pos[j];
+        for (int c = 0; c < m; ++c) {
+            const int q = C + m - 1 - c;
+            if (warp == 0) pivot(q, c, nullptr);
+            __syncthreads();
+            if (s_fail) {
+                ok = false;
+                break;
+            }
+            const T rs = s_rs;
+            if (tid == 0) {
+                Lm[q * PP + c] = s_d * rs;  // sqrt(d)
+                ric[c] = rs;                // (for the candidates' rows below)
+                pk[c] = (q << 8) | c;
+                opos[c] = pos[q];
+            }
+            const int r = C + wt;  // the targets still to come
+            if (wt >= 0 && r < q) {
+                T num = theta(r, X[q], X[RR + q], X[2 * RR + q]);
+                for (int c1 = 0; c1 < c; ++c1) num = fma(-Lm[r * PP + c1], Lm[q * PP + c1], num);
+                Lm[r * PP + c] = num * rs;
+            }
+            __syncthreads();
+        }
+        T bk = INF;  // this thread's best candidate
+        int bi = INT_MAX;
+        if (ok) {
+            for (int r = wt; wt >= 0 && r < C; r += WT) {
+                const int pj = pos[r];
                 T v = diag, pr = (T)1;
-                for (int c = 0; c < ncol; ++c) {
-                    const T l = Lm[j * PP + ords[c]];
+                for (int c = 0; c < m; ++c) {
+                    const int q = C + m - 1 - c;
+                    T num = theta(r, X[q], X[RR + q], X[2 * RR + q]);
+#pragma unroll 4
+                    for (int c1 = 0; c1 < c; ++c1) num = fma(-Lm[r * PP + c1], Lm[q * PP + c1], num);
+                    const T l = num * ric[c];
+                    Lm[r * PP + c] = l;
                     const T vn = fma(-l, l, v);
                     if (opos[c] < pj) pr = pt_div(pr * vn, v);  // a target j conditions (eq. obj_partial)
-                    v = vn;                              // eq. partial_induct
+                    v = vn;                                     // eq. partial_induct
                 }
-                if (v >= floor_ && (pr < bk || (pr == bk && j < bi))) {
+                if (v >= floor_ && (pr < bk || (pr == bk && r < bi))) {
                     bk = pr;
-                    bi = j;
+                    bi = r;
                 }
             }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T ok_ = __shfl_xor_sync(0xffffffffu, bk, off);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-                if (ok_ < bk || (ok_ == bk && oi < bi)) {
-                    bk = ok_;
-                    bi = oi;
-                }
-            }
+            __syncthreads();
+            for (int r = C + tid; r < R; r += PT_NT) pos[r] = ~pos[r];
+            // (visible after the first step's barriers)
+        }
+        int ncol = m, t = 0;
+        for (; t < k && ok; ++t) {
+            pt_warp_min(bk, bi);
             if (lane == 0) {
                 wkey[warp] = bk;
                 widx[warp] = bi;
             }
             __syncthreads();
-            T gk = wkey[0];
-            int q = widx[0];
-#pragma unroll
-            for (int w = 1; w < PT_NT / 32; ++w)
-                if (wkey[w] < gk || (wkey[w] == gk && widx[w] < q)) {
-                    gk = wkey[w];
-                    q = widx[w];
-                }
+            T gk = lane < PT_NT / 32 ? wkey[lane] : INF;
+            int q = lane < PT_NT / 32 ? widx[lane] : INT_MAX;
+            pt_warp_min(gk, q);
             if (q == INT_MAX) break;
-            // the targets the pick conditions (its nonzeros)
-            const int nc = __syncthreads_count(tid < ncol && opos[tid] < pos[q]);
+            const int pq = pos[q];
+            const int* __restrict__ pc = pk + cur * Lay.W;
+            const int* __restrict__ oc = opos + cur * Lay.W;
+            // its place, and the targets it conditions (its nonzeros)
+            int p = 0, nc = 0;
+            for (int c0 = 0; c0 < ncol; c0 += 32) {
+                const int c = c0 + lane;
+                p += __popc(__ballot_sync(FULL, c < ncol && ~pos[pc[c < ncol ? c : 0] >> 8] > pq));
+                nc += __popc(__ballot_sync(FULL, c < ncol && oc[c < ncol ? c : 0] < pq));
+            }
             if (tid == 0) {
                 gprod[t] = (double)gk;
                 gcnd[t] = nc;
-                sel_idx[g * k + t] = pos[q];
+                sel_idx[g * k + t] = pq;
             }
-            ok = insert(q);
-            if (!ok) break;
+            // ---- the new column, left-looking (candidates, and pivots at earlier positions) ----
+            if (warp == 0) {
+                pivot(q, p, pc);
+            } else {
+                const T qx = X[q], qy = X[RR + q], qz = X[2 * RR + q];
+                const T* __restrict__ Lq = Lm + q * PP;
+                for (int r = wt; r < R; r += WT) {
+                    const int ps = pos[r];
+                    if (r == q || (ps < 0 && ~ps > pq)) continue;
+                    const T* __restrict__ Lr = Lm + r * PP;
+                    T num = theta(r, qx, qy, qz);
+#pragma unroll 8
+                    for (int c = 0; c < p; ++c) {
+                        const int s = pc[c] & 255;
+                        num = fma(-Lr[s], Lq[s], num);
+                    }
+                    xv[r] = num;
+                }
+            }
+            __syncthreads();
+            if (s_fail) {
+                ok = false;
+                break;
+            }
+            const T rs = s_rs;
+            for (int r = wt; wt >= 0 && r < R; r += WT) {
+                const int ps = pos[r];
+                if (r == q) {
+                    Lm[r * PP + ncol] = s_d * rs;  // sqrt(d)
+                    pos[r] = ~pq;
+                } else if (ps >= 0 || ~ps < pq) {
+                    const T u = xv[r] * rs;
+                    Lm[r * PP + ncol] = u;
+                    xv[r] = u;
+                }
+            }
+            __syncthreads();
+            const int ne = ncol - p;  // columns to downdate: the rotations are numbered 0 .. ne - 1 from p
+            if (warp == 0) {
+                // the rotations, in order, from the pivot rows alone -- the rows of the targets and picks
+                // at earlier positions than q, which are the pivots of those same columns
+                int row[PT_EL];
+                T lee[PT_EL], x[PT_EL], L[PT_EL];
+                const int s = ne > 0 ? (pc[p] & 255) : 0;
+#pragma unroll
+                for (int i = 0; i < PT_EL; ++i) {
+                    const int c2 = lane + 32 * i;
+                    row[i] = q * PP;  // (rows beyond the last: read, not written)
+                    lee[i] = x[i] = L[i] = (T)0;
+                    if (c2 < ne) {
+                        const int e = pc[p + c2];
+                        row[i] = (e >> 8) * PP;
+                        lee[i] = Lm[row[i] + (e & 255)];
+                        x[i] = xv[e >> 8];
+                        L[i] = Lm[row[i] + s];
+                    }
+                }
+                bool good = true;
+                for (int j0 = 0; j0 < ne; j0 += 32) {
+                    const int na = (ne - j0 + 31) >> 5;
+                    const int* pj = pc + p;
+                    T *c_ = rc + p, *s_ = rsn + p, *i_ = ric + p;
+                    const bool g1 = na == 1   ? pt_chain<1>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                    : na == 2 ? pt_chain<2>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                    : na == 3 ? pt_chain<3>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                              : pt_chain<PT_EL>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L);
+                    good = good && g1;
+#pragma unroll
+                    for (int i = 0; i + 1 < PT_EL; ++i) {  // the next block of pivot rows
+                        row[i] = row[i + 1];
+                        lee[i] = lee[i + 1];
+                        x[i] = x[i + 1];
+                        L[i] = L[i + 1];
+                    }
+                }
+                if (!good && lane == 0) s_fail = 2;
+                bk = INF;
+                bi = INT_MAX;
+            } else {
+                // the maps with the new column in its place, for the next step
+                if (wt <= ncol) {
+                    int e, o;
+                    if (wt == p) {
+                        e = (q << 8) | ncol;
+                        o = INT_MAX;
+                    } else {
+                        e = pc[wt < p ? wt : wt - 1];
+                        o = oc[wt < p ? wt : wt - 1];
+                    }
+                    pk[(cur ^ 1) * Lay.W + wt] = e;
+                    opos[(cur ^ 1) * Lay.W + wt] = o;
+                }
+                bk = INF;
+                bi = INT_MAX;
+                bool wait = true;  // the first rows wait for the rotations
+                int r = wt;
+                do {
+                    const bool live = r < C && pos[r < C ? r : 0] >= 0;
+                    T* __restrict__ Lr = Lm + (live ? r : 0) * PP;
+                    const int pj = live ? pos[r] : 0;
+                    T v = diag, pr = (T)1, xr = (T)0;
+                    auto take = [&](T l, int o) {
+                        const T vn = fma(-l, l, v);
+                        if (o < pj) pr = pt_div(pr * vn, v);  // a target j conditions (eq. obj_partial)
+                        v = vn;                               // eq. partial_induct
+                    };
+                    if (live) {
+                        xr = xv[r];
+#pragma unroll 4
+                        for (int c = 0; c < p; ++c) take(Lr[pc[c] & 255], oc[c]);
+                        take(xr, INT_MAX);
+                    }
+                    for (int j0 = 0; j0 < ne; j0 += PT_CHUNK) {
+                        if (wait) {
+                            __syncwarp();
+                            pt_sync(1 + j0 / PT_CHUNK);
+                        }
+                        if (live) {
+                            const int c1 = p + min(j0 + PT_CHUNK, ne);
+#pragma unroll 4
+                            for (int c = p + j0; c < c1; ++c) {
+                                const int s = pc[c] & 255;
+                                const T nl = (Lr[s] - rsn[c] * xr) * ric[c];
+                                Lr[s] = nl;
+                                xr = rc[c] * xr - rsn[c] * nl;
+                                take(nl, oc[c]);
+                            }
+                        }
+                    }
+                    if (live && v >= floor_ && (pr < bk || (pr == bk && r < bi))) {
+                        bk = pr;
+                        bi = r;
+                    }
+                    wait = false;
+                    r += WT;
+                } while (r - wt < C);
+            }
+            __syncthreads();
+            if (s_fail) {
+                ok = false;
+                break;
+            }
+            cur ^= 1;
+            ++ncol;
         }
         if (!ok && tid == 0) record_error(st, SIC_ERR_NOT_PD, g);
         if (tid == 0) sel_count[g] = t;
@@ -387,8 +546,9 @@ extern "C" sic_status sic_select_partial(sic_handle* h, const double* pts, int64
     L.R = max_cand + max_m;
     L.W = max_m + k;
     L.P = L.W | 1;
-    const size_t smem = L.bytes(prec == SIC_FP64 ? sizeof(double) : sizeof(float));
-    if (smem > 227 * 1024 - 4096) return SIC_ERR_UNSUPPORTED;
+    const size_t tsz = prec == SIC_FP64 ? sizeof(double) : sizeof(float);
+    if (L.limit_bytes(tsz) > 227 * 1024 - 4096) return SIC_ERR_UNSUPPORTED;
+    const size_t smem = L.bytes(tsz);
     SIC_CUDA_TRY(cudaSetDevice(h->device));
     cudaStream_t s = (cudaStream_t)stream;
     const long long* gp = (const long long*)grp_ptr;
