@@ -1,0 +1,393 @@
+// y = (Theta + shift I) x for several right-hand sides, the sums on the 5th-generation tensor cores.
+//
+// The kernel entries are evaluated in FP32 (the same fixed, symmetric rounding of Theta as in pcg.cu's
+// kernel for few right-hand sides); what cost most was summing their products to far below FP32, 11
+// operations per entry and right-hand side.  Here both factors are cut into 8-bit digits, which BF16
+// holds exactly, and the digits' products are summed exactly (after Ozaki et al., Numer. Algorithms 59 (2012)):
+//   Theta_ij / 2^E = sum_a A_a 2^-(7 + 8a), a = 0..5 (2^E >= variance),
+//   x_jr / 2^X_r   = sum_b B_b 2^-(7 + 8b), b = 0..5 (2^X_r > max_j |x_jr|), |A_a|, |B_b| <= 128,
+// with A_0 = round(128 Theta / 2^E), the remainder times 256, and so on (exact FP32 operations).  Products of
+// level a + b = l <= 5 go to one accumulator: 128 sources x 6 pairs x 2^14 < 2^24, so FP32 holds every partial
+// sum exactly; after 128 sources the levels are added to two 64-bit integers per row and right-hand
+// side.  What is left out (digits below 2^-47 of the variance and of max|x|, levels from 6 on) is below 2^-46 max|x|
+// per term, of random sign: about 2^-38 max|x| over 50,000 sources, 1e-12 of a typical result.  The integers do
+// not depend on the order of the sum.
+//
+// A CTA takes 128 rows (TMEM lanes) and, in a cluster, a share of the sources; 256 threads = row and half of a step's
+// 16 sources.  Per step the threads write the six digit tiles of Theta (128 x 16 BF16, K-major core matrices) into
+// one of two buffers and one thread issues six MMAs (digit a against B_0 .. B_(5-a), N = 48, 48, 32, 32, 16, 16 into
+// the columns from level a on; where that is one digit more than needed it lands in level 6, which is not
+// read).  The MMAs run under the next step's evaluation; the accumulators (two sets) are read one chunk late.
+//
+// Bound: FP32 issue of the kernel evaluation and the digits, about 45 operations per entry whatever the
+// number of right-hand sides.  N = 50,001 with 8 of them: 16.6 ms with double-FP32 sums on the CUDA cores, 6.8 ms
+// now (N = 4096: 1.04 -> 0.086 ms); with sqrtf and a run-time smoothness, whose branches keep the evaluations from
+// overlapping, 11.2 ms.
+#include "tc_common.cuh"
+
+namespace {
+
+constexpr int ROWS = 128, CH = 128, SUB = 16, NT = 256;
+constexpr int KD = 6, XD = 6;  // digits of Theta and of x
+constexpr int A_TILE = ROWS * SUB * 2;       // one digit tile
+constexpr int SA = 0;                        // [2 buffers][KD] tiles
+constexpr int SB = SA + 2 * KD * A_TILE;     // [2 chunks] digits of x: XD * 8 rows x CH, K-major
+constexpr int B_TILE = XD * 8 * CH * 2;
+constexpr int SC = SB + 2 * B_TILE;          // [2 chunks][3][CH] negated coordinates
+constexpr int SX = SC + 2 * 3 * CH * 4;      // largest biased exponent per right-hand side, a flag
+constexpr int SBAR = SX + 16 * 4;            // two mbarriers, TMEM address
+constexpr int SMEM_MV = SBAR + 32;
+constexpr int SACC = SA;                     // [ROWS][8][2] 64-bit sums for the cluster (after the last MMA)
+static_assert(ROWS * 8 * 2 * 8 <= SB, "the sums fit in the digit tiles");
+// two CTAs per SM: 256 of the 512 TMEM columns, none waits for them
+constexpr unsigned TMEM_COLS = 128;
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ long long ld_cluster_s64(uint32_t addr, uint32_t rank) {
+    long long v;
+    asm volatile(
+        "{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.s64 %0, [a];\n}\n"
+        : "=l"(v)
+        : "r"(addr), "r"(rank)
+        : "memory");
+    return v;
+}
+
+// The correctly rounded square roots of a pair (sqrtf without its special-case branches, so that the evaluations
+// overlap): from the hardware's reciprocal square root y, g = x y and h = y / 2 by one coupled Newton step, then the
+// residual step g + h (x - g^2) with fused operations (Markstein, IBM J. Res. Dev. 34 (1990)).  Checked over
+// every significand with y off by up to 2.5 ulp.  Below 2^-100 (distances that leave every kernel at its value at 0)
+// the last bits may differ; infinity stays infinite.
+__device__ __forceinline__ float2 sqrt_f2(float2 x) {
+    float ya, yb;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ya) : "f"(fmaxf(x.x, 1.2e-38f)));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yb) : "f"(fmaxf(x.y, 1.2e-38f)));
+    const float2 neg1 = make_float2(-1.f, -1.f), half2 = make_float2(0.5f, 0.5f);
+    const float2 y = make_float2(ya, yb);
+    const float2 g = __fmul2_rn(x, y), h = __fmul2_rn(y, half2);
+    const float2 e = __ffma2_rn(__fmul2_rn(g, neg1), h, half2);
+    const float2 g1 = __ffma2_rn(g, e, g), h1 = __ffma2_rn(h, e, h);
+    const float2 r = __ffma2_rn(__ffma2_rn(__fmul2_rn(g1, neg1), g1, x), h1, g1);
+    return make_float2(x.x < INFINITY ? r.x : x.x, x.y < INFINITY ? r.y : x.y);
+}
+
+// matern<float> (the same operations) with the smoothness a constant
+template <int NU>
+__device__ __forceinline__ float matern_nu(const KP<float>& k, float r) {
+    const float t = k.c_over_ell * r;
+    const float e = sic_exp(-t);
+    if (NU == 1) return k.s2 * e;
+    if (NU == 3) return k.s2 * (1.f + t) * e;
+    return k.s2 * (1.f + t + t * t * (float)(1.0 / 3.0)) * e;
+}
+
+__device__ __forceinline__ int ld_cluster_s32(uint32_t addr, uint32_t rank) {
+    int v;
+    asm volatile(
+        "{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.s32 %0, [a];\n}\n"
+        : "=r"(v)
+        : "r"(addr), "r"(rank)
+        : "memory");
+    return v;
+}
+
+template <int NU>
+__global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ pts, long long n, int dim, KP<float> kp,
+                                                     float to_unit, int E, double diag_extra,
+                                                     const double* __restrict__ x, double* __restrict__ y, int nrhs,
+                                                     int parts, DevStatus* st) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+    int* sx = reinterpret_cast<int*>(sm + SX);  // [0..7] exponents, [8] non-finite source coordinate
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + SBAR);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + SBAR + 16);
+    const uint32_t bar[2] = {smem_u32(bars), smem_u32(bars + 1)};
+    const uint32_t aA = smem_u32(sm + SA), aB = smem_u32(sm + SB);
+
+    if (tid == 0) {
+        for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar[b]) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (tid < 16) sx[tid] = 0;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+
+    // the largest exponent of every right-hand side (by its bits), the cluster's CTAs a share each
+    const uint32_t cluster_part = parts > 1 ? cluster_rank() : 0u;
+    {
+        int ex[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) ex[r] = 0;
+        for (long long j = (long long)cluster_part * NT + tid; j < n; j += (long long)parts * NT) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                if (r < nrhs) ex[r] = max(ex[r], (__double2hiint(x[j * nrhs + r]) >> 20) & 0x7ff);
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int m = __reduce_max_sync(0xffffffffu, ex[r]);
+            if (lane == 0) atomicMax(&sx[r], m);
+        }
+    }
+    // rows, and this CTA's chunks of sources
+    const long long tile = blockIdx.x / parts;
+    const uint32_t rank = cluster_part;
+    const long long i = tile * ROWS + row;
+    float rc[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) rc[d] = (i < n && d < dim) ? (float)pts[i * dim + d] : 0.f;
+    const long long chunks = (n + CH - 1) / CH;
+    const long long c_lo = chunks * rank / parts, c_hi = chunks * (rank + 1) / parts;
+
+    long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+    float chk = 0.f;  // NaN once a kernel entry is
+    bool failed = false;
+    uint32_t par[2] = {0u, 0u};
+    bool used[2] = {false, false};
+    // adds the levels of accumulator set `set` to the sums
+    auto take = [&](int set) {
+        float v[6][4];
+#pragma unroll
+        for (int l = 0; l < 6; ++l) tmem_ld4(lane_addr + set * 64 + 8 * l + 4 * half, v[l]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            hi[r] += ((long long)__float2int_rn(v[0][r]) << 16) + (__float2int_rn(v[1][r]) * 256LL) + __float2int_rn(v[2][r]);
+            lo[r] += ((long long)__float2int_rn(v[3][r]) << 16) + (__float2int_rn(v[4][r]) * 256LL) + __float2int_rn(v[5][r]);
+        }
+    };
+    __syncthreads();
+    if (parts > 1) {
+        cluster_sync_all();
+        int m = 0;
+        if (tid < 8)
+            for (int q = 0; q < parts; ++q) m = max(m, ld_cluster_s32(smem_u32(sx + tid), q));
+        cluster_sync_all();
+        if (tid < 8) sx[tid] = m;
+        __syncthreads();
+    }
+    for (long long c = c_lo; c < c_hi && !failed; ++c) {
+        const int set = (int)((c - c_lo) & 1);
+        // ---- the chunk's coordinates and the digits of its x ----
+        float* nc = reinterpret_cast<float*>(sm + SC) + set * 3 * CH;
+        for (int e = tid; e < 3 * CH; e += NT) {
+            const int d = e / CH, t = e % CH;
+            const long long j = c * CH + t;
+            const float v = (j < n && d < dim) ? (float)pts[j * dim + d] : 0.f;
+            if (!(fabsf(v) < INFINITY)) sx[8] = 1;
+            nc[d * CH + t] = -v;
+        }
+#pragma unroll
+        for (int q = 0; q < CH * 8 / NT; ++q) {
+            const int t = (tid >> 3) + q * (NT / 8), r = tid & 7;
+            const long long j = c * CH + t;
+            long long I = 0;  // round(x 2^(47 - X)), |I| <= 2^47
+            if (j < n && r < nrhs) {
+                const long long u = __double_as_longlong(x[j * nrhs + r]);
+                const int e = (int)((u >> 52) & 0x7ff);
+                const long long mant = (u & 0xfffffffffffffLL) | 0x10000000000000LL;
+                const int sh = sx[r] - e + 6;  // X = sx[r] - 1022
+                if (e > 0 && sh < 55) I = ((mant >> (sh - 1)) + 1) >> 1;
+                if (u < 0) I = -I;
+            }
+            unsigned char* Bt = sm + SB + set * B_TILE;
+#pragma unroll
+            for (int b = XD - 1; b >= 0; --b) {
+                const int dgt = b > 0 ? (int)(signed char)(I & 255) : (int)I;
+                I = (I - dgt) >> 8;
+                *reinterpret_cast<__nv_bfloat16*>(Bt + core_off(b * 8 + r, t, CH)) = __float2bfloat16_rn((float)dgt);
+            }
+        }
+        __syncthreads();
+        for (int s = 0; s < CH / SUB; ++s) {
+            const int buf = s & 1;
+            if (used[buf]) {  // the MMAs that read this buffer last
+                if (!bar_wait(bar[buf], par[buf])) failed = true;
+                par[buf] ^= 1u;
+            }
+            used[buf] = true;
+            // ---- eight kernel entries, two at a time, and their digits ----
+            uint32_t dg[KD][4];
+            const float* cx = nc + s * SUB + half * 8;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const float2 dx = __fadd2_rn(make_float2(rc[0], rc[0]), *reinterpret_cast<const float2*>(cx + 2 * p));
+                const float2 dy =
+                    __fadd2_rn(make_float2(rc[1], rc[1]), *reinterpret_cast<const float2*>(cx + CH + 2 * p));
+                float2 d2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+                if (dim > 2) {
+                    const float2 dz =
+                        __fadd2_rn(make_float2(rc[2], rc[2]), *reinterpret_cast<const float2*>(cx + 2 * CH + 2 * p));
+                    d2 = __ffma2_rn(dz, dz, d2);
+                }
+                const float2 dist = sqrt_f2(d2);
+                const float2 k = make_float2(matern_nu<NU>(kp, dist.x), matern_nu<NU>(kp, dist.y));
+                float2 r = __fmul2_rn(k, make_float2(to_unit, to_unit));
+                const float2 M = make_float2(12582912.f, 12582912.f);  // 1.5 2^23: adding it rounds to an integer
+                const float2 neg1 = make_float2(-1.f, -1.f);
+#pragma unroll
+                for (int a = 0; a < KD; ++a) {
+                    const float f = a == 0 ? 128.f : 256.f;
+                    const float2 f2 = make_float2(f, f);
+                    const float2 nd = __ffma2_rn(__ffma2_rn(r, f2, M), neg1, M);  // minus the digit
+                    if (a == 0) chk += nd.x + nd.y;
+                    if (a + 1 < KD) r = __ffma2_rn(r, f2, nd);  // exact
+                    dg[a][p] = pack2(nd.x, nd.y);
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < KD; ++a)
+                *reinterpret_cast<uint4*>(sm + SA + (buf * KD + a) * A_TILE + core_off(row, half * 8, SUB)) =
+                    make_uint4(dg[a][0], dg[a][1], dg[a][2], dg[a][3]);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            if (__syncthreads_or(failed)) {
+                failed = true;
+                break;
+            }
+            if (tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int a = 0; a < KD; ++a)
+                    mma_f16(tmem + set * 64 + 8 * a, smem_desc(aA + (buf * KD + a) * A_TILE, 128, 256),
+                            smem_desc(aB + set * B_TILE + s * (SUB / 8) * 128, 128, (CH / 8) * 128),
+                            (s > 0 || a > 0) ? 1u : 0u, idesc_bf16(48 - 16 * (a / 2), 0, 0));
+                mma_commit(bar[buf]);
+            }
+            // the previous chunk's last MMAs were waited for in this chunk's first two steps
+            if (s == 2 && c > c_lo) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                take(set ^ 1);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            }
+        }
+    }
+    for (int b = 0; b < 2; ++b)
+        if (used[b] && !failed)
+            if (!bar_wait(bar[b], par[b])) failed = true;
+    if (__syncthreads_or(failed)) failed = true;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!failed && c_hi > c_lo) take((int)((c_hi - 1 - c_lo) & 1));
+    if (failed && tid == 0) record_error(st, SIC_ERR_TIMEOUT, blockIdx.x);
+    // a non-finite kernel entry in either half of the row, or a non-finite source: the row's result is NaN
+    int* flag = reinterpret_cast<int*>(sm + SC);
+    if (half == 0) flag[row] = sx[8];
+    __syncthreads();
+    if (!(fabsf(chk) < INFINITY)) flag[row] = 1;
+    __syncthreads();
+    bool nan_row = flag[row] != 0;
+    // ---- the cluster's sums to its first CTA, the result ----
+    long long* acc = reinterpret_cast<long long*>(sm + SACC);
+    constexpr long long NOT_A_NUMBER = (long long)0x8000000000000000ULL;
+    if (parts > 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            acc[(row * 8 + 4 * half + r) * 2] = nan_row ? NOT_A_NUMBER : hi[r];
+            acc[(row * 8 + 4 * half + r) * 2 + 1] = lo[r];
+        }
+        cluster_sync_all();
+        if (rank == 0) {
+            for (int q = 1; q < parts; ++q) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t at = smem_u32(acc + (row * 8 + 4 * half + r) * 2);
+                    const long long h = ld_cluster_s64(at, q);
+                    if (h == NOT_A_NUMBER) nan_row = true;
+                    hi[r] += h;
+                    lo[r] += ld_cluster_s64(at + 8, q);
+                }
+            }
+        }
+        cluster_sync_all();
+    }
+    if (rank == 0 && i < n && !failed) {
+#pragma unroll
+        for (int r0 = 0; r0 < 4; ++r0) {
+            const int r = 4 * half + r0;
+            if (r >= nrhs) continue;
+            // (the sums have the minus sign of Theta's digits)
+            double v = -(ldexp((double)hi[r0], -30) + ldexp((double)lo[r0], -54));
+            v = ldexp(v, E + sx[r] - 1022);
+            if (nan_row || sx[r] == 0x7ff) v = NAN;
+            y[i * nrhs + r] = v + diag_extra * x[i * nrhs + r];
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+}  // namespace
+
+template <int NU>
+static sic_status launch_matvec_tc(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, double shift,
+                                   const double* x, double* y, int nrhs, cudaStream_t s) {
+    auto kern = k_matvec_tc<NU>;
+    SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MV));
+    const long long tiles = (n + ROWS - 1) / ROWS, slots = 2LL * h->num_sms;
+    // CTAs per row tile (a cluster, at least two chunks of sources each): the number that leaves the last wave of two
+    // CTAs per SM fullest -- N = 50,001: 391 tiles are 1.3 waves, eight parts 10.3
+    int parts = 1;
+    double best = 0.0;
+    for (int p = 1; p <= 8 && (p == 1 || 2 * p <= tiles); p *= 2) {
+        const long long waves = (tiles * p + slots - 1) / slots;
+        const double full = (double)(tiles * p) / (double)(waves * slots);
+        if (full > best + 0.02) {
+            best = full;
+            parts = p;
+        }
+    }
+    int E = 0;
+    const float s2 = (float)kp->variance;
+    if (frexpf(s2, &E) == 0.5f) --E;  // variance <= 2^E
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * parts));
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = SMEM_MV;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)parts;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = parts > 1 ? 1 : 0;
+    SIC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, pts, n, (int)kp->dim, make_kp<float>(*kp), ldexpf(1.f, -E), E,
+                                    kp->nugget + shift, x, y, nrhs, parts, h->d_status));
+    return SIC_OK;
+}
+
+sic_status matvec_tc(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, double shift, const double* x,
+                     double* y, int nrhs, cudaStream_t s) {
+    if (kp->nu_x2 == 1) return launch_matvec_tc<1>(h, pts, n, kp, shift, x, y, nrhs, s);
+    if (kp->nu_x2 == 3) return launch_matvec_tc<3>(h, pts, n, kp, shift, x, y, nrhs, s);
+    return launch_matvec_tc<5>(h, pts, n, kp, shift, x, y, nrhs, s);
+}

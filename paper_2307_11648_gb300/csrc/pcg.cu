@@ -1,16 +1,13 @@
 // Preconditioned conjugate gradients on (Theta + shift I) x = b with the sparse factor
 // as preconditioner M^{-1} = L L^T (the use of the factor studied in Section 6.4).
 //
-// k_matvec<T>: y = (Theta + shift I) x for up to 8 right-hand sides without forming Theta:
-// one thread per target row, source points staged in shared-memory tiles.  With T = float
-// the kernel entries are FP32 (a fixed, symmetric rounding of Theta: K(|x_i - x_j|) is
-// evaluated identically for (i, j) and (j, i)); x is carried as an unevaluated sum of two
-// FP32 numbers (hi + lo) and each tile's sum of products is accumulated as a double-FP32
-// pair with the error-free transformations TwoProduct (by fma) and TwoSum (Knuth), then
-// added to an FP64 accumulator -- so the product is accurate to ~1e-14 of sum |K x| and
-// CG can reach small residuals.  With T = double everything is FP64 (reference mode; the
-// kernel entries by the fill's table-driven exp and Newton square root, about 2 ulp).
-// The diagonal adds the nugget and the shift in FP64.
+// FP32 mode, up to two right-hand sides and many points (k_matvec_f32; else matvec_tc.cu): y = (Theta + shift I) x without
+// forming Theta.  The kernel entries are FP32 (a fixed, symmetric rounding of Theta: K(|x_i - x_j|) is evaluated
+// identically for (i, j) and (j, i)); x is carried as an unevaluated sum of two FP32 numbers (hi + lo) and the
+// products are summed as a double-FP32 pair with the error-free transformations TwoProduct (by fma) and
+// TwoSum (Knuth), 1024 terms at a time, then in FP64 -- so the product is accurate to ~1e-13 of sum |K x| and
+// CG can reach small residuals.  k_matvec_f64 is FP64 throughout (reference mode; the kernel entries by the fill's table-driven exp
+// and Newton square root, about 2 ulp).  The diagonal adds the nugget and the shift in FP64.
 // The CG vector updates and dot products are fused kernels with fixed-order reductions
 // (bit-reproducible); the scalars alpha and beta are formed on the device per RHS.
 // The iteration loop runs on the host (C++), reading back the residual norms each step.
@@ -22,27 +19,160 @@
 
 namespace {
 
-constexpr int MV_NT = 128;   // target rows per CTA
+constexpr int MV_NT = 128;   // FP64: target rows per CTA
 constexpr int MV_TILE = 256; // source points per shared-memory tile
 constexpr int RED_TILE = 4096;
 
-template <typename T, int NR>
-__global__ void __launch_bounds__(MV_NT) k_matvec(const double* __restrict__ pts, long long n, int dim, KP<T> kp,
-                                                  double diag_extra, const double* __restrict__ x,
-                                                  double* __restrict__ y, int nrhs) {
-    constexpr bool F32 = sizeof(T) == 4;
-    __shared__ T sx[MV_TILE], sy[MV_TILE], sz[MV_TILE];
-    __shared__ T sv[MV_TILE * NR];
-    __shared__ float svl[F32 ? MV_TILE * NR : 1];  // low parts of x in FP32 mode
-    __shared__ double tab[F32 ? 1 : EXP_TAB];      // FP64 mode: s2 2^(j/256) for the table-driven exp
-    if constexpr (!F32) exp_table_fill(tab, kp.s2);  // ordered before use by the tile loop's barrier
+// A CTA of 8 warps takes 64 target rows (two per lane, so that a source's values are read once for both and the
+// kernel evaluation runs in packed FP32 pairs); the warps share the staged source tile, 32 sources each, and
+// their sums are added in order at the end.  With one thread per row over all sources, N = 50,001 left an SM
+// ten warps.  Bound: FP32 lanes (11 operations per source, row and right-hand side, about 22 per entry).
+// N = 50,001, one right-hand side: 6.0 ms
+// with a thread per row, 5.2 ms now (two: 8.0 and 5.2).
+constexpr int MVF_WARPS = 8, MVF_ROWS = 64, MVF_FLUSH = 32;  // (tiles between FP64 additions)
+
+// v as hi + lo, hi = v rounded to FP32, lo = the rest rounded to FP32: by integer operations where 2^-99 <= |v| <
+// 2^115 (conversions run on the FP64 pipe), else by conversions
+__device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)((u >> 52) & 0x7ff);
+    if (e > 923 && e < 1138) {
+        const unsigned long long mant = (u & 0xfffffffffffffULL) | 0x10000000000000ULL;
+        const unsigned h = (unsigned)((mant + (1ULL << 28)) >> 29);  // 24 bits, or 2^24
+        const int l = (int)(mant - ((unsigned long long)h << 29));  // |l| <= 2^28
+        const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
+        hi = __fmul_rn(__uint2float_rn(h), __uint_as_float(sg | ((unsigned)(e - 919) << 23)));
+        lo = __fmul_rn(__fmul_rn(__int2float_rn(l), __uint_as_float(sg | ((unsigned)(e - 884) << 23))), 0x1p-64f);
+    } else {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    }
+}
+
+template <int NR>
+__global__ void __launch_bounds__(32 * MVF_WARPS, 2) k_matvec_f32(const double* __restrict__ pts, long long n, int dim,
+                                                                  KP<float> kp, double diag_extra,
+                                                                  const double* __restrict__ x, double* __restrict__ y,
+                                                                  int nrhs) {
+    constexpr int NP = (NR + 1) / 2;  // right-hand sides in pairs
+    constexpr int NT = 32 * MVF_WARPS;
+    __shared__ union Sm {
+        struct {
+            float4 c[MV_TILE];        // coordinates
+            float2 h[MV_TILE][NP];    // high parts of x
+            float2 l[MV_TILE][NP];    // low parts
+        } t;
+        double acc[MVF_WARPS][2 * NP][MVF_ROWS];
+    } sm;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long i0 = blockIdx.x * (long long)MVF_ROWS + lane, i1 = i0 + 32;
+    float2 rx = make_float2(0.f, 0.f), ry = rx, rz = rx;  // the lane's two rows
+    auto coord = [&](long long i, int d) { return i < n && d < dim ? (float)pts[i * dim + d] : 0.f; };
+    rx = make_float2(coord(i0, 0), coord(i1, 0));
+    ry = make_float2(coord(i0, 1), coord(i1, 1));
+    rz = make_float2(coord(i0, 2), coord(i1, 2));
+    const float2 neg1 = make_float2(-1.f, -1.f);
+    float2 S[2][NP], lo[2][NP];
+    double acc[2][2 * NP];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+            S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
+            acc[q][2 * r] = acc[q][2 * r + 1] = 0.0;
+        }
+    auto flush = [&]() {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int r = 0; r < NP; ++r) {
+                acc[q][2 * r] += (double)S[q][r].x + (double)lo[q][r].x;
+                acc[q][2 * r + 1] += (double)S[q][r].y + (double)lo[q][r].y;
+                S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
+            }
+    };
+    int tiles = 0;
+    for (long long j0 = 0; j0 < n; j0 += MV_TILE) {
+        __syncthreads();
+        for (int t = tid; t < MV_TILE; t += NT) {
+            const long long j = j0 + t;
+            sm.t.c[t] = make_float4(coord(j, 0), coord(j, 1), coord(j, 2), 0.f);
+#pragma unroll
+            for (int r = 0; r < NP; ++r) {
+                float2 h = make_float2(0.f, 0.f), l = h;
+                if (j < n) {
+                    if (2 * r < nrhs) split_f64(x[j * nrhs + 2 * r], h.x, l.x);
+                    if (2 * r + 1 < nrhs) split_f64(x[j * nrhs + 2 * r + 1], h.y, l.y);
+                }
+                sm.t.h[t][r] = h;
+                sm.t.l[t][r] = l;
+            }
+        }
+        __syncthreads();
+        const int t0 = warp * (MV_TILE / MVF_WARPS);
+        const int t1 = (int)min((long long)(t0 + MV_TILE / MVF_WARPS), n - j0);
+        for (int t = t0; t < t1; ++t) {
+            const float4 c = sm.t.c[t];
+            const float2 dx = __fadd2_rn(rx, make_float2(-c.x, -c.x)), dy = __fadd2_rn(ry, make_float2(-c.y, -c.y)),
+                         dz = __fadd2_rn(rz, make_float2(-c.z, -c.z));
+            const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+            const float k0 = matern<float>(kp, sqrtf(d2.x)), k1 = matern<float>(kp, sqrtf(d2.y));
+#pragma unroll
+            for (int r = 0; r < NP; ++r) {
+                const float2 xh = sm.t.h[t][r], xl = sm.t.l[t][r];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float2 k = q == 0 ? make_float2(k0, k0) : make_float2(k1, k1);
+                    // TwoProduct, TwoSum (packed operations: lane-wise the scalar roundings)
+                    const float2 p = __fmul2_rn(k, xh);
+                    const float2 pe = __ffma2_rn(k, xl, __ffma2_rn(k, xh, __fmul2_rn(p, neg1)));
+                    const float2 s = __fadd2_rn(S[q][r], p);
+                    const float2 nb = __ffma2_rn(s, neg1, S[q][r]);                       // -(s - S)
+                    const float2 ea = __ffma2_rn(__fadd2_rn(s, nb), neg1, S[q][r]);       // S - (s - (s - S))
+                    lo[q][r] = __fadd2_rn(lo[q][r], __fadd2_rn(__fadd2_rn(ea, __fadd2_rn(p, nb)), pe));
+                    S[q][r] = s;
+                }
+            }
+        }
+        if (++tiles == MVF_FLUSH) {
+            flush();
+            tiles = 0;
+        }
+    }
+    flush();
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 2 * NP; ++r) {
+        sm.acc[warp][r][lane] = acc[0][r];
+        sm.acc[warp][r][lane + 32] = acc[1][r];
+    }
+    __syncthreads();
+    for (int e = tid; e < MVF_ROWS * nrhs; e += NT) {
+        const int row = e / nrhs, r = e - row * nrhs;
+        const long long i = blockIdx.x * (long long)MVF_ROWS + row;
+        if (i >= n) continue;
+        double a = sm.acc[0][r][row];
+#pragma unroll
+        for (int w = 1; w < MVF_WARPS; ++w) a += sm.acc[w][r][row];
+        y[i * nrhs + r] = a + diag_extra * x[i * nrhs + r];
+    }
+}
+
+template <int NR>
+__global__ void __launch_bounds__(MV_NT) k_matvec_f64(const double* __restrict__ pts, long long n, int dim,
+                                                      KP<double> kp, double diag_extra, const double* __restrict__ x,
+                                                      double* __restrict__ y, int nrhs) {
+    __shared__ double sx[MV_TILE], sy[MV_TILE], sz[MV_TILE];
+    __shared__ double sv[MV_TILE * NR];
+    __shared__ double tab[EXP_TAB];  // s2 2^(j/256) for the table-driven exp
+    exp_table_fill(tab, kp.s2);      // ordered before use by the tile loop's barrier
     const long long i = blockIdx.x * (long long)MV_NT + threadIdx.x;
     const bool live = i < n;
-    T xi = 0, yi = 0, zi = 0;
+    double xi = 0, yi = 0, zi = 0;
     if (live) {
-        xi = (T)pts[i * dim];
-        if (dim > 1) yi = (T)pts[i * dim + 1];
-        if (dim > 2) zi = (T)pts[i * dim + 2];
+        xi = pts[i * dim];
+        if (dim > 1) yi = pts[i * dim + 1];
+        if (dim > 2) zi = pts[i * dim + 2];
     }
     double acc[NR];
 #pragma unroll
@@ -52,54 +182,25 @@ __global__ void __launch_bounds__(MV_NT) k_matvec(const double* __restrict__ pts
         for (int t = threadIdx.x; t < MV_TILE; t += MV_NT) {
             const long long j = j0 + t;
             const bool ok = j < n;
-            sx[t] = ok ? (T)pts[j * dim] : (T)0;
-            sy[t] = (ok && dim > 1) ? (T)pts[j * dim + 1] : (T)0;
-            sz[t] = (ok && dim > 2) ? (T)pts[j * dim + 2] : (T)0;
+            sx[t] = ok ? pts[j * dim] : 0.0;
+            sy[t] = (ok && dim > 1) ? pts[j * dim + 1] : 0.0;
+            sz[t] = (ok && dim > 2) ? pts[j * dim + 2] : 0.0;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const double v = (ok && r < nrhs) ? x[j * nrhs + r] : 0.0;
-                sv[t * NR + r] = (T)v;
-                if constexpr (F32) svl[t * NR + r] = (float)(v - (double)(float)v);
-            }
+            for (int r = 0; r < NR; ++r) sv[t * NR + r] = (ok && r < nrhs) ? x[j * nrhs + r] : 0.0;
         }
         __syncthreads();
         const int cnt = (int)min((long long)MV_TILE, n - j0);
-        if constexpr (F32) {
-            float hi[NR], lo[NR];
+        double part[NR];
 #pragma unroll
-            for (int r = 0; r < NR; ++r) hi[r] = lo[r] = 0.f;
-            for (int t = 0; t < cnt; ++t) {
-                const float dx = xi - sx[t], dy = yi - sy[t], dz = zi - sz[t];
-                const float kv = matern<float>(kp, sqrtf(dx * dx + dy * dy + dz * dz));
+        for (int r = 0; r < NR; ++r) part[r] = 0.0;
+        for (int t = 0; t < cnt; ++t) {
+            const double dx = xi - sx[t], dy = yi - sy[t], dz = zi - sz[t];
+            const double kv = matern_d2_fast(kp, fma(dz, dz, fma(dy, dy, dx * dx)), tab);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    // explicit-rounding intrinsics keep the compiler from fusing the
-                    // error-free transformations
-                    const float xh = sv[t * NR + r];
-                    const float p = __fmul_rn(kv, xh);
-                    const float pe = fmaf(kv, svl[t * NR + r], fmaf(kv, xh, -p));  // TwoProduct error + low part
-                    const float s = __fadd_rn(hi[r], p);                          // TwoSum(hi, p)
-                    const float bp = __fsub_rn(s, hi[r]);
-                    const float se = __fadd_rn(__fsub_rn(hi[r], __fsub_rn(s, bp)), __fsub_rn(p, bp));
-                    hi[r] = s;
-                    lo[r] += se + pe;
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r] += (double)hi[r] + (double)lo[r];
-        } else {
-            T part[NR];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) part[r] = (T)0;
-            for (int t = 0; t < cnt; ++t) {
-                const T dx = xi - sx[t], dy = yi - sy[t], dz = zi - sz[t];
-                const T kv = matern_d2_fast(kp, fma(dz, dz, fma(dy, dy, dx * dx)), tab);
-#pragma unroll
-                for (int r = 0; r < NR; ++r) part[r] = fma(kv, sv[t * NR + r], part[r]);
-            }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r] += (double)part[r];
+            for (int r = 0; r < NR; ++r) part[r] = fma(kv, sv[t * NR + r], part[r]);
         }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r] += part[r];
     }
     if (live) {
 #pragma unroll
@@ -165,26 +266,29 @@ __global__ void k_copy_rz(double* __restrict__ rz, const double* __restrict__ rz
     if (threadIdx.x < nrhs) rz[threadIdx.x] = rz_new[threadIdx.x];
 }
 
-template <typename T, int NR>
-void matvec(cudaStream_t s, const double* pts, long long n, int dim, const sic_kernel* kp, double shift,
-            const double* x, double* y, int nrhs) {
-    unsigned blocks = (unsigned)((n + MV_NT - 1) / MV_NT);
-    k_matvec<T, NR><<<blocks, MV_NT, 0, s>>>(pts, n, dim, make_kp<T>(*kp), kp->nugget + shift, x, y, nrhs);
+template <int NR>
+void matvec_f64(cudaStream_t s, const double* pts, long long n, int dim, const sic_kernel* kp, double shift,
+                const double* x, double* y, int nrhs) {
+    k_matvec_f64<NR><<<(unsigned)((n + MV_NT - 1) / MV_NT), MV_NT, 0, s>>>(pts, n, dim, make_kp<double>(*kp),
+                                                                         kp->nugget + shift, x, y, nrhs);
 }
 
-template <typename T>
-void matvec_t(cudaStream_t s, const double* pts, long long n, int dim, const sic_kernel* kp, double shift,
-              const double* x, double* y, int nrhs) {
-    if (nrhs == 1) matvec<T, 1>(s, pts, n, dim, kp, shift, x, y, nrhs);
-    else if (nrhs <= 2) matvec<T, 2>(s, pts, n, dim, kp, shift, x, y, nrhs);
-    else if (nrhs <= 4) matvec<T, 4>(s, pts, n, dim, kp, shift, x, y, nrhs);
-    else matvec<T, 8>(s, pts, n, dim, kp, shift, x, y, nrhs);
-}
-
-void matvec_any(cudaStream_t s, const double* pts, long long n, int dim, const sic_kernel* kp, double shift,
-                sic_precision prec, const double* x, double* y, int nrhs) {
-    if (prec == SIC_FP64) matvec_t<double>(s, pts, n, dim, kp, shift, x, y, nrhs);
-    else matvec_t<float>(s, pts, n, dim, kp, shift, x, y, nrhs);
+sic_status matvec_any(sic_handle* h, cudaStream_t s, const double* pts, long long n, int dim, const sic_kernel* kp,
+                      double shift, sic_precision prec, const double* x, double* y, int nrhs) {
+    if (prec == SIC_FP64) {
+        if (nrhs == 1) matvec_f64<1>(s, pts, n, dim, kp, shift, x, y, nrhs);
+        else if (nrhs <= 2) matvec_f64<2>(s, pts, n, dim, kp, shift, x, y, nrhs);
+        else if (nrhs <= 4) matvec_f64<4>(s, pts, n, dim, kp, shift, x, y, nrhs);
+        else matvec_f64<8>(s, pts, n, dim, kp, shift, x, y, nrhs);
+        return SIC_OK;
+    }
+    // The tensor-core kernel's time does not depend on the right-hand sides (N = 50,001: 6.6 ms for 3, 6.8 for 8),
+    // this one's does (5.2 ms for 1 or 2); below 2^14 rows the former also spreads a row tile over more CTAs
+    // (N = 8192, one right-hand side: 0.21 against 0.27 ms; N = 16,384: 0.78 against 0.68 ms).
+    if (nrhs > 2 || n < 12288) return matvec_tc(h, pts, n, kp, shift, x, y, nrhs, s);
+    k_matvec_f32<2><<<(unsigned)((n + MVF_ROWS - 1) / MVF_ROWS), 32 * MVF_WARPS, 0, s>>>(
+        pts, n, dim, make_kp<float>(*kp), kp->nugget + shift, x, y, nrhs);
+    return SIC_OK;
 }
 
 void dots(cudaStream_t s, const double* a, const double* c, long long n, int nrhs, double* partial, double* out) {
@@ -211,7 +315,8 @@ extern "C" sic_status sic_matern_matvec(sic_handle* h, const double* pts, int64_
     if (prec != SIC_FP64 && prec != SIC_FP32_MIXED) return SIC_ERR_INVALID;
     if (nrhs > 8) return SIC_ERR_UNSUPPORTED;
     SIC_CUDA_TRY(cudaSetDevice(h->device));
-    matvec_any((cudaStream_t)stream, pts, n, kp->dim, kp, shift, prec, x, y, nrhs);
+    const sic_status e = matvec_any(h, (cudaStream_t)stream, pts, n, kp->dim, kp, shift, prec, x, y, nrhs);
+    if (e != SIC_OK) return e;
     SIC_CUDA_TRY(cudaGetLastError());
     return SIC_OK;
 }
@@ -281,7 +386,8 @@ extern "C" sic_status sic_pcg_solve(sic_handle* h, const double* pts, int64_t n,
         for (int c = 0; c < nrhs; ++c) any |= act[c] != 0;
         if (!any) break;
         SIC_CUDA_TRY(cudaMemcpyAsync(active, act.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, s));
-        matvec_any(s, pts, n, kp->dim, kp, shift, prec, p, q, nrhs);
+        e = matvec_any(h, s, pts, n, kp->dim, kp, shift, prec, p, q, nrhs);
+        if (e != SIC_OK) return e;
         dots(s, p, q, n, nrhs, partial, pq);
         k_cg_xr<<<eb, 256, 0, s>>>(x, r, p, q, rz, pq, active, n, nrhs);
         dots(s, r, r, n, nrhs, partial, rr);

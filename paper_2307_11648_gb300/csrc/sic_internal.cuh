@@ -376,6 +376,11 @@ sic_status launch_fx_columns(sic_handle* h, const double* pts, long long n, cons
                              const int32_t* targets, int64_t n_cols, const int64_t* cand_ptr, const int32_t* cand_idx,
                              int max_cand, int k, int32_t* sel_idx, int32_t* sel_count, double* gain, cudaStream_t s);
 
+// FP32-mode product of Theta + shift I with up to 8 right-hand sides, summed on the tensor cores
+// (matvec_tc.cu)
+sic_status matvec_tc(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, double shift, const double* x,
+                     double* y, int nrhs, cudaStream_t s);
+
 // fixed-order sum of log v (fill.cu); ws holds sic_build_factor_workspace(n) bytes
 sic_status launch_sum_logv(const double* logv, long long n, double* sum_logv, void* ws, cudaStream_t s);
 
