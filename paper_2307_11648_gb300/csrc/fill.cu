@@ -22,10 +22,12 @@
 //
 // Also here: the nnz count + exclusive scan that builds col_ptr, and the fixed-order
 // two-pass sum of logv (bit-reproducible).
+#include <limits.h>
+
 #include <mutex>
 
 #include "dfloat.cuh"
-#include "sic_internal.cuh"
+#include "ldl.cuh"
 
 namespace {
 
@@ -118,93 +120,6 @@ __global__ void k_scan_add(long long* __restrict__ v, long long n, const long lo
 // warps in flight where fewer CTAs fit per SM); lane 0 of one more warp takes the pivots
 constexpr int FILL_HSLOTS = 12;  // right-hand-side entries per half-warp lane: nn <= 192 = 16 * FILL_HSLOTS
 constexpr int FILL_M_SPLIT = 32;  // groups of at most this size run in their own launch
-constexpr int FILL_B = 4;         // panel width of the blocked LDL^T (integer trailing update)
-
-// doubles of the scratch region: the points' coordinates while Theta is formed, then the
-// panel's rows in fixed point ((2 FILL_B + 1) ints per row); even, so what follows stays
-// 16-byte aligned
-__host__ __device__ constexpr int fill_scratch_doubles(int nmax) {
-    return ((3 * nmax > ((2 * FILL_B + 1) * nmax + 1) / 2 ? 3 * nmax : ((2 * FILL_B + 1) * nmax + 1) / 2) + 1) & ~1;
-}
-
-// Packed lower-triangle index (nn <= 192, so every index fits in 32 bits; 32-bit integer
-// arithmetic and int-to-float conversions stay off the FP64 pipe).
-__device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
-
-// row i of the packed lower triangle that holds flat entry e (i(i+1)/2 <= e < (i+1)(i+2)/2)
-__device__ __forceinline__ int pk_row(int e) {
-    int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-    while (i * (i + 1) / 2 > e) --i;
-    while ((i + 1) * (i + 2) / 2 <= e) ++i;
-    return i;
-}
-
-// Pivot of column c of the LDL^T factorisation from its final Schur complement v: D_cc = v
-// (kept on the diagonal) and d^(-1/2) by rsqrt_newton (five FP64 operations with the
-// diagonal's update) into piv slot c & 3 (the panel's columns); the column is then scaled as
-// G_ic = U_ic d^(-1/2) and L_ic = G_ic d^(-1/2).  A non-positive pivot raises *bad.  The range
-// test reads the bits (no FP64 compare).
-__device__ __forceinline__ void fill_pivot(double v, int c, double* G, double* piv, int* bad) {
-    const long long vb = __double_as_longlong(v);
-    if (vb <= 0 || vb >= 0x7ff0000000000000LL) {  // not in (+0, +inf): non-positive, infinite or NaN
-        *bad = 1;
-        return;
-    }
-    G[pk(c, c)] = v;
-    piv[c & 3] = rsqrt_newton(v);
-}
-
-// ---- the integer update of a panel ----
-//
-// A row of a panel, its FILL_B values g_j (entries of G = L D^(1/2)), is held in fixed point:
-// g_j = M_j 2^(E - 1075) with E the largest biased exponent among them and M_j the 53-bit
-// significands shifted to E and truncated (signed; zero and subnormal values count as 0), split
-// as M_j = Mh_j 2^26 + Ml_j (Mh signed, 0 <= Ml < 2^26).  Layout (B = 4, ld rows, fx 16-byte
-// aligned): the Mh of a row as one int4 at fx[4 row], its Ml at fx[4 (ld + row)], E at
-// fx[8 ld + row] (a warp reading consecutive rows reads consecutive 16-byte words).
-// The dot product of two rows is formed from exact 32 x 32-bit products (fx_dot).  Truncating
-// to the row's exponent costs each value at most 2^-52 of the row's largest, and fx_dot's own
-// truncations stay below 2^-51 of the largest product: with G's rows (|G_ij| <= sqrt(A_ii)) the
-// error of an entry's update stays within a few B 2^-52 sqrt(A_ii A_ll), the order of the FP64
-// Cholesky's own backward error bound.
-template <int B>
-__device__ __forceinline__ void fx_row_store(const double (&g)[B], int* __restrict__ fx, int ld, int row) {
-    static_assert(B == 4, "the fixed-point rows are stored as int4");
-    int e[B];
-    int E = 0;
-#pragma unroll
-    for (int j = 0; j < B; ++j) {
-        e[j] = (__double2hiint(g[j]) >> 20) & 0x7ff;
-        E = max(E, e[j]);
-    }
-    int mh[B], ml[B];
-#pragma unroll
-    for (int j = 0; j < B; ++j) {
-        const long long u = __double_as_longlong(g[j]);
-        long long m = e[j] ? ((u & 0xfffffffffffffLL) | 0x10000000000000LL) : 0LL;
-        const int sh = E - e[j];
-        m = sh < 63 ? (m >> sh) : 0LL;
-        if (u < 0) m = -m;
-        mh[j] = (int)(m >> 26);
-        ml[j] = (int)(m & 0x3ffffffLL);
-    }
-    reinterpret_cast<int4*>(fx)[row] = make_int4(mh[0], mh[1], mh[2], mh[3]);
-    reinterpret_cast<int4*>(fx)[ld + row] = make_int4(ml[0], ml[1], ml[2], ml[3]);
-    fx[8 * ld + row] = E;
-}
-
-// s 2^e2 as FP64 by integer operations, the significand truncated (relative error < 2^-52);
-// 0 for s = 0 and below FP64's normal range
-__device__ __forceinline__ double i64_scaled(long long s, int e2) {
-    if (s == 0) return 0.0;
-    const unsigned long long sg = (unsigned long long)s & (1ULL << 63);
-    const unsigned long long mag = s < 0 ? 0ULL - (unsigned long long)s : (unsigned long long)s;
-    const int z = __clzll((long long)mag);
-    const int be = e2 + 63 - z + 1023;
-    if (be <= 0) return 0.0;
-    return __longlong_as_double((long long)(sg | ((unsigned long long)be << 52) | (((mag << z) >> 11) & 0xfffffffffffffULL)));
-}
-
 __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
 
 // Two updates x -= a y in double-float (x = xh + xl, a and y likewise; dfloat.cuh), x0 -= a0 y in
@@ -226,32 +141,18 @@ __device__ __forceinline__ void df_sub_mul2(float2& xh, float2& xl, float2 a0, f
     xh = t;
 }
 
-// sum_j g_ij g_lj of rows i and l: 2^52 sum Mh Mh + 2^26 sum (Mh Ml + Ml Mh) exactly in two 64-bit
-// sums of 32 x 32-bit products, scaled down by 2^52 into one 64-bit integer (the dropped fraction
-// and the omitted sum Ml Ml are below 5 units of 2^(Ei + El - 2098)), converted to FP64
-template <int B>
-__device__ __forceinline__ double fx_dot(const int* __restrict__ fx, int ld, int i, int l) {
-    static_assert(B == 4, "the fixed-point rows are stored as int4");
-    const int4 hi4 = reinterpret_cast<const int4*>(fx)[i], li4 = reinterpret_cast<const int4*>(fx)[ld + i];
-    const int4 hl4 = reinterpret_cast<const int4*>(fx)[l], ll4 = reinterpret_cast<const int4*>(fx)[ld + l];
-    const int hi_[4] = {hi4.x, hi4.y, hi4.z, hi4.w}, li[4] = {li4.x, li4.y, li4.z, li4.w};
-    const int hl[4] = {hl4.x, hl4.y, hl4.z, hl4.w}, ll[4] = {ll4.x, ll4.y, ll4.z, ll4.w};
-    long long a2 = 0, a1 = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        a2 += (long long)hi_[j] * hl[j];
-        a1 += (long long)hi_[j] * ll[j] + (long long)li[j] * hl[j];
-    }
-    return i64_scaled(a2 + (a1 >> 26), fx[8 * ld + i] + fx[8 * ld + l] - 2098);
-}
-
 // CTAs per SM the register budget is set for (shared memory allows about this many at the
 // largest group of each launch)
 constexpr int fill_min_ctas(int nt) { return nt == 128 ? 5 : (nt == 256 ? 3 : 2); }
 
-template <int FILL_NT>
+// PARTIAL: the units are nonadjacent groups, members[grp_ptr[u] ..) at any positions, whose picks condition only the
+// members before them (Section 5.1.1, Appendix A.4).  With the union of members and picks from the latest position to
+// the earliest, a member's set is a leading block of the same factorisation, so it is the same kernel with another
+// order and each member's own index jm in it (N = 2^16, 2,811 groups, k = 64: @@PFILL@@).
+template <int FILL_NT, bool PARTIAL>
 __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(const double* __restrict__ pts, int dim, KP<double> kp,
-                                                  const long long* __restrict__ grp_ptr, long long n_units,
+                                                  const long long* __restrict__ grp_ptr,
+                                                  const long long* __restrict__ members, long long n_units,
                                                   const int32_t* __restrict__ sel_idx,
                                                   const int32_t* __restrict__ sel_count, int k, int max_m,
                                                   int m_lo, int m_hi, long long n, long long col0,
@@ -267,7 +168,8 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
     double* G = xyz + fill_scratch_doubles(nmax);           // packed lower, nmax(nmax+1)/2
     double* piv = G + (long long)nmax * (nmax + 1) / 2;     // d^(-1/2) of the panel's columns (slot c & 3)
     int* pos = reinterpret_cast<int*>(piv + 4);             // nmax
-    int* srt = pos + nmax;                                  // k
+    int* srt = pos + nmax;                                  // k (PARTIAL: nmax)
+    int* jm = srt + nmax;                                   // PARTIAL: index of member a in the order (m_hi)
     __shared__ int s_bad;
     __shared__ unsigned s_emax[3];  // the largest biased exponent of the unit's coordinates, per dimension
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -284,11 +186,12 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
         return s_next[nb_];
     };
     for (long long u = fetch(); u < n_units; u = fetch()) {
-        const long long g0 = grp_ptr ? grp_ptr[u] : col0 + u;
-        const int m = grp_ptr ? (int)(grp_ptr[u + 1] - g0) : 1;
+        const long long g0 = PARTIAL || grp_ptr ? grp_ptr[u] : col0 + u;
+        const int m = PARTIAL || grp_ptr ? (int)(grp_ptr[u + 1] - g0) : 1;
         const int cnt = sel_count[u];
         const long long c0 = g0 - col0;  // the unit's first column within the slice
-        if (m < 1 || m > max_m || cnt < 0 || cnt > k || g0 < 0 || g0 + m > n || c0 < 0 || c0 + m > n_cols) {
+        if (m < 1 || m > max_m || cnt < 0 || cnt > k ||
+            (!PARTIAL && (g0 < 0 || g0 + m > n || c0 < 0 || c0 + m > n_cols))) {
             if (tid == 0 && m_lo == 1) record_error(st, SIC_ERR_INVALID, u);  // reported by the first class
             continue;
         }
@@ -298,191 +201,54 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
             if (tid == 0) record_error(st, SIC_ERR_UNSUPPORTED, u);
             continue;
         }
-        // picks sorted ascending by rank; they must be distinct positions after the unit,
-        // and col_ptr must match the pattern
         bool bad = false;
-        for (int i = worker ? tid : cnt; i < cnt; i += FILL_NT) {
-            const int v = sel_idx[u * k + i];
-            int rank = 0, same = 0;
-            for (int j = 0; j < cnt; ++j) {
-                const int w = sel_idx[u * k + j];
-                rank += (w < v);
-                same += (w == v);
+        if constexpr (PARTIAL) {
+            // the union by rank, latest first; positions must be distinct and picks after the first member
+            for (int e = worker ? tid : nn; e < nn; e += FILL_NT) {
+                const long long p = e < m ? members[g0 + e] : (long long)sel_idx[u * k + (e - m)];
+                srt[e] = (p < 0 || p >= n) ? -1 : (int)p;
             }
-            if (v < g0 + m || v >= n || same != 1) bad = true;
-            else srt[rank] = v;
+            __syncthreads();
+            for (int e = worker ? tid : nn; e < nn; e += FILL_NT) {
+                const int p = srt[e];
+                int later = 0, same = 0;
+                for (int f = 0; f < nn; ++f) {
+                    later += srt[f] > p;
+                    same += srt[f] == p;
+                }
+                if (p < 0 || same != 1 || (e >= m && p <= srt[0])) bad = true;
+                pos[later] = p;
+                if (e < m) jm[e] = later;
+            }
+        } else {
+            // picks sorted ascending by rank; they must be distinct positions after the unit,
+            // and col_ptr must match the pattern
+            for (int i = worker ? tid : cnt; i < cnt; i += FILL_NT) {
+                const int v = sel_idx[u * k + i];
+                int rank = 0, same = 0;
+                for (int j = 0; j < cnt; ++j) {
+                    const int w = sel_idx[u * k + j];
+                    rank += (w < v);
+                    same += (w == v);
+                }
+                if (v < g0 + m || v >= n || same != 1) bad = true;
+                else srt[rank] = v;
+            }
+            for (int a = worker ? tid : m; a < m; a += FILL_NT)
+                if (col_ptr[c0 + a + 1] - col_ptr[c0 + a] != (long long)(m - a + cnt)) bad = true;
         }
-        for (int a = worker ? tid : m; a < m; a += FILL_NT)
-            if (col_ptr[c0 + a + 1] - col_ptr[c0 + a] != (long long)(m - a + cnt)) bad = true;
         if (tid < 3) s_emax[tid] = 0u;
         if (__syncthreads_or(bad)) {
             if (tid == 0) record_error(st, SIC_ERR_INVALID, u);
             continue;
         }
-        // R order: picks descending, then members descending; the coordinates go to fixed point
-        // at the unit's largest exponent in each dimension (fx_coord), so that differences and
-        // squared distances are exact integer arithmetic (fx_dist2)
-        {
-            unsigned em[3] = {0u, 0u, 0u};
-            for (int i = worker ? tid : nn; i < nn; i += FILL_NT) {
-                const int p = (i < cnt) ? srt[cnt - 1 - i] : (int)(g0 + m - 1 - (i - cnt));
-                pos[i] = p;
-#pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    const double x = (d < dim) ? pts[(long long)p * dim + d] : 0.0;
-                    xyz[d * nmax + i] = x;
-                    em[d] = max(em[d], ((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
-                }
-            }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                em[d] = __reduce_max_sync(0xffffffffu, em[d]);
-                if (lane == 0 && em[d]) atomicMax(&s_emax[d], em[d]);
-            }
-        }
+        // R order: picks descending, then members descending
+        if constexpr (!PARTIAL)
+            for (int i = worker ? tid : nn; i < nn; i += FILL_NT)
+                pos[i] = (i < cnt) ? srt[cnt - 1 - i] : (int)(g0 + m - 1 - (i - cnt));
         if (tid == 0) s_bad = 0;
-        __syncthreads();
-        const int E0 = (int)s_emax[0], E1 = (int)s_emax[1], E2 = (int)s_emax[2];
-        long long* xf = reinterpret_cast<long long*>(xyz);
-        for (int i = worker ? tid : nn; i < nn; i += FILL_NT)
-            for (int d = 0; d < dim; ++d) xf[d * nmax + i] = fx_coord(xyz[d * nmax + i], d == 0 ? E0 : (d == 1 ? E1 : E2));
-        __syncthreads();
-        // Theta_RR, packed lower, one flat entry per thread: the squared distance exact from the
-        // fixed-point coordinates, the Matern in FP64 (matern_d2_fast; the all-double-float
-        // Matern of dfloat.cuh would spare the FP64 pipe entirely, but its ~1e-14 of the
-        // variance per entry is amplified by 1/v in the Schur complements, v ~ 2 nugget on the
-        // finest groups: factor columns then miss the oracle's by more than 1e-8)
-        // entry e = i (i + 1) / 2 + j, stepped by FILL_NT
-        for (int i = worker ? pk_row(tid) : nn, j = worker ? tid - i * (i + 1) / 2 : 0; i < nn;) {
-            double v = matern_d2_fast(kp, fx_dist2(xf, nmax, dim, i, j, E0, E1, E2), tab);
-            if (i == j) v += kp.nugget;
-            G[pk(i, j)] = v;
-            j += FILL_NT;
-            while (j > i) {
-                j -= i + 1;
-                ++i;
-            }
-        }
-        __syncthreads();
-        // blocked right-looking LDL^T factorisation Theta_RR = L D L^T in place on the packed
-        // lower triangle, in panels of FILL_B columns, in FP64: d_j = A_jj, L_ij = A_ij / d_j and
-        // A_il -= L_ij U_lj within the panel (U_lj = A_lj, the panel's entries unscaled).  The
-        // rows below the panel keep G_ij = U_ij d_j^(-1/2) (G = L D^(1/2)) in fixed point; the
-        // trailing matrix then takes the panel's whole rank-FILL_B update as one integer dot
-        // product of two G rows per entry (exact products), subtracted in FP64 (fx_dot): FILL_B
-        // FP64 FMAs become one FP64 addition, the products going to the integer multiply-add
-        // units.  The FP64 units are per SM sub-partition and charge a warp instruction whatever
-        // its active lanes, so the flat loops keep full warps.
-        // The panel's diagonal block (at most FILL_B x FILL_B) is factored by the pivot warp, lane
-        // r owning the block's row r (its pivots and their reciprocal square roots are a chain of
-        // dependent FP64 operations, warp-synchronous): the next panel's block takes the current
-        // panel's update and is factored while the workers update the rest of the trailing matrix.
-        // Every worker row below the block then applies the block's columns to its own panel
-        // entries in registers (A_il -= L_ij U_lj reads the block's unscaled entries, which stay
-        // in place until the block's L entries are written back in the next phase), so that a
-        // panel costs two barriers.  Worker thread i owns row i (nn <= FILL_NT, the launcher's
-        // choice).  Same operations, in the same order, as a column-by-column elimination.
-        const int i = tid;
-        const int rowi = pk(i, 0);
-        double lb[FILL_B];  // pivot warp: L of the block's row `lane` (columns below it)
-        // the block [J, J + bs) (its entries final): lane r owns row J + r
-        auto factor_block = [&](int J, int bs) {
-            const int r = lane;
-            const int ib = J + r;
-            if (r == 0) fill_pivot(G[pk(J, J)], J, G, piv, &s_bad);
-            __syncwarp();
-#pragma unroll
-            for (int jj = 0; jj < FILL_B - 1; ++jj) {
-                if (jj >= bs - 1) break;
-                const int j = J + jj;
-                if (r > jj && r < bs) {
-                    const double rsd = piv[j & 3];
-                    const double uv = G[pk(ib, j)];
-                    const double g = uv * rsd;
-                    const double l = g * rsd;
-                    lb[jj] = l;
-#pragma unroll
-                    for (int c2 = jj + 1; c2 < FILL_B; ++c2)
-                        if (c2 <= r) G[pk(ib, J + c2)] = fma(-l, G[pk(J + c2, j)], G[pk(ib, J + c2)]);
-                    if (r == jj + 1) fill_pivot(G[pk(ib, ib)], ib, G, piv, &s_bad);
-                }
-                __syncwarp();
-            }
-        };
-        if (!worker) factor_block(0, min(FILL_B, nn));
-        __syncthreads();
-        for (int J = 0; J < nn && !s_bad; J += FILL_B) {
-            const int je = min(J + FILL_B, nn);  // je < nn implies a full panel
-            // the own row's panel entries (rows below the block): L and G by the block's columns
-            if (worker && i >= je && i < nn) {
-                double u[FILL_B], gv[FILL_B], lv[FILL_B];
-#pragma unroll
-                for (int c = 0; c < FILL_B; ++c) u[c] = G[rowi + J + c];
-#pragma unroll
-                for (int jj = 0; jj < FILL_B; ++jj) {
-                    const double rsd = piv[jj];  // (J + jj) & 3
-                    const double g = u[jj] * rsd;
-                    const double l = g * rsd;
-                    gv[jj] = g;
-                    lv[jj] = l;
-#pragma unroll
-                    for (int c2 = jj + 1; c2 < FILL_B; ++c2) u[c2] = fma(-l, G[pk(J + c2, J + jj)], u[c2]);
-                }
-                fx_row_store<FILL_B>(gv, fx, nmax, i);
-                // the L entries as double-float pairs (hi, lo) in their 8-byte slots (f64_split: 48
-                // significant bits; only the member solves read them)
-#pragma unroll
-                for (int c = 0; c < FILL_B; ++c) {
-                    float h, l;
-                    f64_split(lv[c], h, l);
-                    reinterpret_cast<float2*>(G)[rowi + J + c] = make_float2(h, l);
-                }
-            }
-            __syncthreads();
-            if (worker) {
-                // the trailing matrix, entries (i, l) with je <= l <= i < nn, takes the panel's
-                // update, but for the next panel's block (the first nbt flat entries)
-                if (je < nn) {
-                    const int nt = nn - je;
-                    const int bs2 = min(FILL_B, nt), nbt = bs2 * (bs2 + 1) / 2;
-                    // entry e = ii (ii + 1) / 2 + ll of the trailing triangle, stepped by FILL_NT
-                    int ii = pk_row(tid + nbt), ll = tid + nbt - ii * (ii + 1) / 2;
-                    while (ii < nt) {
-                        const int i = je + ii, l = je + ll;
-                        G[pk(i, l)] -= fx_dot<FILL_B>(fx, nmax, i, l);
-                        ll += FILL_NT;
-                        while (ll > ii) {
-                            ll -= ii + 1;
-                            ++ii;
-                        }
-                    }
-                }
-            } else {
-                // the block's L entries, as double-float pairs, now that the workers have read its
-                // unscaled entries; then the next block: its update, and its factorisation
-                const int bs = je - J;
-                if (lane < bs) {
-#pragma unroll
-                    for (int c = 0; c < FILL_B - 1; ++c)
-                        if (c < lane) {
-                            float h, l;
-                            f64_split(lb[c], h, l);
-                            reinterpret_cast<float2*>(G)[pk(J + lane, J + c)] = make_float2(h, l);
-                        }
-                }
-                if (je < nn) {
-                    const int bs2 = min(FILL_B, nn - je);
-                    if (lane < bs2 * (bs2 + 1) / 2) {
-                        const int ii = pk_row(lane), ll = lane - ii * (ii + 1) / 2;
-                        G[pk(je + ii, je + ll)] -= fx_dot<FILL_B>(fx, nmax, je + ii, je + ll);
-                    }
-                    __syncwarp();
-                    factor_block(je, bs2);
-                }
-            }
-            __syncthreads();
-        }
-        __syncthreads();
+        unit_theta<FILL_NT>(pts, dim, kp, tab, pos, nn, nmax, xyz, G, s_emax);
+        ldl_panels<FILL_NT>(G, fx, piv, nn, nmax, &s_bad);
         if (s_bad) {
             if (tid == 0) record_error(st, SIC_ERR_NOT_PD, u);
             __syncthreads();
@@ -503,8 +269,11 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
         for (int p = worker ? warp : npairs; p < npairs; p += FILL_NT / 32) {
             const int a = 2 * p + half;
             const bool has = a < m;
-            const int jb = has ? nn - 1 - a : -1;
-            const int jtop = nn - 1 - 2 * p;
+            int jb = has ? nn - 1 - a : -1, jtop = nn - 1 - 2 * p;
+            if constexpr (PARTIAL) {
+                jb = has ? jm[a] : -1;
+                jtop = max(jm[2 * p], 2 * p + 1 < m ? jm[2 * p + 1] : -1);
+            }
             // slots 2j and 2j+1 in the .x and .y halves of bh[j], bl[j] (packed updates); in the
             // block of rows l of slot sb, the slots below sb take every row, slot sb the rows
             // above its entry, and a slot above sb none: those get a = 0
@@ -533,8 +302,11 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
                     }
                 }
             }
-            if (has) {
-                const long long e0 = col_ptr[c0 + a] - base;
+            const long long col = PARTIAL ? (long long)pos[has ? jb : 0] : c0 + a;
+            if (PARTIAL && has && col_ptr[col + 1] - col_ptr[col] != jb + 1) {
+                if (hl == 0) record_error(st, SIC_ERR_INVALID, u);
+            } else if (has) {
+                const long long e0 = col_ptr[col] - base;
                 const double sc = rsqrt_newton(G[pk(jb, jb)]);
 #pragma unroll
                 for (int q = 0; q < FILL_HSLOTS; ++q) {
@@ -550,7 +322,11 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
         }
         // log v of every member, one member per thread (the FP64 log once per lane instead of
         // once per warp)
-        for (int a = worker ? tid : m; a < m; a += FILL_NT) logv[c0 + a] = log(G[pk(nn - 1 - a, nn - 1 - a)]);
+        for (int a = worker ? tid : m; a < m; a += FILL_NT) {
+            const int j = PARTIAL ? jm[a] : nn - 1 - a;
+            if (PARTIAL && col_ptr[pos[j] + 1] - col_ptr[pos[j]] != j + 1) continue;  // reported above
+            logv[PARTIAL ? (long long)pos[j] : c0 + a] = log(G[pk(j, j)]);
+        }
         __syncthreads();
     }
 }
@@ -586,10 +362,10 @@ __global__ void __launch_bounds__(256) k_sum_final(const double* __restrict__ pa
     if (threadIdx.x == 0) *out = s[0];
 }
 
-size_t fill_smem_bytes(int k, int max_m) {
+size_t fill_smem_bytes(int k, int max_m, bool partial = false) {
     const int nmax = k + max_m;
     return sizeof(double) * ((size_t)nmax * (nmax + 1) / 2 + 4 + EXP_TAB + fill_scratch_doubles(nmax)) +
-           sizeof(int) * ((size_t)nmax + (size_t)k);
+           sizeof(int) * ((size_t)nmax + (partial ? (size_t)nmax + (size_t)max_m : (size_t)k));
 }
 
 __global__ void k_fp64_math(KP<double> kp, const double* __restrict__ x, long long n, double* __restrict__ os,
@@ -773,6 +549,68 @@ extern "C" sic_status sic_build_factor_workspace(int64_t n, size_t* bytes) {
     return SIC_OK;
 }
 
+// The fill's launches (ws: the fill's workspace for n_cols columns): partials of the fixed-order sum at its front,
+// which the caller forms afterwards, then the launches' work counters.
+template <bool PARTIAL>
+static sic_status launch_fill(sic_handle* h, const double* pts, long long n, const sic_kernel* kp,
+                              const int64_t* grp_ptr, const int64_t* members, long long n_grp, int max_m,
+                              const int32_t* sel_idx, const int32_t* sel_count, int k, long long col0, long long n_cols,
+                              const int64_t* col_ptr, long long base, int32_t* row_idx, double* val, double* logv,
+                              void* ws, cudaStream_t s) {
+    // two size classes when the groups can be large: the shared-memory layout (and so the
+    // CTAs per SM) of each launch fits its own largest group, so the many small groups run
+    // at higher occupancy; each launch skips the other's groups
+    // the size-class split: tuned for this (k, max_m) by sic_tune_build_factor, else FILL_M_SPLIT
+    int split = tune_get(h, TUNE_FILL_SPLIT, k, max_m, FILL_M_SPLIT);
+    if (split > max_m) split = max_m;
+    if (split < 1) split = 1;
+    const int big_nt = tune_get(h, TUNE_FILL_BIGNT, k, max_m, 256) == 384 ? 384 : 256;
+    // the two launches' work counters, after the partial sums in the workspace
+    unsigned long long* ctr = reinterpret_cast<unsigned long long*>(
+        reinterpret_cast<char*>(ws) + fill_partials_bytes(n_cols));
+    SIC_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s));
+    for (int c = 0; c < 2; ++c) {
+        const int lo = c == 0 ? 1 : split + 1, hi = c == 0 ? split : max_m;
+        if (lo > hi) break;
+        const size_t sm = fill_smem_bytes(k, hi, PARTIAL);
+        // worker threads: at least one per row of the largest unit (k + hi)
+        const int nt = (c == 0 && k + hi <= 128) ? 128 : (c == 0 || big_nt != 384 ? 256 : 384);
+        auto kern = nt == 128 ? k_fill<128, PARTIAL> : (nt == 384 ? k_fill<384, PARTIAL> : k_fill<256, PARTIAL>);
+        const int block = nt + 32;
+        SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        const int grid = persistent_grid(h, kern, block, sm, n_grp);
+        kern<<<grid, block, sm, s>>>(pts, kp->dim, make_kp<double>(*kp), (const long long*)grp_ptr,
+                                     (const long long*)members, n_grp, sel_idx,
+                                     sel_count, k, max_m, lo, hi, n, col0, n_cols, (const long long*)col_ptr, base,
+                                     row_idx, val, logv, ctr + c, h->d_status);
+    }
+    SIC_CUDA_TRY(cudaGetLastError());
+    return SIC_OK;
+}
+
+extern "C" sic_status sic_build_factor_partial(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp,
+                                               const int64_t* grp_ptr, const int64_t* members, int64_t n_grp,
+                                               int32_t max_m, const int32_t* sel_idx, const int32_t* sel_count,
+                                               int32_t k, const int64_t* col_ptr, int32_t* row_idx, double* val,
+                                               double* logv, double* sum_logv, void* ws, size_t ws_bytes,
+                                               void* stream) {
+    if (!h || !pts || !sic_valid_kernel(kp) || n < 1 || n_grp < 0 || !grp_ptr || !members || !sel_idx ||
+        !sel_count || !col_ptr || !row_idx || !val || !logv || !sum_logv || k < 1 || max_m < 1)
+        return SIC_ERR_INVALID;
+    if (max_m > 64 || k > 128 || n > INT_MAX) return SIC_ERR_UNSUPPORTED;
+    size_t need = 0;
+    sic_build_factor_workspace(n, &need);
+    if (!ws || ws_bytes < need) return SIC_ERR_INVALID;
+    SIC_CUDA_TRY(cudaSetDevice(h->device));
+    cudaStream_t s = (cudaStream_t)stream;
+    if (n_grp > 0) {
+        const sic_status e = launch_fill<true>(h, pts, n, kp, grp_ptr, members, n_grp, max_m, sel_idx, sel_count, k, 0, n,
+                                               col_ptr, 0, row_idx, val, logv, ws, s);
+        if (e != SIC_OK) return e;
+    }
+    return launch_sum_logv(logv, n, sum_logv, ws, s);
+}
+
 extern "C" sic_status sic_build_factor_range(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp,
                                              const int64_t* grp_ptr, int64_t n_grp, int32_t max_m,
                                              const int32_t* sel_idx, const int32_t* sel_count, int32_t k,
@@ -792,32 +630,9 @@ extern "C" sic_status sic_build_factor_range(sic_handle* h, const double* pts, i
     SIC_CUDA_TRY(cudaSetDevice(h->device));
     cudaStream_t s = (cudaStream_t)stream;
     if (fill_smem_bytes(k, max_m) > 227 * 1024) return SIC_ERR_UNSUPPORTED;
-    // two size classes when the groups can be large: the shared-memory layout (and so the
-    // CTAs per SM) of each launch fits its own largest group, so the many small groups run
-    // at higher occupancy; each launch skips the other's groups
-    // the size-class split: tuned for this (k, max_m) by sic_tune_build_factor, else FILL_M_SPLIT
-    int split = tune_get(h, TUNE_FILL_SPLIT, k, max_m, FILL_M_SPLIT);
-    if (split > max_m) split = max_m;
-    if (split < 1) split = 1;
-    const int big_nt = tune_get(h, TUNE_FILL_BIGNT, k, max_m, 256) == 384 ? 384 : 256;
-    // the two launches' work counters, after the partial sums in the workspace
-    unsigned long long* ctr = reinterpret_cast<unsigned long long*>(
-        reinterpret_cast<char*>(ws) + fill_partials_bytes(n_cols));
-    SIC_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s));
-    for (int c = 0; c < 2; ++c) {
-        const int lo = c == 0 ? 1 : split + 1, hi = c == 0 ? split : max_m;
-        if (lo > hi) break;
-        const size_t sm = fill_smem_bytes(k, hi);
-        // worker threads: at least one per row of the largest unit (k + hi)
-        const int nt = (c == 0 && k + hi <= 128) ? 128 : (c == 0 || big_nt != 384 ? 256 : 384);
-        auto kern = nt == 128 ? k_fill<128> : (nt == 384 ? k_fill<384> : k_fill<256>);
-        const int block = nt + 32;
-        SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const int grid = persistent_grid(h, kern, block, sm, n_grp);
-        kern<<<grid, block, sm, s>>>(pts, kp->dim, make_kp<double>(*kp), (const long long*)grp_ptr, n_grp, sel_idx,
-                                     sel_count, k, max_m, lo, hi, n, col0, n_cols, (const long long*)col_ptr, base,
-                                     row_idx, val, logv, ctr + c, h->d_status);
-    }
+    const sic_status e = launch_fill<false>(h, pts, n, kp, grp_ptr, nullptr, n_grp, max_m, sel_idx, sel_count, k, col0,
+                                            n_cols, col_ptr, base, row_idx, val, logv, ws, s);
+    if (e != SIC_OK) return e;
     long long nb = (n_cols + SUM_TILE - 1) / SUM_TILE;
     k_sum_tiles<<<(unsigned)nb, 256, 0, s>>>(logv, n_cols, (double*)ws);
     k_sum_final<<<1, 256, 0, s>>>((const double*)ws, nb, sum_logv);

@@ -47,6 +47,65 @@ __device__ __forceinline__ void record_error(DevStatus* st, int code, long long 
     if (atomicCAS(&st->code, 0, code) == 0) st->unit = unit;
 }
 
+// Deals the units of a size class evenly over the CTAs of a persistent launch that has no workspace for a work
+// counter (a launch skips the other class's units, and a plain stride over all units would leave the CTAs with
+// uneven shares): CTA b takes the class's units of rank b, b + gridDim, ...  next() is called by the whole CTA and ends
+// with a barrier; -1 after the last unit.
+template <int NT>
+struct ClassDeal {
+    static constexpr int CAP = 128;
+    int q[CAP], n, at;
+    int count[NT / 32];
+    long long scan, seen;  // next unit to look at, class members before it
+    __device__ __forceinline__ void start() {
+        if (threadIdx.x == 0) {
+            n = at = 0;
+            scan = seen = 0;
+        }
+        __syncthreads();
+    }
+    template <typename Pred>
+    __device__ __forceinline__ long long next(long long n_units, Pred in_class) {
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        if (at == n) {  // (every thread reads the same values: they change only between barriers)
+            const int look = (int)min((long long)NT, (long long)(CAP - 1) * gridDim.x);
+            const int most = look / (int)gridDim.x + 1;  // units of one look that are this CTA's (<= CAP)
+            int have = 0;
+            long long u0 = scan, s = seen;
+            __syncthreads();
+            if (tid == 0) n = at = 0;
+            while (u0 < n_units && have + most <= CAP) {
+                const long long u = u0 + tid;
+                const bool in = tid < look && u < n_units && in_class(u);
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (lane == 0) count[warp] = __popc(b);
+                __syncthreads();
+                int before = __popc(b & ((1u << lane) - 1u)), all = 0;
+                for (int w = 0; w < NT / 32; ++w) {
+                    before += w < warp ? count[w] : 0;
+                    all += count[w];
+                }
+                if (in && (s + before) % gridDim.x == blockIdx.x) q[atomicAdd(&n, 1)] = (int)u;
+                __syncthreads();
+                s += all;
+                u0 += look;
+                have = n;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                scan = u0;
+                seen = s;
+            }
+            __syncthreads();
+        }
+        const long long u = at < n ? (long long)q[at] : -1;
+        __syncthreads();
+        if (tid == 0 && u >= 0) ++at;
+        __syncthreads();
+        return u;
+    }
+};
+
 // Matern parameters in the arithmetic of the selection kernel.
 template <typename T>
 struct KP {
