@@ -11,15 +11,19 @@
 // appends u_j = (Theta_{jq} - F_j . F_q)/sqrt(var_q) and downdates var and cov
 // (eq. cond_select).  out_var traces the target's conditional variance.
 //
-// Bound: the FP64 pipe (n k (k/2 + 17) operations; the factor, 8 n k bytes, stays in L2) plus
-// a barrier and three dependent L2 round trips per step.  One block on one SM was the whole
-// kernel before: 98.3 ms for
-// n = 65,536, k = 64 in FP64 (3-D, Matern 5/2); spread over the grid 1.16 ms.
-#include "sic_internal.cuh"
+// In FP64 the factor is held in fixed point (fx.cuh, select_fx.cu): exact integer dot products instead of FP64
+// multiply-adds, and scores in FP32 first, the FP64 quotient only where a row is within 2^-18 of its block's largest.
+//
+// Bound: a barrier and four dependent L2 round trips per step, then the factor's L2 traffic (4 n k^2 bytes) and the FP64
+// pipe.  One block on one SM was the whole kernel: 98.3 ms for n = 65,536, k = 64 in FP64 (3-D, Matern 5/2); over
+// the grid with FP64 multiply-adds and divisions 1.16 ms, in fixed point 0.85 ms.
+// Error of out_var against 128-bit arithmetic over six problems (n 300 .. 4000, k 30 .. 64): 2.0e-15 on average, 2.2e-15
+// with the library exponential and FP64 sums.
+#include "fx.cuh"
 
 namespace {
 
-constexpr int NT_MAX = 256;
+constexpr int NT_MAX = 512;
 constexpr int NW_MAX = NT_MAX / 32;
 constexpr int WAIT_POLLS = 1 << 24;  // a grid barrier gives up after this many polls
 
@@ -31,7 +35,7 @@ __device__ __forceinline__ bool better(T s, long long i, T bs, long long bi) {
 // a block's best candidate of a step
 template <typename T>
 struct Best {
-    T score, var, cov;
+    T score;
     long long idx;
 };
 
@@ -66,20 +70,26 @@ __device__ __forceinline__ bool grid_wait(unsigned* count, unsigned target) {
 
 template <typename T>
 __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restrict__ xtr, long long n, int dim,
-                                                          const double* __restrict__ xt, KP<T> kp, T floor_, int k,
-                                                          int32_t* __restrict__ out_idx,
+                                                          const double* __restrict__ xt, KP<T> kp, T floor_, int e,
+                                                          int k, int32_t* __restrict__ out_idx,
                                                           double* __restrict__ out_var,
                                                           int32_t* __restrict__ out_count, T* ws, unsigned* count,
                                                           DevStatus* st) {
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* piv = reinterpret_cast<T*>(smem_raw);  // k
+    T* piv = reinterpret_cast<T*>(smem_raw);         // k: the pivot's row (FP64: fixed point, int2)
+    __shared__ unsigned wkey[NW_MAX];
     __shared__ Best<T> wbest[NW_MAX];
-    __shared__ Best<T> gbest;
+    __shared__ long long s_q;
+    __shared__ T s_rs, s_ut;
     __shared__ int s_ok;
-    __shared__ double tab[sizeof(T) == 8 ? EXP_TAB : 1];  // s2 2^(j/256): the FP64 Matern's exp
+    __shared__ double tab[F64 ? EXP_TAB : 1];  // s2 2^(j/256): the FP64 Matern's exp
     T* F = ws;
     T* var = F + (long long)k * n;
     T* cov = var + n;
+    int2* Fx = reinterpret_cast<int2*>(ws);
+    const int2* px = reinterpret_cast<const int2*>(piv);
     Best<T>* bests = reinterpret_cast<Best<T>*>(count + 4);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const long long j0 = blockIdx.x * (long long)blockDim.x + tid, jstep = (long long)gridDim.x * blockDim.x;
@@ -87,18 +97,18 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
     double org[3] = {0.0, 0.0, 0.0};
     for (int d = 0; d < dim; ++d) org[d] = xt[d];
     auto coord = [&](long long j, int d) -> T {
-        if constexpr (sizeof(T) == 8) return (T)xtr[j * dim + d];
+        if constexpr (F64) return (T)xtr[j * dim + d];
         return (T)(xtr[j * dim + d] - org[d]);
     };
     // Theta at squared distance d2 (no nugget): in FP64 the table-driven exp and the Newton
     // square root (few FP64-pipe operations, about 2 ulp)
     auto theta = [&](T d2) -> T {
-        if constexpr (sizeof(T) == 8)
+        if constexpr (F64)
             return matern_d2_fast(kp, d2, tab);
         else
             return matern<T>(kp, sic_sqrt(d2));
     };
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (F64) {
         exp_table_fill(tab, kp.s2);
         __syncthreads();
     }
@@ -113,80 +123,100 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
     }
     double vt = (double)(kp.s2 + kp.nugget);
     if (j0 == 0) out_var[0] = vt;
+    // FP32 score key of a row (0: not a candidate)
+    auto key_of = [&](long long j) -> unsigned {
+        const T v = var[j];
+        if (!(v >= floor_)) return 0u;
+        const float c = fx_f32(fabs((double)cov[j]), 2 * e);
+        return __float_as_uint(__fdividef(c * c, fx_f32((double)v, 2 * e))) + 1u;
+    };
+    auto warp_best = [&](Best<T>& b) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const T os = __shfl_xor_sync(FULL, b.score, off);
+            const long long oi = __shfl_xor_sync(FULL, b.idx, off);
+            if (better(os, oi, b.score, b.idx)) b = Best<T>{os, oi};
+        }
+    };
     int t = 0;
     for (; t < k; ++t) {
-        Best<T> b;
-        b.score = NEG;
-        b.idx = NONE;
-        b.var = b.cov = (T)0;
-        auto take = [&](const Best<T>& o) {
-            if (better(o.score, o.idx, b.score, b.idx)) b = o;
-        };
-        for (long long j = j0; j < n; j += jstep) {
-            const T v = var[j];
-            if (v >= floor_) {
-                const T c = cov[j];
-                take(Best<T>{c * c / v, v, c, j});
-            }
+        Best<T> b{NEG, NONE};
+        unsigned lim = 1u, mine = 0u;
+        if constexpr (F64) {
+            for (long long j = j0; j < n; j += jstep) mine = max(mine, key_of(j));
+            const unsigned m = __reduce_max_sync(FULL, mine);
+            if (lane == 0) wkey[warp] = m;
+            __syncthreads();
+            const unsigned gk = __reduce_max_sync(FULL, lane < nw ? wkey[lane] : 0u);
+            // within 2^-18 of the block's largest, or every live row where FP32 cannot tell (or it is not finite)
+            if (gk > 0x0da24260u && gk < 0x7f000000u) lim = gk - 32u;  // 1e-30
         }
-        auto block_best = [&]() {  // b of every thread -> the block's best in gbest
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Best<T> o;
-                o.score = __shfl_xor_sync(0xffffffffu, b.score, off);
-                o.var = __shfl_xor_sync(0xffffffffu, b.var, off);
-                o.cov = __shfl_xor_sync(0xffffffffu, b.cov, off);
-                o.idx = __shfl_xor_sync(0xffffffffu, b.idx, off);
-                take(o);
+        // the exact scores (FP64: of those rows only), the block's best
+        if (!F64 || __any_sync(FULL, mine >= lim)) {
+            if (!F64 || mine >= lim)
+                for (long long j = j0; j < n; j += jstep) {
+                    const T v = var[j];
+                    if (v >= floor_ && (!F64 || key_of(j) >= lim)) {
+                        const T c = cov[j];
+                        const T s = c * c / v;
+                        if (better(s, j, b.score, b.idx)) b = Best<T>{s, j};
+                    }
+                }
+            __syncwarp();
+            warp_best(b);
+        }
+        if (lane == 0) wbest[warp] = b;
+        __syncthreads();
+        if (warp == 0) {
+            b = lane < nw ? wbest[lane] : Best<T>{NEG, NONE};
+            warp_best(b);
+            int ok = 1;
+            if (gridDim.x > 1) {
+                Best<T>* all = bests + (t & 1) * gridDim.x;
+                if (lane == 0) {
+                    all[blockIdx.x] = b;
+                    ok = grid_wait(count, (unsigned)gridDim.x * (unsigned)(t + 1));
+                }
+                ok = __shfl_sync(FULL, ok, 0);
+                b = Best<T>{NEG, NONE};
+                for (int i = lane; ok && i < (int)gridDim.x; i += 32) {
+                    const Best<T> o{__ldcg(&all[i].score), __ldcg(&all[i].idx)};
+                    if (better(o.score, o.idx, b.score, b.idx)) b = o;
+                }
+                warp_best(b);
             }
-            if (lane == 0) wbest[warp] = b;
-            __syncthreads();
-            if (tid == 0) {
-                for (int w = 1; w < nw; ++w) take(wbest[w]);
-                gbest = b;
+            if (lane == 0) {
+                s_ok = ok;
+                const bool go = ok && b.idx != NONE && b.score > (T)0;
+                s_q = go ? b.idx : NONE;
+                if (go) {
+                    const T vq = __ldcg(&var[b.idx]), cq = __ldcg(&cov[b.idx]);
+                    if constexpr (F64)
+                        s_rs = rsqrt_newton(vq);
+                    else
+                        s_rs = (T)1 / sic_sqrt(vq);
+                    s_ut = cq * s_rs;
+                }
             }
-        };
-        block_best();
-        if (gridDim.x > 1) {
-            Best<T>* mine = bests + (t & 1) * gridDim.x;
-            if (tid == 0) {
-                mine[blockIdx.x] = gbest;
-                s_ok = grid_wait(count, (unsigned)gridDim.x * (unsigned)(t + 1));
-            }
-            __syncthreads();
-            if (!s_ok) {
-                if (tid == 0) record_error(st, SIC_ERR_TIMEOUT, -1);
-                break;
-            }
-            b.score = NEG;
-            b.idx = NONE;
-            for (int i = tid; i < (int)gridDim.x; i += blockDim.x) {
-                Best<T> o;
-                o.score = __ldcg(&mine[i].score);
-                o.var = __ldcg(&mine[i].var);
-                o.cov = __ldcg(&mine[i].cov);
-                o.idx = __ldcg(&mine[i].idx);
-                take(o);
-            }
-            block_best();
         }
         __syncthreads();
-        const long long q = gbest.idx;
-        if (q == NONE || !(gbest.score > (T)0)) break;
-        const T vq = gbest.var, cq = gbest.cov;
+        if (!s_ok) {
+            if (tid == 0) record_error(st, SIC_ERR_TIMEOUT, -1);
+            break;
+        }
+        const long long q = s_q;
+        if (q == NONE) break;
+        const T rs = s_rs, ut = s_ut;
         T qx[3] = {(T)0, (T)0, (T)0};
         for (int d = 0; d < dim; ++d) qx[d] = coord(q, d);
         for (int tau = tid; tau < t; tau += blockDim.x) piv[tau] = __ldcg(&F[(long long)tau * n + q]);
         __syncthreads();
-        T rs;
-        if constexpr (sizeof(T) == 8)
-            rs = rsqrt_newton(vq);
-        else
-            rs = (T)1 / sic_sqrt(vq);
-        const T ut = cq * rs;
+        long long M = 0;
+        int h = 0;
+        if constexpr (F64) fx_factor(rs, e, M, h);
         for (long long j = j0; j < n; j += jstep) {
             const T vj = var[j];
-            if (vj == NEG) continue;
+            if (!(vj != NEG)) continue;
             T d2 = (T)0;
             for (int d = 0; d < dim; ++d) {
                 T df = coord(j, d) - qx[d];
@@ -194,18 +224,39 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
             }
             T num = theta(d2);
             if (j == q) num += kp.nugget;
-            const T* Fj = F + j;
-            int tau = 0;
-            for (; tau + 8 <= t; tau += 8) {  // eight loads in flight, the sum in order
-                T f[8];
+            T u;
+            if constexpr (F64) {
+                long long sum = 0, ux = 0;
+                for (int c0 = 0; c0 < t; c0 += 256) {  // (the cross sums stay in 64 bits over 256 columns)
+                    const int c1 = min(t, c0 + 256);
+                    FxSum a{0, 0};
+                    for (int c = c0; c < c1; c += 8) {  // eight loads in flight
+                        int2 f[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) f[i] = Fj[(long long)(tau + i) * n];
+                        for (int i = 0; i < 8; ++i) f[i] = Fx[(long long)min(c + i, c1 - 1) * n + j];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) num = fma(-f[i], piv[tau + i], num);
+                        for (int i = 0; i < 8; ++i)
+                            if (c + i < c1) a.add(f[i], px[c + i]);
+                    }
+                    sum += a.value();
+                }
+                if (!not_finite(num)) ux = fx_mul(fx_of_positive(num, FXS - 2 * e) - sum, M, h);
+                if (t + 1 < k) Fx[(long long)t * n + j] = fx_split(ux);  // the last column has no reader
+                u = not_finite(num) ? NAN : fx_to_double(ux, e - FXS);   // (never a candidate again)
+            } else {
+                const T* Fj = F + j;
+                int tau = 0;
+                for (; tau + 8 <= t; tau += 8) {  // eight loads in flight, the sum in order
+                    T f[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) f[i] = Fj[(long long)(tau + i) * n];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) num = fma(-f[i], piv[tau + i], num);
+                }
+                for (; tau < t; ++tau) num = fma(-Fj[(long long)tau * n], piv[tau], num);
+                u = num * rs;
+                if (t + 1 < k) F[(long long)t * n + j] = u;  // the last column has no reader
             }
-            for (; tau < t; ++tau) num = fma(-Fj[(long long)tau * n], piv[tau], num);
-            const T u = num * rs;
-            if (t + 1 < k) F[(long long)t * n + j] = u;  // the last column has no reader
             if (j == q) {
                 var[j] = NEG;
             } else {
@@ -226,8 +277,8 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
 }
 
 // Rows per block: the step chain (barrier, reduction, pivot row) costs the same at any block
-// size, so small n spreads over the SMs in blocks of 64 rows; from 152 x 256 rows on two blocks of
-// 256 share an SM and further rows are strided.
+// size, so small n spreads over the SMs in blocks of 64 rows; from 152 x 512 rows on further rows are
+// strided.
 template <typename T>
 sic_status launch_single(sic_handle* h, const double* x_train, int64_t n, const double* x_target,
                          const sic_kernel* kp, int32_t k, int32_t* out_idx, double* out_var, int32_t* out_count,
@@ -237,23 +288,24 @@ sic_status launch_single(sic_handle* h, const double* x_train, int64_t n, const 
     if (smem > 40 * 1024)
         SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long per = (n + h->num_sms - 1) / h->num_sms;
-    const int nt = per <= 64 ? 64 : (per <= 128 ? 128 : 256);
+    const int nt = per <= 64 ? 64 : (per <= 128 ? 128 : (per <= 256 ? 256 : 512));
     int grid = persistent_grid(h, kern, nt, smem, (n + nt - 1) / nt);
-    if (grid > 2 * h->num_sms) grid = 2 * h->num_sms;
+    if (grid > h->num_sms) grid = h->num_sms;
     T* w = (T*)ws;
     int dim = kp->dim;
     long long nn = n;
     KP<T> kpt = make_kp<T>(*kp);
     T fl = (T)sic_floor_of(kp);
+    int e = fx_exponent(kp);
     unsigned* count = scratch_of<T>(w, n, k);
     if (grid > 1) SIC_CUDA_TRY(cudaMemsetAsync(count, 0, 16, s));
     for (;;) {
         if (grid == 1) {
-            kern<<<1, nt, smem, s>>>(x_train, nn, dim, x_target, kpt, fl, k, out_idx, out_var, out_count, w, count,
+            kern<<<1, nt, smem, s>>>(x_train, nn, dim, x_target, kpt, fl, e, k, out_idx, out_var, out_count, w, count,
                                  h->d_status);
             break;
         }
-        void* args[] = {&x_train, &nn, &dim, &x_target, &kpt, &fl, &k, &out_idx, &out_var, &out_count, &w, &count,
+        void* args[] = {&x_train, &nn, &dim, &x_target, &kpt, &fl, &e, &k, &out_idx, &out_var, &out_count, &w, &count,
                         &h->d_status};
         cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3((unsigned)nt), args, smem, s);
         if (e != cudaErrorCooperativeLaunchTooLarge) break;
