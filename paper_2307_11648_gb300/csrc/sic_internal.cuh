@@ -435,6 +435,13 @@ sic_status launch_fx_columns(sic_handle* h, const double* pts, long long n, cons
                              const int32_t* targets, int64_t n_cols, const int64_t* cand_ptr, const int32_t* cand_idx,
                              int max_cand, int k, int32_t* sel_idx, int32_t* sel_count, double* gain, cudaStream_t s);
 
+// one-warp fill of single columns (fill_columns.cu), for k up to 48 picks
+bool fill_columns_applies(int k);
+sic_status launch_fill_columns(sic_handle* h, const double* pts, long long n, const sic_kernel* kp,
+                               const int32_t* sel_idx, const int32_t* sel_count, int k, long long col0,
+                               long long n_cols, const int64_t* col_ptr, long long base, int32_t* row_idx, double* val,
+                               double* logv, cudaStream_t s);
+
 // FP32-mode product of Theta + shift I with up to 8 right-hand sides, summed on the tensor cores
 // (matvec_tc.cu)
 sic_status matvec_tc(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, double shift, const double* x,

