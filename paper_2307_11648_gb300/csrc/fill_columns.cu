@@ -11,8 +11,8 @@
 // FP64, b_i -= F_li x_l, lane = entry; log v = log of the target's pivot, 32 columns' logarithms at a time.
 //
 // The CTA-wide fill (k_fill) spends 5 warps and two barriers per panel on a 33 x 33 block: 65,536 columns of 32 picks
-// 4.19 ms; here 2.3 ms.  Bound: the FP64 pipe (Theta's 8 operations per entry, the pivots' reciprocal
-// square roots, the substitution: about 330 warp instructions per column of 32 picks).
+// 4.19 ms; here 2.2 ms (2.3 with the pivots' reciprocal square roots in FP64).  Bound: the FP64 pipe (Theta's 8
+// operations per entry, the substitution: about 300 warp instructions per column of 32 picks).
 #include <limits.h>
 
 #include "fx.cuh"
@@ -21,34 +21,6 @@ namespace {
 
 constexpr int WARPS = 4;
 constexpr unsigned FULL = 0xffffffffu;
-
-constexpr int FCS = 60;  // 2^FCS stands for 2^e (factor entries) or 2^(2e) (products)
-
-__device__ __forceinline__ int2 fc_split(long long x) {
-    const int h = (int)((x + (1LL << 29)) >> 30);  // |h| < 2^30.5, |l| <= 2^29
-    return make_int2(h, (int)(x - ((long long)h << 30)));
-}
-// sum of products: up to 48 terms keep every word below 2^62.3
-struct FcSum {
-    long long hh, c1, c2;
-    __device__ __forceinline__ void add(int2 a, int2 b) {
-        hh += (long long)a.x * b.x;
-        c1 += (long long)a.x * b.y;
-        c2 += (long long)a.y * b.x;
-    }
-    __device__ __forceinline__ void add2(int4 a, int4 b) {
-        add(make_int2(a.x, a.y), make_int2(b.x, b.y));
-        add(make_int2(a.z, a.w), make_int2(b.z, b.w));
-    }
-    __device__ __forceinline__ long long value() const { return hh + (((c1 >> 2) + (c2 >> 2)) >> 28); }
-};
-// round(n r 2^e) for r = M 2^(...) by fx_factor (shift h there), |n| < 2^61: the top of the 128-bit product
-__device__ __forceinline__ long long fc_mul(long long n, long long M, int h) {
-    const long long a = n << 1, hi = __mul64hi(a, M);  // hi 2^64 + lo = n M 2
-    const unsigned long long lo = (unsigned long long)a * (unsigned long long)M;
-    const int s = h + 3;  // n M 2^-63 2^s, s >= 1
-    return (hi << s) | (long long)(lo >> (64 - s));
-}
 
 // pair p of columns holds rows 2p .. N - 1
 __host__ __device__ __forceinline__ int pair_base(int p, int N) { return p * N - p * (p - 1); }
@@ -65,23 +37,6 @@ __device__ __forceinline__ long long warp_sum(long long v) {
     const int c = (int)(v >> 52);
     return (long long)__reduce_add_sync(FULL, a) + ((long long)__reduce_add_sync(FULL, b) << 26) +
            ((long long)__reduce_add_sync(FULL, c) << 52);
-}
-
-// fx_factor's multiplier M of r ~ d^(-1/2) (off by about 2^-53) to some 60 bits, d = dj 2^(2e - FCS): one Newton step
-// M (1 + E / 2) on the residual E = 1 - d r^2, formed in integers.  An update F_i F_l with the factor rounded to FP64
-// would be off by 2^-52 of itself, 2e-16 of the variance in the first columns, whatever the products' exactness.
-__device__ __forceinline__ long long fc_refine(long long dj, long long M) {
-    const unsigned long long m = (unsigned long long)M;  // [2^61, 2^62)
-    const unsigned long long D = (unsigned long long)dj << (__clzll(dj) - 1);  // [2^62, 2^63)
-    const unsigned long long t = __umul64hi(D << 1, m << 2);  // D m 2^-61
-    const unsigned long long hi = __umul64hi(t, m), lo = t * m;  // D m^2 2^-61 is within 2^-51 of a power of two, 2^K
-    const int K = 64 + 63 - __clzll((long long)(hi + (hi >> 20)));
-    // (2^K - hi:lo) >> 16, below 2^60 in magnitude
-    const unsigned long long rl = 0ULL - lo, rh = (1ULL << (K - 64)) - hi - (lo ? 1ULL : 0ULL);
-    const long long R = (long long)((rh << 48) | (rl >> 16));
-    // M E / 2 = M R 2^(16 - K - 1)
-    const float corr = (float)R * (float)M * __uint_as_float((unsigned)(127 - 58) << 23);
-    return M + (long long)rintf(corr * __uint_as_float((unsigned)(127 + 58 + 15 - K) << 23));
 }
 
 // S sets of 32 picks
@@ -163,8 +118,10 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
         }
         __syncwarp();
         auto theta = [&](int i, int j) -> long long {
-            const double th = matern_d2_fast(kp, fx_dist2(xf, k + 1, dim, i, j, E[0], E[1], E[2]), tab);
-            return not_finite(th) ? LLONG_MIN : fx_of_positive(th, FCS - 2 * e);
+            const double d2 = fx_dist2(xf, k + 1, dim, i, j, E[0], E[1], E[2]);
+            const double th = matern_d2_fast(kp, d2, tab);
+            // (without a nugget coincident points make Theta singular, whatever the factorisation's rounding)
+            return not_finite(th) || (d2 == 0.0 && !(kp.nugget > 0.0)) ? LLONG_MIN : fx_of_positive(th, FCS - 2 * e);
         };
         // ---- Theta of the picks into the triangle (flat), the target's row into the lanes ----
         bool nan_ = false;
@@ -247,11 +204,10 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
                 npd = true;
                 break;
             }
-            const double rs = rsqrt_newton(fx_to_double(dj, 2 * e - FCS));
             long long M;
             int h;
-            fx_factor(rs, e, M, h);
-            M = fc_refine(dj, M);
+            fc_pivot(dj, M, h);
+            const double rs = fx_to_double(M, h - FCS - e);
             __syncwarp();
 #pragma unroll
             for (int s = 0; s < S; ++s) {

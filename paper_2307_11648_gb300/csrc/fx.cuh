@@ -66,6 +66,71 @@ struct FxSum {
     __device__ __forceinline__ long long value() const { return hh + (cr >> 29); }
 };
 
+// ---- 60 bits: factors that are themselves the result (fill_columns.cu) ----
+
+constexpr int FCS = 60;  // 2^FCS stands for 2^e (factor entries) or 2^(2e) (products)
+
+__device__ __forceinline__ int2 fc_split(long long x) {
+    const int h = (int)((x + (1LL << 29)) >> 30);  // |h| < 2^30.5, |l| <= 2^29
+    return make_int2(h, (int)(x - ((long long)h << 30)));
+}
+// sum of products: up to 48 terms of a row keep every word below 2^63 (the entries' squares sum to at most
+// 1.9 2^(2 FCS))
+struct FcSum {
+    long long hh, c1, c2;
+    __device__ __forceinline__ void add(int2 a, int2 b) {
+        hh += (long long)a.x * b.x;
+        c1 += (long long)a.x * b.y;
+        c2 += (long long)a.y * b.x;
+    }
+    __device__ __forceinline__ void add2(int4 a, int4 b) {
+        add(make_int2(a.x, a.y), make_int2(b.x, b.y));
+        add(make_int2(a.z, a.w), make_int2(b.z, b.w));
+    }
+    __device__ __forceinline__ long long value() const { return hh + (((c1 >> 2) + (c2 >> 2)) >> 28); }
+};
+// round(n r 2^e) for r by fc_pivot, |n| < 2^61: the top of the 128-bit product
+__device__ __forceinline__ long long fc_mul(long long n, long long M, int h) {
+    const long long a = n << 1, hi = __mul64hi(a, M);  // hi 2^64 + lo = n M 2
+    const unsigned long long lo = (unsigned long long)a * (unsigned long long)M;
+    const int s = h + 3;  // n M 2^-63 2^s, s >= 1
+    return (hi << s) | (long long)(lo >> (64 - s));
+}
+
+// Multiplier M (60 bits) and shift h of r = d^(-1/2), fc_mul's, for the pivot d = dj 2^(2e - FCS), dj > 0: an FP32
+// reciprocal square root of the normalised pivot, one Newton step in double-float (2^-42), one on the residual
+// 1 - d r^2 formed in integers (2^-61).  No FP64 operation (a chain of them takes 64 cycles each).  A factor rounded to
+// FP64 would put an update F_i F_l off by 2^-52 of itself, 2e-16 of the variance in the first columns, whatever the
+// products' exactness.
+__device__ __forceinline__ void fc_pivot(long long dj, long long& M, int& h) {
+    const int z = __clzll(dj) - 1;
+    const unsigned long long D = (unsigned long long)dj << z;  // [2^62, 2^63)
+    const int odd = z & 1;
+    h = ((z + 1) >> 1) - 3;
+    // X = D 2^-62 (z even) or twice that: [1, 4), in two floats
+    const float xh = (float)(int)(D >> 39) * __uint_as_float((unsigned)(127 - 23 + odd) << 23);
+    const float xl = (float)(int)((D >> 15) & 0xffffffULL) * __uint_as_float((unsigned)(127 - 47 + odd) << 23);
+    const float y = rsqrtf(xh);  // (0.5, 1]
+    const float y2 = __fmul_rn(y, y);
+    const float y2e = __fmaf_rn(y, y, -y2);
+    const float p = __fmul_rn(xh, y2);
+    const float pe = __fmaf_rn(xh, y2, -p);
+    const float e0 = __fmaf_rn(-xl, y2, __fmaf_rn(-xh, y2e, __fsub_rn(__fsub_rn(1.f, p), pe)));
+    const float c = __fmul_rn(0.5f * y, e0);
+    const unsigned yb = __float_as_uint(y);
+    const long long TOP = (1LL << 62) - 1;
+    long long m = ((long long)((yb & 0x7fffffu) | 0x800000u) << (38 + (int)(yb >> 23) - 126)) +
+                  ((long long)__float2int_rn(c * 0x1p50f) << 12);  // r 2^62, off by 2^-42
+    m = m < TOP ? m : TOP;
+    const unsigned long long t = __umul64hi(D << 1, (unsigned long long)m << 2);  // D m 2^-61
+    const unsigned long long hi = __umul64hi(t, (unsigned long long)m), lo = t * (unsigned long long)m;
+    // 2^K (1 - E): K = 125 - odd; R = E 2^71, below 2^31 in magnitude
+    const unsigned long long rl = 0ULL - lo, rh = (1ULL << (61 - odd)) - hi - (lo ? 1ULL : 0ULL);
+    const int R = odd ? (int)((rh << 11) | (rl >> 53)) : (int)((rh << 10) | (rl >> 54));
+    m += __float2int_rn((float)R * y * 0x1p-10f);  // m E / 2
+    M = m < TOP ? m : TOP;
+}
+
 // FP32 value (truncated) of a double scaled by 2^-off, by its bits; 0 below FP32's range and for
 // negative values
 __device__ __forceinline__ float fx_f32(double x, int off) {
