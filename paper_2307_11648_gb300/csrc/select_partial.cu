@@ -22,7 +22,7 @@
 //            from the pivot rows (the targets and picks), the candidate rows apply them.
 // Columns live in physical slots in insertion order; `pk/opos` map the logical (latest-first)
 // order to the pivot row and slot and to the target position (INT_MAX for a pick).  One CTA per
-// group (persistent), L in shared memory, rows spread over the threads of all warps but the first.
+// group (persistent, two size classes), L in shared memory, rows spread over the threads of all warps but the first.
 //
 // A step walks each candidate row's columns twice: the left-looking product over the first p, then
 // one walk that applies the rotations and takes the next step's score as it goes.  The first warp
@@ -31,14 +31,16 @@
 // named barriers; the target block is factored once, before the candidates' rows, which need no barrier then.
 // Bound: that chain, about 200 cycles per column in one warp's instructions (a chain without the
 // shuffle took as long), with the walk of two warps per scheduler behind it.  N = 2^16, 256 candidates, k = 64 (2,811
-// groups): 16.1 ms with score, columns and rotations one after the other, 9.0 ms now.
+// groups): 16.1 ms with score, columns and rotations one after the other, 9.0 ms with one CTA per SM, 7.1 ms now that
+// the smaller groups run two to an SM.
 #include <limits.h>
 
 #include "sic_internal.cuh"
 
 namespace {
 
-constexpr int PT_NT = 512;
+constexpr int PT_NT = 512;     // one CTA per SM
+constexpr int PT_NT_2 = 288;   // groups whose state fits an SM twice: a row per thread up to 256 candidates
 
 __device__ __forceinline__ float pt_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double pt_div(double a, double b) { return a / b; }
@@ -80,14 +82,18 @@ struct PtLayout {
     }
 };
 
+constexpr int PT_STATIC = 4096;  // static shared memory and what the system keeps of a CTA's share, at most
+constexpr int PT_MIN_CLASS = 4;
 constexpr int PT_CHUNK = 16;  // columns handed over per named barrier
 constexpr int PT_EL = 6;      // element rows per lane of the first warp: 32 * PT_EL = 192 columns
 
+template <int NT>
 __device__ __forceinline__ void pt_arrive(int id) {
-    asm volatile("barrier.arrive %0, %1;" ::"r"(id), "n"(PT_NT) : "memory");
+    asm volatile("barrier.arrive %0, %1;" ::"r"(id), "n"(NT) : "memory");
 }
+template <int NT>
 __device__ __forceinline__ void pt_sync(int id) {
-    asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(PT_NT) : "memory");
+    asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(NT) : "memory");
 }
 
 // The least (key, index) over the warp, key INFINITY where there is none
@@ -114,7 +120,7 @@ __device__ __forceinline__ void pt_warp_min(double& key, int& idx) {
 // (block 0) and of j0 + 32 i + lane (block i < NA, to which the rotations are applied), with each row's downdate
 // value x, its offset in Lm, its entry L in the current column and its pivot entry lee.  pc: (row << 8 | slot) of
 // the columns from the first rotation on.  Rotations go to rc / rsn / ric and are handed over per chunk.
-template <int NA, typename T>
+template <int NT, int NA, typename T>
 __device__ __forceinline__ bool pt_chain(T* __restrict__ Lm, const int* __restrict__ pc, T* __restrict__ rc,
                                          T* __restrict__ rsn, T* __restrict__ ric, int j0, int ne, int lane,
                                          const int (&row)[PT_EL], const T (&lee)[PT_EL], T (&x)[PT_EL], T (&L)[PT_EL]) {
@@ -153,16 +159,17 @@ __device__ __forceinline__ bool pt_chain(T* __restrict__ Lm, const int* __restri
         if (lane == cc) Lm[row[0] + s] = rr;
         s = s1;
         s1 = s2;
-        if ((j & (PT_CHUNK - 1)) == PT_CHUNK - 1 || j == ne - 1) pt_arrive(1 + j / PT_CHUNK);
+        if ((j & (PT_CHUNK - 1)) == PT_CHUNK - 1 || j == ne - 1) pt_arrive<NT>(1 + j / PT_CHUNK);
     }
     return ok;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
+// groups of m_lo .. m_hi members
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, NT == PT_NT ? 1 : 2) k_select_partial(
     const double* __restrict__ pts, long long n, int dim, KP<T> kp, T floor_, const long long* __restrict__ grp_ptr,
     const long long* __restrict__ members, long long n_grp, const long long* __restrict__ cand_ptr,
-    const int32_t* __restrict__ cand_idx, int max_cand, int max_m, int k, int32_t* __restrict__ sel_idx,
+    const int32_t* __restrict__ cand_idx, int max_cand, int max_m, int m_lo, int m_hi, int k, int32_t* __restrict__ sel_idx,
     int32_t* __restrict__ sel_count, double* __restrict__ gain, PtLayout Lay, DevStatus* st) {
     extern __shared__ __align__(16) unsigned char smraw[];
     T* Lm = reinterpret_cast<T*>(smraw);              // [R][P]
@@ -176,19 +183,26 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
     int* opos = pk + 2 * Lay.W;                       // 2 x [W] target position of column c (INT_MAX: a pick)
     __shared__ T s_rs, s_d;
     __shared__ int s_fail;
-    __shared__ T wkey[PT_NT / 32];
-    __shared__ int widx[PT_NT / 32];
+    __shared__ T wkey[NT / 32];
+    __shared__ int widx[NT / 32];
     __shared__ double gprod[128];
     __shared__ int gcnd[128];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int WT = PT_NT - 32;  // threads of the walking warps
+    constexpr int WT = NT - 32;  // threads of the walking warps
     constexpr unsigned FULL = 0xffffffffu;
     const int wt = tid - 32;
     const int PP = Lay.P, RR = Lay.R;
     const T diag = kp.s2 + kp.nugget;
     const T INF = (T)INFINITY;
 
-    for (long long g = blockIdx.x; g < n_grp; g += gridDim.x) {
+    __shared__ ClassDeal<NT> deal;
+    // this launch's groups (the invalid ones are the first class's to report)
+    auto in_class = [&](long long g) {
+        const long long m = grp_ptr[g + 1] - grp_ptr[g];
+        return m < 1 || m > max_m ? m_lo == 1 : m >= m_lo && m <= m_hi;
+    };
+    deal.start();
+    for (long long g = deal.next(n_grp, in_class); g >= 0; g = deal.next(n_grp, in_class)) {
         const long long a0 = grp_ptr[g];
         const int m = (int)(grp_ptr[g + 1] - a0);
         const long long b0 = cand_ptr[g];
@@ -198,7 +212,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                 record_error(st, SIC_ERR_INVALID, g);
                 sel_count[g] = 0;
             }
-            for (int q = tid; q < k; q += PT_NT) sel_idx[g * k + q] = -1;
+            for (int q = tid; q < k; q += NT) sel_idx[g * k + q] = -1;
             continue;
         }
         const int R = C + m;
@@ -209,7 +223,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
             if (first >= 0 && first < n)
                 for (int d = 0; d < dim; ++d) org[d] = pts[first * dim + d];
         __syncthreads();
-        for (int r = tid; r < R; r += PT_NT) {
+        for (int r = tid; r < R; r += NT) {
             long long p = r < C ? (long long)cand_idx[b0 + r] : members[a0 + (r - C)];
             const bool bad = p < 0 || p >= n || (r < C && p <= first) ||
                              (r > C && p <= members[a0 + (r - C) - 1]);
@@ -227,7 +241,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                 record_error(st, SIC_ERR_INVALID, g);
                 sel_count[g] = 0;
             }
-            for (int q = tid; q < k; q += PT_NT) sel_idx[g * k + q] = -1;
+            for (int q = tid; q < k; q += NT) sel_idx[g * k + q] = -1;
             __syncthreads();
             continue;
         }
@@ -301,7 +315,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                 }
             }
             __syncthreads();
-            for (int r = C + tid; r < R; r += PT_NT) pos[r] = ~pos[r];
+            for (int r = C + tid; r < R; r += NT) pos[r] = ~pos[r];
             // (visible after the first step's barriers)
         }
         int ncol = m, t = 0;
@@ -312,8 +326,8 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                 widx[warp] = bi;
             }
             __syncthreads();
-            T gk = lane < PT_NT / 32 ? wkey[lane] : INF;
-            int q = lane < PT_NT / 32 ? widx[lane] : INT_MAX;
+            T gk = lane < NT / 32 ? wkey[lane] : INF;
+            int q = lane < NT / 32 ? widx[lane] : INT_MAX;
             pt_warp_min(gk, q);
             if (q == INT_MAX) break;
             const int pq = pos[q];
@@ -393,10 +407,10 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                     const int na = (ne - j0 + 31) >> 5;
                     const int* pj = pc + p;
                     T *c_ = rc + p, *s_ = rsn + p, *i_ = ric + p;
-                    const bool g1 = na == 1   ? pt_chain<1>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
-                                    : na == 2 ? pt_chain<2>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
-                                    : na == 3 ? pt_chain<3>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
-                                              : pt_chain<PT_EL>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L);
+                    const bool g1 = na == 1   ? pt_chain<NT, 1>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                    : na == 2 ? pt_chain<NT, 2>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                    : na == 3 ? pt_chain<NT, 3>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L)
+                                              : pt_chain<NT, PT_EL>(Lm, pj, c_, s_, i_, j0, ne, lane, row, lee, x, L);
                     good = good && g1;
 #pragma unroll
                     for (int i = 0; i + 1 < PT_EL; ++i) {  // the next block of pivot rows
@@ -446,7 +460,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
                     for (int j0 = 0; j0 < ne; j0 += PT_CHUNK) {
                         if (wait) {
                             __syncwarp();
-                            pt_sync(1 + j0 / PT_CHUNK);
+                            pt_sync<NT>(1 + j0 / PT_CHUNK);
                         }
                         if (live) {
                             const int c1 = p + min(j0 + PT_CHUNK, ne);
@@ -478,11 +492,11 @@ __global__ void __launch_bounds__(PT_NT, 1) k_select_partial(
         }
         if (!ok && tid == 0) record_error(st, SIC_ERR_NOT_PD, g);
         if (tid == 0) sel_count[g] = t;
-        for (int q = t + tid; q < k; q += PT_NT) sel_idx[g * k + q] = -1;
+        for (int q = t + tid; q < k; q += NT) sel_idx[g * k + q] = -1;
         if (gain) {
             __syncthreads();
             // decrease of the objective per nonzero (the targets the pick conditions)
-            for (int q = tid; q < t; q += PT_NT) gain[g * k + q] = -log(gprod[q]) / (gcnd[q] > 0 ? gcnd[q] : 1);
+            for (int q = tid; q < t; q += NT) gain[g * k + q] = -log(gprod[q]) / (gcnd[q] > 0 ? gcnd[q] : 1);
         }
         __syncthreads();
     }
@@ -542,32 +556,45 @@ extern "C" sic_status sic_select_partial(sic_handle* h, const double* pts, int64
     if (k > 128 || max_m > 64 || n > INT_MAX) return SIC_ERR_UNSUPPORTED;
     if (n_grp == 0) return SIC_OK;
     if (max_cand > 0 && !cand_idx) return SIC_ERR_INVALID;
-    PtLayout L;
-    L.R = max_cand + max_m;
-    L.W = max_m + k;
-    L.P = L.W | 1;
     const size_t tsz = prec == SIC_FP64 ? sizeof(double) : sizeof(float);
-    if (L.limit_bytes(tsz) > 227 * 1024 - 4096) return SIC_ERR_UNSUPPORTED;
-    const size_t smem = L.bytes(tsz);
+    auto layout = [&](int m) {
+        PtLayout L;
+        L.R = max_cand + m;
+        L.W = m + k;
+        L.P = L.W | 1;
+        return L;
+    };
+    if (layout(max_m).limit_bytes(tsz) > 227 * 1024 - 4096) return SIC_ERR_UNSUPPORTED;
+    if (prec != SIC_FP64 && prec != SIC_FP32_MIXED) return SIC_ERR_INVALID;
+    if (n_grp > INT_MAX) return SIC_ERR_UNSUPPORTED;
     SIC_CUDA_TRY(cudaSetDevice(h->device));
     cudaStream_t s = (cudaStream_t)stream;
-    const long long* gp = (const long long*)grp_ptr;
-    const long long* mb = (const long long*)members;
-    const long long* cp = (const long long*)cand_ptr;
-    if (prec == SIC_FP64) {
-        auto kern = k_select_partial<double>;
-        SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        const int grid = persistent_grid(h, kern, PT_NT, smem, n_grp);
-        kern<<<grid, PT_NT, smem, s>>>(pts, n, kp->dim, make_kp<double>(*kp), sic_floor_of(kp), gp, mb, n_grp, cp,
-                                       cand_idx, max_cand, max_m, k, sel_idx, sel_count, gain, L, h->d_status);
-    } else if (prec == SIC_FP32_MIXED) {
-        auto kern = k_select_partial<float>;
-        SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        const int grid = persistent_grid(h, kern, PT_NT, smem, n_grp);
-        kern<<<grid, PT_NT, smem, s>>>(pts, n, kp->dim, make_kp<float>(*kp), (float)sic_floor_of(kp), gp, mb, n_grp,
-                                       cp, cand_idx, max_cand, max_m, k, sel_idx, sel_count, gain, L, h->d_status);
-    } else {
-        return SIC_ERR_INVALID;
+    // Two size classes: a step's time is its chain of dependent operations, so two groups on an SM take little longer than
+    // one.  Up to `two` members the state fits twice (256 candidates, k = 64 in FP32: 25 members).  N = 2^16, 2,811
+    // groups: 9.0 ms as one class, 7.1 as two.
+    int two = max_m;
+    while (two > 0 && layout(two).bytes(tsz) > 227 * 1024 / 2 - PT_STATIC) --two;
+    if (two < PT_MIN_CLASS && two < max_m) two = 0;  // a few small groups are not worth a launch
+    for (int c = 0; c < 2; ++c) {
+        const int lo = c == 0 ? 1 : two + 1, hi = c == 0 ? two : max_m;
+        if (lo > hi) continue;
+        const PtLayout L = layout(hi);
+        const size_t smem = L.bytes(tsz);
+        const int nt = c == 0 ? PT_NT_2 : PT_NT;
+        auto launch = [&](auto kern, auto kpt, auto floor_) -> sic_status {
+            SIC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            const int grid = persistent_grid(h, kern, nt, smem, n_grp);
+            kern<<<grid, nt, smem, s>>>(pts, n, kp->dim, kpt, floor_, (const long long*)grp_ptr,
+                                        (const long long*)members, n_grp, (const long long*)cand_ptr, cand_idx, max_cand,
+                                        max_m, lo, hi, k, sel_idx, sel_count, gain, L, h->d_status);
+            return SIC_OK;
+        };
+        const double fl = sic_floor_of(kp);
+        const sic_status e =
+            prec == SIC_FP64
+                ? launch(c == 0 ? k_select_partial<double, PT_NT_2> : k_select_partial<double, PT_NT>, make_kp<double>(*kp), fl)
+                : launch(c == 0 ? k_select_partial<float, PT_NT_2> : k_select_partial<float, PT_NT>, make_kp<float>(*kp), (float)fl);
+        if (e != SIC_OK) return e;
     }
     SIC_CUDA_TRY(cudaGetLastError());
     return SIC_OK;
