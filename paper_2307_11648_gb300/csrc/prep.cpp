@@ -33,22 +33,23 @@ int threads_of(int n_threads) {
 
 template <typename F>
 void parallel_for(int64_t count, int n_threads, int64_t chunk, F f) {
-    int nt = threads_of(n_threads);
-    if (nt <= 1 || count <= chunk) {
+    const int nt = (int)std::min<int64_t>(threads_of(n_threads), (count + chunk - 1) / chunk);
+    if (nt <= 1) {
         for (int64_t i = 0; i < count; ++i) f(i);
         return;
     }
     std::atomic<int64_t> next(0);
+    auto work = [&]() {
+        for (;;) {
+            int64_t b = next.fetch_add(chunk);
+            if (b >= count) break;
+            int64_t e = std::min(count, b + chunk);
+            for (int64_t i = b; i < e; ++i) f(i);
+        }
+    };
     std::vector<std::thread> pool;
-    for (int t = 0; t < nt; ++t)
-        pool.emplace_back([&]() {
-            for (;;) {
-                int64_t b = next.fetch_add(chunk);
-                if (b >= count) break;
-                int64_t e = std::min(count, b + chunk);
-                for (int64_t i = b; i < e; ++i) f(i);
-            }
-        });
+    for (int t = 1; t < nt; ++t) pool.emplace_back(work);
+    work();  // the calling thread takes its share
     for (auto& th : pool) th.join();
 }
 
@@ -160,6 +161,14 @@ struct SuffixGrids {
             size.push_back(s);
             if (s == n) break;
         }
+        fill(pts, n, dim, n_threads);
+    }
+    // the one level that queries with `first` >= n - s need
+    void build_one(const double* pts, int64_t n, int dim, int64_t s) {
+        size.push_back(std::min(s, n));
+        fill(pts, n, dim, 1);
+    }
+    void fill(const double* pts, int64_t n, int dim, int n_threads) {
         grid.resize(size.size());
         parallel_for((int64_t)size.size(), n_threads, 1, [&](int64_t l) {
             std::vector<int64_t> rows(size[l]);
@@ -225,14 +234,17 @@ int32_t knn_query(const double* pts, int64_t n, int dim, const SuffixGrids& sg, 
                 }
         if (covers_all) break;
         if ((int64_t)buf.size() >= C) {
-            double reach = ring * hmin;
-            std::nth_element(buf.begin(), buf.begin() + (C - 1), buf.end());
-            if (buf[C - 1].key <= reach * reach) break;
+            // the C-th nearest lies within reach exactly if C keys do
+            const double reach = ring * hmin, reach2 = reach * reach;
+            int64_t within = 0;
+            for (const KeyPos& e : buf) within += e.key <= reach2;
+            if (within >= C) break;
         }
         if ((int64_t)buf.size() >= avail) break;
     }
     int32_t take = (int32_t)std::min<int64_t>(C, (int64_t)buf.size());
-    std::partial_sort(buf.begin(), buf.begin() + take, buf.end());
+    if (take < (int64_t)buf.size()) std::nth_element(buf.begin(), buf.begin() + take, buf.end());
+    std::sort(buf.begin(), buf.begin() + take);
     for (int32_t t = 0; t < take; ++t) out[t] = (int32_t)buf[t].pos;
     return take;
 }
@@ -326,9 +338,10 @@ extern "C" sic_status sic_prep_candidates_targets(const double* pts, int64_t n, 
     cand_ptr[0] = 0;
     if (n_targets == 0) return SIC_OK;
     SuffixGrids sg;
-    sg.build(pts, n, dim, std::max<int64_t>(256, n - n_targets), n_threads);
+    sg.build_one(pts, n, dim, std::max<int64_t>(256, n - n_targets));  // every query takes the training points
     std::vector<int32_t> cnt(n_targets, 0);
-    parallel_for(n_targets, n_threads, 256, [&](int64_t i) {
+    // 8 queries (some 100 us) outweigh a thread's start
+    parallel_for(n_targets, n_threads, 8, [&](int64_t i) {
         thread_local std::vector<KeyPos> buf;
         int64_t t = i;
         cnt[i] = knn_query(pts, n, dim, sg, &t, 1, n_targets, n_cand, cand_idx + i * (int64_t)n_cand, buf);
