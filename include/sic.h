@@ -62,7 +62,8 @@ typedef struct {
 
 /* Arithmetic of the selection kernels.  The fill and the KL sum are always FP64.
  * SIC_FP64 evaluates the kernel with a table-driven exp and Newton square roots (about
- * 2 ulp); SIC_FP32_MIXED uses the hardware's approximate reciprocal, reciprocal square
+ * 2 ulp) and holds factor entries in 58-bit fixed point, their products summed exactly;
+ * SIC_FP32_MIXED uses the hardware's approximate reciprocal, reciprocal square
  * root and exp (a few ulp of FP32), far below the FP32 state's own resolution. */
 typedef enum {
     SIC_FP64 = 0,        /* scores, partial factor and downdates in FP64 */
@@ -387,7 +388,7 @@ sic_status sic_tune_build_factor(sic_handle* h, const double* pts, int64_t n, co
  * has no counterpart): the same arguments and results as sic_select_aggregated, but it runs
  * the selection once per launch plan that gives the same picks -- threads per CTA (128 or 256
  * for the register-resident FP32 kernel with at most 128 candidates; 256 or 512 for the
- * generic kernel) and the generic kernel's state in shared memory (when it fits) or in the
+ * generic FP32 kernel; 128, 256, 512 or 1024 in FP64) and the generic kernel's state in shared memory (when it fits) or in the
  * workspace (when `ws` holds it) --, each three times with CUDA events on `stream`
  * (synchronising it; not for stream capture), keeps the fastest in the handle for (k, prec,
  * max_cand, max_m) (op 3 of the table: value = 2 * threads + 1 if in shared memory, or the
@@ -463,8 +464,9 @@ sic_status sic_apply_factor(sic_handle* h, int64_t n, const int64_t* col_ptr, co
 
 /* y = (Theta + shift I) x without forming Theta (O(n^2) kernel evaluations), x, y
  * n x nrhs row-major FP64, 1 <= nrhs <= 8.  SIC_FP32_MIXED evaluates the kernel entries
- * in FP32 (a fixed symmetric rounding of Theta) and sums the products with double-FP32
- * compensated arithmetic (x split into two FP32 parts), tiles added in FP64; SIC_FP64
+ * in FP32 (a fixed symmetric rounding of Theta) and sums the products exactly from BF16
+ * digits of the entries and of x (one or two right-hand sides at n >= 12288: with double-FP32
+ * compensated arithmetic, x split into two FP32 parts, tiles added in FP64); SIC_FP64
  * is FP64 throughout (reference for small n).  x and y must not overlap. */
 sic_status sic_matern_matvec(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp, double shift,
                              sic_precision prec, const double* x, double* y, int32_t nrhs, void* stream);
