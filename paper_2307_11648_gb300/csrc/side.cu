@@ -120,6 +120,166 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
     }
 }
 
+// ---- few units ----
+//
+// Both factorisations of a unit at once, right-looking over all 256 threads, two barriers per pivot.  It takes more
+// work than the panels, but a unit's chain is shorter and there is one launch of one class: while there are
+// few units per SM, that is the time.  N = 5,641 (262 units, k = 55) 260 us against 451 by the panels, 19,528 (857) 589
+// against 636; 48,858 (1,996) 1,400 against 1,225, 65,536 (2,796) 1,980 against 1,750.
+constexpr int FLAT_NT = 256;
+
+struct FlatLayout {
+    int nmax, k;
+    int dec;  // 1: the packed-triangle decode table follows the doubles (when it fits)
+    __host__ __device__ int tab() const { return 0; }
+    __host__ __device__ int A() const { return EXP_TAB; }
+    __host__ __device__ int B() const { return A() + nmax * (nmax + 1) / 2; }
+    __host__ __device__ int xyz() const { return B() + k * (k + 1) / 2; }
+    __host__ __device__ int clA() const { return xyz() + 3 * nmax; }
+    __host__ __device__ int clB() const { return clA() + nmax; }
+    __host__ __device__ int rdA() const { return clB() + k; }
+    __host__ __device__ int rdB() const { return rdA() + nmax; }
+    __host__ __device__ int size() const { return rdB() + k; }  // doubles
+    // then the decode table of the packed triangle: entry e -> (row << 8) | column
+    __host__ __device__ int tri() const { return nmax * (nmax + 1) / 2; }
+    __host__ __device__ size_t bytes() const {
+        return sizeof(double) * (size_t)size() + (dec ? sizeof(uint16_t) * (size_t)tri() : 0);
+    }
+};
+
+__global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict__ pts, long long n, int dim,
+                                                  KP<double> kp, const long long* __restrict__ grp_ptr,
+                                                  const int32_t* __restrict__ targets, long long n_units,
+                                                  const int32_t* __restrict__ sel_idx,
+                                                  const int32_t* __restrict__ sel_count, int k, int max_m,
+                                                  FlatLayout L, double* __restrict__ pvar,
+                                                  double* __restrict__ pvar_p, double* __restrict__ gain,
+                                                  DevStatus* st) {
+    extern __shared__ double sm[];
+    double* tab = sm + L.tab();
+    double* A = sm + L.A();
+    double* B = sm + L.B();
+    double* xyz = sm + L.xyz();
+    double* clA = sm + L.clA();
+    double* clB = sm + L.clB();
+    double* rdA = sm + L.rdA();
+    double* rdB = sm + L.rdB();
+    uint16_t* dec = reinterpret_cast<uint16_t*>(sm + L.size());  // packed-triangle decode table
+    __shared__ int s_bad;  // 1: invalid unit or pick, 2: a pivot not positive
+    const int tid = threadIdx.x, NMAX = L.nmax;
+    const double diag = kp.s2 + kp.nugget;
+    const double NaN = __longlong_as_double(0x7ff8000000000000LL);
+    exp_table_fill(tab, kp.s2);
+    if (L.dec)
+        for (int e = threadIdx.x; e < L.tri(); e += blockDim.x) {
+            const int r = pk_row(e);
+            dec[e] = (uint16_t)((r << 8) | (e - r * (r + 1) / 2));
+        }
+    // row and column of packed-triangle element e: from the table, else by the square root
+    auto decode = [&](int e, int& r, int& c) {
+        if (L.dec) {
+            const unsigned v = dec[e];
+            r = (int)(v >> 8);
+            c = (int)(v & 255u);
+        } else {
+            r = pk_row(e);
+            c = e - r * (r + 1) / 2;
+        }
+    };
+
+    for (long long u = blockIdx.x; u < n_units; u += gridDim.x) {
+        long long p0;
+        int m;
+        if (grp_ptr) {
+            p0 = grp_ptr[u];
+            m = (int)(grp_ptr[u + 1] - p0);
+        } else {
+            p0 = targets ? (long long)targets[u] : u;
+            m = 1;
+        }
+        const int cnt_raw = sel_count[u];
+        const bool bad_unit = m < 1 || m > max_m || p0 < 0 || p0 + m > n || cnt_raw < 0 || cnt_raw > k;
+        const int cnt = bad_unit ? 0 : cnt_raw;
+        const int nn = m + cnt;
+        if (tid == 0) s_bad = bad_unit ? 1 : 0;
+        __syncthreads();
+        for (int i = tid; i < (bad_unit ? 0 : nn); i += FLAT_NT) {
+            long long p = i < m ? p0 + i : (long long)sel_idx[u * k + (i - m)];
+            if (p < 0 || p >= n) {
+                s_bad = 1;
+                p = p0;
+            }
+#pragma unroll
+            for (int d = 0; d < 3; ++d) xyz[d * NMAX + i] = (d < dim) ? pts[p * dim + d] : 0.0;
+        }
+        __syncthreads();
+        if (!s_bad && cnt > 0) {
+            // Theta over [P; S] (packed lower) and a copy of its S block
+            const int tri = nn * (nn + 1) / 2;
+            for (int e = tid; e < tri; e += FLAT_NT) {
+                int a, b;
+                decode(e, a, b);
+                double v = diag;
+                if (a != b) {
+                    const double dx = xyz[a] - xyz[b], dy = xyz[NMAX + a] - xyz[NMAX + b],
+                                 dz = xyz[2 * NMAX + a] - xyz[2 * NMAX + b];
+                    v = matern_d2_fast(kp, fma(dz, dz, fma(dy, dy, dx * dx)), tab);
+                }
+                A[e] = v;
+                if (b >= m) B[pk(a - m, b - m)] = v;
+            }
+            if (tid == 0) {
+                rdA[0] = 1.0 / diag;
+                rdB[0] = 1.0 / diag;
+            }
+            __syncthreads();
+            for (int j = 0; j < nn; ++j) {
+                const bool jb = j < cnt;
+                const double ra = rdA[j], rb = jb ? rdB[j] : 0.0;
+                for (int a = j + 1 + tid; a < nn; a += FLAT_NT) clA[a] = A[pk(a, j)] * ra;
+                if (jb)
+                    for (int a = j + 1 + tid; a < cnt; a += FLAT_NT) clB[a] = B[pk(a, j)] * rb;
+                __syncthreads();
+                const int TA = nn - j - 1, TB = jb ? cnt - j - 1 : 0;
+                const int eA = TA * (TA + 1) / 2, eB = TB * (TB + 1) / 2;
+                for (int e = tid; e < eA + eB; e += FLAT_NT) {
+                    const bool inA = e < eA;
+                    const int f = inA ? e : e - eA;
+                    int r, c;
+                    decode(f, r, c);
+                    const int a = j + 1 + r, b = j + 1 + c;
+                    double* M = inA ? A : B;
+                    const double* cl = inA ? clA : clB;
+                    const double v = fma(-cl[a], M[pk(b, j)], M[pk(a, b)]);
+                    M[pk(a, b)] = v;
+                    if (r == 0) {  // the next pivot (a = b = j + 1)
+                        if (!(v > 0.0)) s_bad = 2;
+                        (inA ? rdA : rdB)[j + 1] = 1.0 / v;
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        const int bad = s_bad;
+        if (bad && tid == 0) record_error(st, bad == 2 ? SIC_ERR_NOT_PD : SIC_ERR_INVALID, u);
+        const int nout = bad_unit ? ((cnt_raw > 0 && cnt_raw <= k) ? cnt_raw : 0) : cnt;
+        for (int t = tid; t < nout; t += FLAT_NT) {
+            double v1 = NaN, v2 = NaN, g = NaN;
+            if (!bad) {
+                v1 = B[pk(t, t)];
+                v2 = A[pk(m + t, m + t)];
+                g = log(v1 / v2) / m;
+            }
+            if (pvar) pvar[u * k + t] = v1;
+            if (pvar_p) pvar_p[u * k + t] = v2;
+            if (gain) gain[u * k + t] = g;
+        }
+        __syncthreads();
+    }
+}
+
+constexpr int FLAT_UNITS_PER_SM = 7;
+
 }  // namespace
 
 extern "C" sic_status sic_side_state_fp64(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp,
@@ -134,6 +294,22 @@ extern "C" sic_status sic_side_state_fp64(sic_handle* h, const double* pts, int6
     if (!sel_idx || !sel_count) return SIC_ERR_INVALID;
     if (n_units > 0x7fffffffLL) return SIC_ERR_UNSUPPORTED;
     SIC_CUDA_TRY(cudaSetDevice(h->device));
+    FlatLayout F;
+    F.nmax = max_m + k;
+    F.k = k;
+    F.dec = 1;
+    if (F.bytes() > 227 * 1024 - 1024) F.dec = 0;
+    if (n_units <= (int64_t)FLAT_UNITS_PER_SM * h->num_sms && F.bytes() <= 227 * 1024 - 1024) {
+        const size_t smem = F.bytes();
+        SIC_CUDA_TRY(cudaFuncSetAttribute(k_side_flat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const int grid = persistent_grid(h, k_side_flat, FLAT_NT, smem, n_units);
+        k_side_flat<<<grid, FLAT_NT, smem, (cudaStream_t)stream>>>(pts, n, kp->dim, make_kp<double>(*kp),
+                                                                   (const long long*)grp_ptr, targets, n_units, sel_idx,
+                                                                   sel_count, k, max_m, F, pvar, pvar_p, gain,
+                                                                   h->d_status);
+        SIC_CUDA_TRY(cudaGetLastError());
+        return SIC_OK;
+    }
     // two size classes, as in the fill: the shared memory (and so the CTAs per SM) of each launch fits its own
     // largest unit
     const int split = max_m < SIDE_M_SPLIT ? max_m : SIDE_M_SPLIT;
