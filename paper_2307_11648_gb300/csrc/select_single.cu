@@ -11,6 +11,10 @@
 // appends u_j = (Theta_{jq} - F_j . F_q)/sqrt(var_q) and downdates var and cov
 // (eq. cond_select).  out_var traces the target's conditional variance.
 //
+// Between two barriers no block reads what another one writes: a block publishes its best row's variance and
+// covariance with the score (var[q] and cov[q] themselves change in the same step), in slots of two alternating
+// parities, and the pivot's row has only columns of earlier steps.
+//
 // In FP64 the factor is held in fixed point (fx.cuh, select_fx.cu): exact integer dot products instead of FP64
 // multiply-adds, and scores in FP32 first, the FP64 quotient only where a row is within 2^-18 of its block's largest.
 //
@@ -32,10 +36,10 @@ __device__ __forceinline__ bool better(T s, long long i, T bs, long long bi) {
     return s > bs || (s == bs && i < bi);
 }
 
-// a block's best candidate of a step
+// a block's best candidate of a step, with what the others need of its state
 template <typename T>
 struct Best {
-    T score;
+    T score, var, cov;
     long long idx;
 };
 
@@ -131,16 +135,23 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
         return __float_as_uint(__fdividef(c * c, fx_f32((double)v, 2 * e))) + 1u;
     };
     auto warp_best = [&](Best<T>& b) {
+        T s = b.score;
+        long long i = b.idx;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            const T os = __shfl_xor_sync(FULL, b.score, off);
-            const long long oi = __shfl_xor_sync(FULL, b.idx, off);
-            if (better(os, oi, b.score, b.idx)) b = Best<T>{os, oi};
+            const T os = __shfl_xor_sync(FULL, s, off);
+            const long long oi = __shfl_xor_sync(FULL, i, off);
+            if (better(os, oi, s, i)) {
+                s = os;
+                i = oi;
+            }
         }
+        const int src = __ffs(__ballot_sync(FULL, b.idx == i)) - 1;
+        b = Best<T>{s, __shfl_sync(FULL, b.var, src), __shfl_sync(FULL, b.cov, src), i};
     };
     int t = 0;
     for (; t < k; ++t) {
-        Best<T> b{NEG, NONE};
+        Best<T> b{NEG, (T)0, (T)0, NONE};
         unsigned lim = 1u, mine = 0u;
         if constexpr (F64) {
             for (long long j = j0; j < n; j += jstep) mine = max(mine, key_of(j));
@@ -159,7 +170,7 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
                     if (v >= floor_ && (!F64 || key_of(j) >= lim)) {
                         const T c = cov[j];
                         const T s = c * c / v;
-                        if (better(s, j, b.score, b.idx)) b = Best<T>{s, j};
+                        if (better(s, j, b.score, b.idx)) b = Best<T>{s, v, c, j};
                     }
                 }
             __syncwarp();
@@ -168,7 +179,7 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
         if (lane == 0) wbest[warp] = b;
         __syncthreads();
         if (warp == 0) {
-            b = lane < nw ? wbest[lane] : Best<T>{NEG, NONE};
+            b = lane < nw ? wbest[lane] : Best<T>{NEG, (T)0, (T)0, NONE};
             warp_best(b);
             int ok = 1;
             if (gridDim.x > 1) {
@@ -178,9 +189,9 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
                     ok = grid_wait(count, (unsigned)gridDim.x * (unsigned)(t + 1));
                 }
                 ok = __shfl_sync(FULL, ok, 0);
-                b = Best<T>{NEG, NONE};
+                b = Best<T>{NEG, (T)0, (T)0, NONE};
                 for (int i = lane; ok && i < (int)gridDim.x; i += 32) {
-                    const Best<T> o{__ldcg(&all[i].score), __ldcg(&all[i].idx)};
+                    const Best<T> o{__ldcg(&all[i].score), __ldcg(&all[i].var), __ldcg(&all[i].cov), __ldcg(&all[i].idx)};
                     if (better(o.score, o.idx, b.score, b.idx)) b = o;
                 }
                 warp_best(b);
@@ -190,12 +201,11 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
                 const bool go = ok && b.idx != NONE && b.score > (T)0;
                 s_q = go ? b.idx : NONE;
                 if (go) {
-                    const T vq = __ldcg(&var[b.idx]), cq = __ldcg(&cov[b.idx]);
                     if constexpr (F64)
-                        s_rs = rsqrt_newton(vq);
+                        s_rs = rsqrt_newton(b.var);
                     else
-                        s_rs = (T)1 / sic_sqrt(vq);
-                    s_ut = cq * s_rs;
+                        s_rs = (T)1 / sic_sqrt(b.var);
+                    s_ut = b.cov * s_rs;
                 }
             }
         }
