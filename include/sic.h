@@ -202,7 +202,8 @@ sic_status sic_select_columns(sic_handle* h, const double* pts, int64_t n, const
  * targets (eq. greedy_mult).  sel_idx[n_grp * k], sel_count[n_grp] [device] as in
  * sic_select_columns.  1 <= k <= 128.  grp_ptr, cand_ptr [device].  The workspace
  * (sic_select_aggregated_workspace bytes, [device]) also holds the launches' work counters,
- * which the call zeroes on the stream itself; one call at a time per workspace. */
+ * which the call zeroes on the stream itself; one call at a time per workspace.  In SIC_FP64 it
+ * may have any alignment. */
 sic_status sic_select_aggregated_workspace(sic_handle* h, int64_t n_grp, int32_t max_cand, int32_t max_m,
                                            int32_t k, sic_precision prec, size_t* bytes);
 sic_status sic_select_aggregated(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp,

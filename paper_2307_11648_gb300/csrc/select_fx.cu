@@ -467,7 +467,8 @@ FxPlan fx_plan(sic_handle* h, long long units, int dim, int max_cand, int mm, in
              : nt == 256 ? fx_grid<256, ONE>(h, P.smem, work)
              : nt == 512 ? fx_grid<512, ONE>(h, P.smem, work)
                          : fx_grid<1024, ONE>(h, P.smem, work);
-    P.ws_bytes = 8 * L.words(L.cols - L.nc) * (size_t)P.grid;
+    // (16 more: the slabs start at the next 16-byte boundary of a workspace of any alignment)
+    P.ws_bytes = L.nc < L.cols ? 8 * L.words(L.cols - L.nc) * (size_t)P.grid + 16 : 0;
     return P;
 }
 
@@ -477,6 +478,7 @@ sic_status fx_launch(sic_handle* h, const FxPlan& P, const double* pts, long lon
                      const int32_t* cand_idx, int max_cand, int mm, int k, int32_t* sel_idx, int32_t* sel_count,
                      double* gain, void* ws, cudaStream_t s) {
     if (P.ws_bytes > 0 && !ws) return SIC_ERR_INVALID;
+    int4* slabs = reinterpret_cast<int4*>((reinterpret_cast<uintptr_t>(ws) + 15) / 16 * 16);
     FxLayout L = fx_layout<ONE>(max_cand, mm, k);
     L.nc = P.nc;
     const int e = fx_exponent(kp);
@@ -485,7 +487,7 @@ sic_status fx_launch(sic_handle* h, const FxPlan& P, const double* pts, long lon
 #define SIC_FX_LAUNCH(NTV)                                                                                      \
     k_select_fx<NTV, ONE><<<P.grid, NTV, P.smem, s>>>(pts, n, kp->dim, p, fl, e, targets, (const long long*)grp_ptr, \
                                                       units, (const long long*)cand_ptr, cand_idx, max_cand, k, \
-                                                      sel_idx, sel_count, (int4*)ws, L, gain, fl, h->d_status)
+                                                      sel_idx, sel_count, slabs, L, gain, fl, h->d_status)
     if (P.nt == 128)
         SIC_FX_LAUNCH(128);
     else if (P.nt == 256)
