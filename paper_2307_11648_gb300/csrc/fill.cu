@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
             for (int i = worker ? tid : nn; i < nn; i += FILL_NT)
                 pos[i] = (i < cnt) ? srt[cnt - 1 - i] : (int)(g0 + m - 1 - (i - cnt));
         if (tid == 0) s_bad = 0;
-        unit_theta<FILL_NT>(pts, dim, kp, tab, pos, nn, nmax, xyz, G, s_emax);
-        ldl_panels<FILL_NT>(G, fx, piv, nn, nmax, &s_bad);
+        unit_theta<FILL_NT, PARTIAL>(pts, dim, kp, tab, pos, nn, nmax, xyz, G, s_emax, &s_bad, false);
+        ldl_panels<FILL_NT, PARTIAL>(G, fx, piv, nn, nmax, &s_bad);
         if (s_bad) {
             if (tid == 0) record_error(st, SIC_ERR_NOT_PD, u);
             __syncthreads();
@@ -275,31 +275,52 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
                 jb = has ? jm[a] : -1;
                 jtop = max(jm[2 * p], 2 * p + 1 < m ? jm[2 * p + 1] : -1);
             }
-            // slots 2j and 2j+1 in the .x and .y halves of bh[j], bl[j] (packed updates); in the
-            // block of rows l of slot sb, the slots below sb take every row, slot sb the rows
-            // above its entry, and a slot above sb none: those get a = 0
-            const float2* Lf = reinterpret_cast<const float2*>(G);  // the L entries (hi, lo)
-            float2 bh[FILL_HSLOTS / 2], bl[FILL_HSLOTS / 2];
+            // (PARTIAL: FP64; else double-float)
+            double b64[PARTIAL ? FILL_HSLOTS : 1];
+            float2 bh[PARTIAL ? 1 : FILL_HSLOTS / 2], bl[PARTIAL ? 1 : FILL_HSLOTS / 2];
+            if constexpr (PARTIAL) {
 #pragma unroll
-            for (int j = 0; j < FILL_HSLOTS / 2; ++j) {
-                bh[j] = make_float2((hl + 32 * j == jb) ? 1.f : 0.f, (hl + 32 * j + 16 == jb) ? 1.f : 0.f);
-                bl[j] = make_float2(0.f, 0.f);
-            }
+                for (int q = 0; q < FILL_HSLOTS; ++q) b64[q] = hl + 16 * q == jb ? 1.0 : 0.0;
 #pragma unroll
-            for (int sb = FILL_HSLOTS - 1; sb >= 0; --sb) {
-                if (16 * sb > jtop) continue;
-                const int top = min(jtop, 16 * sb + 15);
-                for (int l = top; l >= 16 * sb; --l) {
-                    const int src = (lane & 16) | (l & 15);
-                    const float yh = __shfl_sync(0xffffffffu, (sb & 1) ? bh[sb / 2].y : bh[sb / 2].x, src);
-                    const float yl = __shfl_sync(0xffffffffu, (sb & 1) ? bl[sb / 2].y : bl[sb / 2].x, src);
-                    const int rl = pk(l, 0);
+                for (int sb = FILL_HSLOTS - 1; sb >= 0; --sb) {
+                    if (16 * sb > jtop) continue;
+                    const int top = min(jtop, 16 * sb + 15);
+                    for (int l = top; l >= 16 * sb; --l) {
+                        const double y = __shfl_sync(0xffffffffu, b64[sb], (lane & 16) | (l & 15));
+                        const double* Ll = G + pk(l, 0);
 #pragma unroll
-                    for (int j = 0; 2 * j <= sb; ++j) {
-                        const int i0 = hl + 32 * j, i1 = i0 + 16;
-                        const float2 a0 = (2 * j < sb || i0 < l) ? Lf[rl + i0] : make_float2(0.f, 0.f);
-                        const float2 a1 = (2 * j + 1 < sb || i1 < l) ? Lf[rl + i1] : make_float2(0.f, 0.f);
-                        df_sub_mul2(bh[j], bl[j], a0, a1, yh, yl);
+                        for (int q = 0; q <= sb; ++q) {
+                            const int i = hl + 16 * q;
+                            b64[q] = fma(q < sb || i < l ? -Ll[i] : 0.0, y, b64[q]);
+                        }
+                    }
+                }
+            } else {
+                // slots 2j and 2j+1 in the .x and .y halves of bh[j], bl[j] (packed updates); in the
+                // block of rows l of slot sb, the slots below sb take every row, slot sb the rows
+                // above its entry, and a slot above sb none: those get a = 0
+                const float2* Lf = reinterpret_cast<const float2*>(G);  // the L entries (hi, lo)
+#pragma unroll
+                for (int j = 0; j < FILL_HSLOTS / 2; ++j) {
+                    bh[j] = make_float2((hl + 32 * j == jb) ? 1.f : 0.f, (hl + 32 * j + 16 == jb) ? 1.f : 0.f);
+                    bl[j] = make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int sb = FILL_HSLOTS - 1; sb >= 0; --sb) {
+                    if (16 * sb > jtop) continue;
+                    const int top = min(jtop, 16 * sb + 15);
+                    for (int l = top; l >= 16 * sb; --l) {
+                        const int src = (lane & 16) | (l & 15);
+                        const float yh = __shfl_sync(0xffffffffu, (sb & 1) ? bh[sb / 2].y : bh[sb / 2].x, src);
+                        const float yl = __shfl_sync(0xffffffffu, (sb & 1) ? bl[sb / 2].y : bl[sb / 2].x, src);
+                        const int rl = pk(l, 0);
+#pragma unroll
+                        for (int j = 0; 2 * j <= sb; ++j) {
+                            const int i0 = hl + 32 * j, i1 = i0 + 16;
+                            const float2 a0 = (2 * j < sb || i0 < l) ? Lf[rl + i0] : make_float2(0.f, 0.f);
+                            const float2 a1 = (2 * j + 1 < sb || i1 < l) ? Lf[rl + i1] : make_float2(0.f, 0.f);
+                            df_sub_mul2(bh[j], bl[j], a0, a1, yh, yl);
+                        }
                     }
                 }
             }
@@ -313,10 +334,16 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
                 for (int q = 0; q < FILL_HSLOTS; ++q) {
                     const int i = hl + 16 * q;
                     if (i <= jb) {
-                        const float h = (q & 1) ? bh[q / 2].y : bh[q / 2].x;
-                        const float l = (q & 1) ? bl[q / 2].y : bl[q / 2].x;
+                        double x;
+                        if constexpr (PARTIAL) {
+                            x = b64[q];
+                        } else {
+                            const float h = (q & 1) ? bh[q / 2].y : bh[q / 2].x;
+                            const float l = (q & 1) ? bl[q / 2].y : bl[q / 2].x;
+                            x = f32_as_f64(h) + f32_as_f64(l);
+                        }
                         row_idx[e0 + jb - i] = pos[i];
-                        val[e0 + jb - i] = (f32_as_f64(h) + f32_as_f64(l)) * sc;
+                        val[e0 + jb - i] = x * sc;
                     }
                 }
             }
@@ -430,12 +457,12 @@ __global__ void k_fixed_point(const double* __restrict__ pa, const double* __res
             g1[j] = live ? ga[i * 4 + j] : 0.0;
             g2[j] = live ? gb[i * 4 + j] : 0.0;
         }
-        fx_row_store<4>(g1, fx, 512, 2 * t);
-        fx_row_store<4>(g2, fx, 512, 2 * t + 1);
+        fx_row_store<4, false>(g1, fx, 512, 2 * t);
+        fx_row_store<4, false>(g2, fx, 512, 2 * t + 1);
         __syncthreads();
         if (live) {
             d2[i] = fx_dist2(xf, 512, dim, 2 * t, 2 * t + 1, E[0], E[1], E[2]);
-            dot[i] = fx_dot<4>(fx, 512, 2 * t, 2 * t + 1);
+            dot[i] = fx_dot<4, false>(fx, 512, 2 * t, 2 * t + 1);
         }
         __syncthreads();
     }

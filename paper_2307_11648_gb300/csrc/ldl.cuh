@@ -1,6 +1,10 @@
 // The blocked LDL^T of the kernel matrix of a small point set in shared memory (one CTA: NT worker threads and
 // a pivot warp), shared by the fills (fill.cu, consecutive and nonadjacent groups) and the FP64 side state
 // (side.cu): Theta by unit_theta, the factorisation by ldl_panels.
+//
+// F64 (nonadjacent groups and side state): nothing is held in fewer bits than FP64 -- distances from FP64
+// differences, panel rows in 58 bits and rounded, L kept in FP64.  Consecutive groups: coordinates in fixed point,
+// panel rows truncated to 53 bits of the row's largest entry, L as double-float pairs of 48 bits.
 #pragma once
 
 #include "sic_internal.cuh"
@@ -55,7 +59,11 @@ __device__ __forceinline__ void fill_pivot(double v, int c, double* G, double* p
 // truncations stay below 2^-51 of the largest product: with G's rows (|G_ij| <= sqrt(A_ii)) the
 // error of an entry's update stays within a few B 2^-52 sqrt(A_ii A_ll), the order of the FP64
 // Cholesky's own backward error bound.
-template <int B>
+//
+// F64: M_j has five more bits (g_j = M_j 2^(E - 1080)) and is rounded, split at 2^29.  An entry is then held exactly
+// while its exponent is within 5 of E, else to 2^-59 of the row's largest, and what fx_dot leaves out is below 5 units of
+// 2^-58 of the largest product: the FP64 rounding of the sum and of the subtraction are what remains.
+template <int B, bool F64>
 __device__ __forceinline__ void fx_row_store(const double (&g)[B], int* __restrict__ fx, int ld, int row) {
     static_assert(B == 4, "the fixed-point rows are stored as int4");
     int e[B];
@@ -71,18 +79,22 @@ __device__ __forceinline__ void fx_row_store(const double (&g)[B], int* __restri
         const long long u = __double_as_longlong(g[j]);
         long long m = e[j] ? ((u & 0xfffffffffffffLL) | 0x10000000000000LL) : 0LL;
         const int sh = E - e[j];
-        m = sh < 63 ? (m >> sh) : 0LL;
+        if constexpr (F64)
+            m = sh < 60 ? (((m << 6) >> sh) + 1) >> 1 : 0LL;
+        else
+            m = sh < 63 ? (m >> sh) : 0LL;
         if (u < 0) m = -m;
-        mh[j] = (int)(m >> 26);
-        ml[j] = (int)(m & 0x3ffffffLL);
+        mh[j] = (int)(m >> (F64 ? 29 : 26));
+        ml[j] = (int)(m & (F64 ? 0x1fffffffLL : 0x3ffffffLL));
     }
     reinterpret_cast<int4*>(fx)[row] = make_int4(mh[0], mh[1], mh[2], mh[3]);
     reinterpret_cast<int4*>(fx)[ld + row] = make_int4(ml[0], ml[1], ml[2], ml[3]);
     fx[8 * ld + row] = E;
 }
 
-// s 2^e2 as FP64 by integer operations, the significand truncated (relative error < 2^-52);
+// s 2^e2 as FP64 by integer operations, the significand truncated (relative error < 2^-52) or, with ROUND, to nearest;
 // 0 for s = 0 and below FP64's normal range
+template <bool ROUND>
 __device__ __forceinline__ double i64_scaled(long long s, int e2) {
     if (s == 0) return 0.0;
     const unsigned long long sg = (unsigned long long)s & (1ULL << 63);
@@ -90,13 +102,18 @@ __device__ __forceinline__ double i64_scaled(long long s, int e2) {
     const int z = __clzll((long long)mag);
     const int be = e2 + 63 - z + 1023;
     if (be <= 0) return 0.0;
+    if constexpr (ROUND) {  // the significand's leading bit (or the carry to 2^53) adds to the exponent field
+        const unsigned long long m = (((mag << z) >> 10) + 1ULL) >> 1;
+        return __longlong_as_double((long long)(sg | (((unsigned long long)(be - 1) << 52) + m)));
+    }
     return __longlong_as_double((long long)(sg | ((unsigned long long)be << 52) | (((mag << z) >> 11) & 0xfffffffffffffULL)));
 }
 
 // sum_j g_ij g_lj of rows i and l: 2^52 sum Mh Mh + 2^26 sum (Mh Ml + Ml Mh) exactly in two 64-bit
 // sums of 32 x 32-bit products, scaled down by 2^52 into one 64-bit integer (the dropped fraction
-// and the omitted sum Ml Ml are below 5 units of 2^(Ei + El - 2098)), converted to FP64
-template <int B>
+// and the omitted sum Ml Ml are below 5 units of 2^(Ei + El - 2098)), converted to FP64.  (F64: 2^58 and 2^29, units of
+// 2^(Ei + El - 2102), the sums below 2^61.)
+template <int B, bool F64>
 __device__ __forceinline__ double fx_dot(const int* __restrict__ fx, int ld, int i, int l) {
     static_assert(B == 4, "the fixed-point rows are stored as int4");
     const int4 hi4 = reinterpret_cast<const int4*>(fx)[i], li4 = reinterpret_cast<const int4*>(fx)[ld + i];
@@ -109,7 +126,7 @@ __device__ __forceinline__ double fx_dot(const int* __restrict__ fx, int ld, int
         a2 += (long long)hi_[j] * hl[j];
         a1 += (long long)hi_[j] * ll[j] + (long long)li[j] * hl[j];
     }
-    return i64_scaled(a2 + (a1 >> 26), fx[8 * ld + i] + fx[8 * ld + l] - 2098);
+    return i64_scaled<F64>(a2 + (a1 >> (F64 ? 29 : 26)), fx[8 * ld + i] + fx[8 * ld + l] - (F64 ? 2102 : 2098));
 }
 
 // Theta over the nn points pos[0 .. nn) into G (packed lower): the coordinates go to fixed point at the
@@ -117,12 +134,15 @@ __device__ __forceinline__ double fx_dot(const int* __restrict__ fx, int ld, int
 // arithmetic (fx_dist2); the Matern in FP64 (matern_d2_fast; the all-double-float Matern of dfloat.cuh would
 // spare the FP64 pipe entirely, but its ~1e-14 of the variance per entry is amplified by 1/v in the Schur
 // complements, v ~ 2 nugget on the finest groups: factor columns then miss the oracle's by more than 1e-8).
+// F64: FP64 differences, which keep every pair's own precision whatever else is in the unit (a point far out
+// takes bits from the others' fixed-point coordinates); a non-finite entry raises *bad.
 // pos[i] is written by thread i mod NT; emax: three words, zero; ends with a barrier.  NT workers and one more warp.
-// With `twin` non-null, *twin becomes 2 if two points coincide.
-template <int NT>
+// Coincident points without a nugget (`singular`) make Theta singular: *bad is raised then, whatever the
+// factorisation's rounding would leave of the pivot.
+template <int NT, bool F64>
 __device__ __forceinline__ void unit_theta(const double* __restrict__ pts, int dim, const KP<double>& kp,
                                            const double* __restrict__ tab, const int* pos, int nn, int nmax, double* xyz,
-                                           double* G, unsigned* emax, int* twin = nullptr) {
+                                           double* G, unsigned* emax, int* bad, bool singular) {
     const int tid = threadIdx.x, lane = tid & 31;
     const bool worker = tid < NT;
     {
@@ -133,27 +153,41 @@ __device__ __forceinline__ void unit_theta(const double* __restrict__ pts, int d
             for (int d = 0; d < 3; ++d) {
                 const double x = (d < dim) ? pts[(long long)p * dim + d] : 0.0;
                 xyz[d * nmax + i] = x;
-                em[d] = max(em[d], ((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
+                if (!F64) em[d] = max(em[d], ((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
             }
         }
+        if constexpr (!F64) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            em[d] = __reduce_max_sync(0xffffffffu, em[d]);
-            if (lane == 0 && em[d]) atomicMax(&emax[d], em[d]);
+            for (int d = 0; d < 3; ++d) {
+                em[d] = __reduce_max_sync(0xffffffffu, em[d]);
+                if (lane == 0 && em[d]) atomicMax(&emax[d], em[d]);
+            }
         }
     }
     __syncthreads();
-    const int E0 = (int)emax[0], E1 = (int)emax[1], E2 = (int)emax[2];
+    int E0 = 0, E1 = 0, E2 = 0;
     long long* xf = reinterpret_cast<long long*>(xyz);
-    for (int i = worker ? tid : nn; i < nn; i += NT)
-        for (int d = 0; d < dim; ++d) xf[d * nmax + i] = fx_coord(xyz[d * nmax + i], d == 0 ? E0 : (d == 1 ? E1 : E2));
-    __syncthreads();
+    if constexpr (!F64) {
+        E0 = (int)emax[0], E1 = (int)emax[1], E2 = (int)emax[2];
+        for (int i = worker ? tid : nn; i < nn; i += NT)
+            for (int d = 0; d < dim; ++d)
+                xf[d * nmax + i] = fx_coord(xyz[d * nmax + i], d == 0 ? E0 : (d == 1 ? E1 : E2));
+        __syncthreads();
+    }
     // entry e = i (i + 1) / 2 + j, stepped by NT
     for (int i = worker ? pk_row(tid) : nn, j = worker ? tid - i * (i + 1) / 2 : 0; i < nn;) {
-        const double d2 = fx_dist2(xf, nmax, dim, i, j, E0, E1, E2);
+        double d2;
+        if constexpr (F64) {
+            const double dx = xyz[i] - xyz[j], dy = xyz[nmax + i] - xyz[nmax + j],
+                         dz = xyz[2 * nmax + i] - xyz[2 * nmax + j];
+            d2 = fma(dz, dz, fma(dy, dy, dx * dx));
+        } else {
+            d2 = fx_dist2(xf, nmax, dim, i, j, E0, E1, E2);
+        }
         double v = matern_d2_fast(kp, d2, tab);
-        if (i == j) v += kp.nugget;
-        else if (twin && d2 == 0.0) *twin = 2;
+        if (F64 && i != j && ((unsigned)__double2hiint(v) & 0x7ff00000u) == 0x7ff00000u) *bad = 2;
+        if (i == j) v = F64 ? kp.s2 + kp.nugget : v + kp.nugget;
+        else if (singular && __double_as_longlong(d2) == 0LL) *bad = 2;
         G[pk(i, j)] = v;
         j += NT;
         while (j > i) {
@@ -183,14 +217,23 @@ __device__ __forceinline__ void unit_theta(const double* __restrict__ pts, int d
 // panel costs two barriers.  Worker thread i owns row i (nn <= NT, the launcher's
 // choice).  Same operations, in the same order, as a column-by-column elimination.
 // (*bad becomes 1 where a pivot is not positive; piv: four doubles, fx: the scratch of fill_scratch_doubles; G's
-// off-diagonal entries end as double-float pairs; ends with a barrier.)
-template <int NT>
+// off-diagonal entries end as L, as double-float pairs or (F64) in FP64; ends with a barrier.)
+template <int NT, bool F64>
 __device__ __forceinline__ void ldl_panels(double* G, int* fx, double* piv, int nn, int nmax, int* bad) {
     const int tid = threadIdx.x, lane = tid & 31;
     const bool worker = tid < NT;
     const int i = tid;
     const int rowi = pk(i, 0);
     double lb[FILL_B];  // pivot warp: L of the block's row `lane` (columns below it)
+    auto store_l = [&](int at, double v) {
+        if constexpr (F64) {
+            G[at] = v;
+        } else {
+            float h, l;
+            f64_split(v, h, l);
+            reinterpret_cast<float2*>(G)[at] = make_float2(h, l);
+        }
+    };
     // the block [J, J + bs) (its entries final): lane r owns row J + r
     auto factor_block = [&](int J, int bs) {
         const int r = lane;
@@ -234,15 +277,11 @@ __device__ __forceinline__ void ldl_panels(double* G, int* fx, double* piv, int 
 #pragma unroll
                 for (int c2 = jj + 1; c2 < FILL_B; ++c2) u[c2] = fma(-l, G[pk(J + c2, J + jj)], u[c2]);
             }
-            fx_row_store<FILL_B>(gv, fx, nmax, i);
+            fx_row_store<FILL_B, F64>(gv, fx, nmax, i);
             // the L entries as double-float pairs (hi, lo) in their 8-byte slots (f64_split: 48
             // significant bits; only the member solves read them)
 #pragma unroll
-            for (int c = 0; c < FILL_B; ++c) {
-                float h, l;
-                f64_split(lv[c], h, l);
-                reinterpret_cast<float2*>(G)[rowi + J + c] = make_float2(h, l);
-            }
+            for (int c = 0; c < FILL_B; ++c) store_l(rowi + J + c, lv[c]);
         }
         __syncthreads();
         if (worker) {
@@ -255,7 +294,7 @@ __device__ __forceinline__ void ldl_panels(double* G, int* fx, double* piv, int 
                 int ii = pk_row(tid + nbt), ll = tid + nbt - ii * (ii + 1) / 2;
                 while (ii < nt) {
                     const int i = je + ii, l = je + ll;
-                    G[pk(i, l)] -= fx_dot<FILL_B>(fx, nmax, i, l);
+                    G[pk(i, l)] -= fx_dot<FILL_B, F64>(fx, nmax, i, l);
                     ll += NT;
                     while (ll > ii) {
                         ll -= ii + 1;
@@ -264,23 +303,19 @@ __device__ __forceinline__ void ldl_panels(double* G, int* fx, double* piv, int 
                 }
             }
         } else {
-            // the block's L entries, as double-float pairs, now that the workers have read its
+            // the block's L entries, now that the workers have read its
             // unscaled entries; then the next block: its update, and its factorisation
             const int bs = je - J;
             if (lane < bs) {
 #pragma unroll
                 for (int c = 0; c < FILL_B - 1; ++c)
-                    if (c < lane) {
-                        float h, l;
-                        f64_split(lb[c], h, l);
-                        reinterpret_cast<float2*>(G)[pk(J + lane, J + c)] = make_float2(h, l);
-                    }
+                    if (c < lane) store_l(pk(J + lane, J + c), lb[c]);
             }
             if (je < nn) {
                 const int bs2 = min(FILL_B, nn - je);
                 if (lane < bs2 * (bs2 + 1) / 2) {
                     const int ii = pk_row(lane), ll = lane - ii * (ii + 1) / 2;
-                    G[pk(je + ii, je + ll)] -= fx_dot<FILL_B>(fx, nmax, je + ii, je + ll);
+                    G[pk(je + ii, je + ll)] -= fx_dot<FILL_B, F64>(fx, nmax, je + ii, je + ll);
                 }
                 __syncwarp();
                 factor_block(je, bs2);

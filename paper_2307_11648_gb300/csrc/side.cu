@@ -54,8 +54,6 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
     const bool worker = tid < NT;
     const double NaN = __longlong_as_double(0x7ff8000000000000LL);
     exp_table_fill(tab, kp.s2);
-    // without a nugget coincident points make Theta singular: exactly so, whatever the factorisation's rounding
-    int* twin = kp.nugget > 0.0 ? nullptr : &s_npd;
 
     // this launch's units (the invalid ones are the first class's to report)
     auto in_class = [&](long long u) {
@@ -94,8 +92,8 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
                     pos[i] = i < m0 ? (int)(p0 + i) : sel_idx[u * k + (i - m0)];
                 if (tid < 3) s_emax[tid] = 0u;
                 __syncthreads();
-                unit_theta<NT>(pts, dim, kp, tab, pos, nn, NMAX, xyz, G, s_emax, twin);
-                ldl_panels<NT>(G, fx, piv, nn, NMAX, &s_npd);
+                unit_theta<NT, false>(pts, dim, kp, tab, pos, nn, NMAX, xyz, G, s_emax, &s_npd, !(kp.nugget > 0.0));
+                ldl_panels<NT, false>(G, fx, piv, nn, NMAX, &s_npd);
                 if (pass == 0) {
                     for (int t = tid; t < cnt; t += NT + 32) v1s[t] = G[pk(t, t)];
                     __syncthreads();
