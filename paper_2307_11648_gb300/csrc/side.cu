@@ -49,7 +49,6 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
     int* pos = reinterpret_cast<int*>(sm + L.size());
     __shared__ ClassDeal<NT + 32> deal;
     __shared__ int s_bad, s_npd;  // invalid unit or pick; a pivot not positive
-    __shared__ unsigned s_emax[3];
     const int tid = threadIdx.x, NMAX = L.nmax;
     const bool worker = tid < NT;
     const double NaN = __longlong_as_double(0x7ff8000000000000LL);
@@ -90,10 +89,10 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
                 const int m0 = pass == 0 ? 0 : m, nn = m0 + cnt;
                 for (int i = worker ? tid : nn; i < nn; i += NT)
                     pos[i] = i < m0 ? (int)(p0 + i) : sel_idx[u * k + (i - m0)];
-                if (tid < 3) s_emax[tid] = 0u;
                 __syncthreads();
-                unit_theta<NT, false>(pts, dim, kp, tab, pos, nn, NMAX, xyz, G, s_emax, &s_npd, !(kp.nugget > 0.0));
-                ldl_panels<NT, false>(G, fx, piv, nn, NMAX, &s_npd);
+                unit_theta<NT, true>(pts, dim, kp, tab, pos, nn, NMAX, xyz, G, nullptr, &s_npd,
+                                     !(kp.nugget > 0.0));
+                ldl_panels<NT, true>(G, fx, piv, nn, NMAX, &s_npd);
                 if (pass == 0) {
                     for (int t = tid; t < cnt; t += NT + 32) v1s[t] = G[pk(t, t)];
                     __syncthreads();
@@ -221,7 +220,8 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
                 if (a != b) {
                     const double dx = xyz[a] - xyz[b], dy = xyz[NMAX + a] - xyz[NMAX + b],
                                  dz = xyz[2 * NMAX + a] - xyz[2 * NMAX + b];
-                    v = matern_d2_fast(kp, fma(dz, dz, fma(dy, dy, dx * dx)), tab);
+                    const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
+                    v = matern_d2_fast(kp, d2, tab);
                 }
                 A[e] = v;
                 if (b >= m) B[pk(a - m, b - m)] = v;

@@ -111,6 +111,30 @@ def test_partial_fill_with_a_far_point(env):  # noqa: F811
     assert err.max() <= 1e-12 and lerr.max() <= 1e-12
 
 
+@pytest.mark.parametrize("units", [40, 1800])  # the flat kernel and the panels
+def test_side_state_with_a_far_point(env, units):  # noqa: F811
+    torch, sic, pipeline, h = env
+    kp = sic.kernel(2, 5, 0.2, 1.3, 1e-2)
+    n, k = 2000, 19
+    pts = synthetic.points(n, 2, 14)
+    pts[n - 1] = FAR
+    targets = (5 * (np.arange(units) % 300)).astype(np.int32)
+    sel = np.stack([1500 + (7 * np.arange(k) + 13 * (u % 31)) % 480 for u in range(units)]).astype(np.int32)
+    sel[:, -1] = n - 1
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()  # noqa: E731
+
+    def side(cnt):
+        out = [torch.zeros(units * k, dtype=torch.float64, device="cuda") for _ in range(2)]
+        sic.side_state_fp64(h, dpts, kp, d(sel.reshape(-1)), d(np.full(units, cnt, np.int32)), k, targets=d(targets),
+                            pvar=out[0], pvar_p=out[1])
+        h.sync()
+        return [x.view(units, k).cpu().numpy()[:, :k - 1] for x in out]
+
+    dpts = d(pts)
+    for a, b in zip(side(k), side(k - 1)):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf])
 def test_a_point_without_coordinates_has_no_factor(env, value):  # noqa: F811
     torch, sic, pipeline, h = env
@@ -121,3 +145,13 @@ def test_a_point_without_coordinates_has_no_factor(env, value):  # noqa: F811
     with pytest.raises(sic.SicError) as e:
         _partial(env, pts, kp, groups, 12)
     assert e.value.code == sic.SIC_ERR_NOT_PD
+    for units in (20, 1800):
+        d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()  # noqa: E731
+        sel = np.tile(groups[0][1].astype(np.int32), (units, 1))
+        out = torch.zeros(units * 12, dtype=torch.float64, device="cuda")
+        sic.side_state_fp64(h, d(pts), kp, d(sel.reshape(-1)), d(np.full(units, 12, np.int32)), 12,
+                            targets=d(np.zeros(units, np.int32)), pvar=out)
+        with pytest.raises(sic.SicError) as e:
+            h.sync()
+        assert e.value.code == sic.SIC_ERR_NOT_PD
+        assert np.all(np.isnan(out.cpu().numpy()))
