@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(c
             for (int i = worker ? tid : nn; i < nn; i += FILL_NT)
                 pos[i] = (i < cnt) ? srt[cnt - 1 - i] : (int)(g0 + m - 1 - (i - cnt));
         if (tid == 0) s_bad = 0;
-        unit_theta<FILL_NT, PARTIAL>(pts, dim, kp, tab, pos, nn, nmax, xyz, G, s_emax, &s_bad, false);
+        unit_theta<FILL_NT, PARTIAL>(pts, dim, kp, tab, pos, nn, nmax, xyz, G, s_emax, &s_bad, !(kp.nugget > 0.0));
         ldl_panels<FILL_NT, PARTIAL>(G, fx, piv, nn, nmax, &s_bad);
         if (s_bad) {
             if (tid == 0) record_error(st, SIC_ERR_NOT_PD, u);

@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
     __shared__ int s_bad;  // 1: invalid unit or pick, 2: a pivot not positive
     const int tid = threadIdx.x, NMAX = L.nmax;
     const double diag = kp.s2 + kp.nugget;
+    const bool singular = !(kp.nugget > 0.0);
     const double NaN = __longlong_as_double(0x7ff8000000000000LL);
     exp_table_fill(tab, kp.s2);
     if (L.dec)
@@ -221,6 +222,8 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
                     const double dx = xyz[a] - xyz[b], dy = xyz[NMAX + a] - xyz[NMAX + b],
                                  dz = xyz[2 * NMAX + a] - xyz[2 * NMAX + b];
                     const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
+                    // coincident points without a nugget: singular, whatever rounding leaves of the pivot
+                    if (singular && __double_as_longlong(d2) == 0LL) s_bad = 2;
                     v = matern_d2_fast(kp, d2, tab);
                 }
                 A[e] = v;
