@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
     long long* rM = reinterpret_cast<long long*>(T + (ONE ? 0 : tri_row((L.mm + 1) / 2 * 2)));
     int* rS = reinterpret_cast<int*>(rM + (ONE ? 0 : L.mm));
     // coordinates: as read, then in fixed point at the unit's largest exponent per dimension (fx_coord)
+    // where that is exact (a point near zero or far out leaves no room for all bits), else in FP64
     double* X = reinterpret_cast<double*>(rS + (ONE ? 0 : 2 * L.mm));
     const long long* Xf = reinterpret_cast<const long long*>(X);
     const int ldx = L.Cm + (ONE ? 0 : L.mm);
@@ -129,8 +130,19 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
     auto entry = [&](int c, int r) -> int2* {  // entry of column c, row r
         return reinterpret_cast<int2*>((c < nc ? S : W) + (c >> 1) * Cm + r) + (c & 1);
     };
+    bool plain = false;  // the unit's coordinates stay in FP64
     auto theta = [&](int i, int j) -> double {
-        return matern_d2_fast(kp, fx_dist2(Xf, ldx, dim, i, j, s_ex[0], s_ex[1], s_ex[2]), tab);
+        double d2;
+        if (plain) {
+            d2 = 0.0;
+            for (int d = 0; d < dim; ++d) {
+                const double df = X[d * ldx + i] - X[d * ldx + j];
+                d2 = fma(df, df, d2);
+            }
+        } else {
+            d2 = fx_dist2(Xf, ldx, dim, i, j, s_ex[0], s_ex[1], s_ex[2]);
+        }
+        return matern_d2_fast(kp, d2, tab);
     };
     // sum over columns c0 .. c0 + len (c0 even) of row r with the pivot's entries p; where len is odd the
     // pivot's next entry is zero (the column's may be anything)
@@ -219,11 +231,16 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
             if (lane == 0 && b > 0) atomicMax(&s_ex[d], b);
         }
         __syncthreads();
-        for (int i = tid; i < C + mt; i += NT) {
-            const int xi = i < C ? i : Cm + (i - C);
-            for (int d = 0; d < dim; ++d)
-                reinterpret_cast<long long*>(X)[d * ldx + xi] = fx_coord(X[d * ldx + xi], s_ex[d]);
-        }
+        bool cut = false;
+        for (int i = tid; i < C + mt; i += NT)
+            for (int d = 0; d < dim; ++d) cut = cut || !fx_coord_exact(X[d * ldx + (i < C ? i : Cm + (i - C))], s_ex[d]);
+        plain = __syncthreads_or(cut);
+        if (!plain)
+            for (int i = tid; i < C + mt; i += NT) {
+                const int xi = i < C ? i : Cm + (i - C);
+                for (int d = 0; d < dim; ++d)
+                    reinterpret_cast<long long*>(X)[d * ldx + xi] = fx_coord(X[d * ldx + xi], s_ex[d]);
+            }
         if (!ONE) __syncthreads();
         if constexpr (ONE) {
             for (int i = tid; i < C; i += NT) VB[i] = matern_d2_fast(kp, VB[i], tab);

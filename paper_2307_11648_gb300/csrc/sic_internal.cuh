@@ -322,6 +322,15 @@ __device__ __forceinline__ long long fx_coord(double x, int E) {
     return u < 0 ? -f : f;
 }
 
+// whether fx_coord(x, E) is x itself, and E far enough from overflow for fx_dist2
+__device__ __forceinline__ bool fx_coord_exact(double x, int E) {
+    const long long u = __double_as_longlong(x);
+    const int e = (int)((u >> 52) & 0x7ff), drop = E - e - 9;  // low bits of the significand cut off
+    if ((u << 1) == 0LL) return true;
+    if (e == 0 || E > 1500) return false;
+    return drop <= 0 || (drop < 53 && (u & ((1LL << drop) - 1)) == 0LL);
+}
+
 // dx^2 of one dimension, exact in 128 bits (h:l), for a difference |dx| < 2^63
 __device__ __forceinline__ void sq128(long long dx, unsigned long long& h, unsigned long long& l) {
     const unsigned long long a = dx < 0 ? 0ULL - (unsigned long long)dx : (unsigned long long)dx;
