@@ -49,6 +49,12 @@ __device__ __forceinline__ long long fx_mul(long long n, long long M, int s) {
     return s >= 0 ? p << s : (p + (1LL << (-s - 1))) >> -s;  // s >= -2: r^2 >= 2^(-2e) / 1.9
 }
 
+// binary exponent of x (-1023 for zero); integer operations only
+__device__ __forceinline__ int exponent_of(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// covariances with the target below 2^(2e - FX_COV_BITS) are selected with FP64 rows (select_fx.cu)
+constexpr int FX_COV_BITS = 30;
+
 __device__ __forceinline__ bool not_finite(double x) {
     return ((unsigned)__double2hiint(x) & 0x7ff00000u) == 0x7ff00000u;
 }

@@ -26,6 +26,12 @@
 // a rule) go to a list, and of several the FP64 quotient decides, ties to the lowest candidate index;
 // the pivot's rows are staged, every row gets its new entries and its variances are downdated.
 //
+// Single columns are scored by their covariance with the target, which may be far below the variance (points many
+// length scales apart) and is then down to products of entries below the fixed point's resolution.  When the best
+// candidate's covariance falls below 2^-30 of the variance -- what the format still resolves to 2^-28 -- the column
+// starts over with its rows in FP64 (same storage).  Variances ratios (supernodes) lose nothing: an entry below the
+// resolution changes no variance.
+//
 // Bound: latency of the step's phases (with 1024 candidates per supernode 44 % of the issue slots and
 // 35 % of the FP64 pipe are busy, L2 delivers 30 bytes per clock and SM); half of each scheduler's warps therefore
 // evaluate Theta while the others sum.  N = 2^16 with 1024 candidates, k = 64 (2,811 supernodes): 61.3 ms with FP64
@@ -173,7 +179,8 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
         return a.value();
     };
 
-    for (long long g = blockIdx.x; g < n_units; g += gridDim.x) {
+    bool rows64 = false;  // (columns) the unit once more, its factor rows in FP64
+    for (long long g = blockIdx.x; g < n_units; g += rows64 ? 0LL : (long long)gridDim.x) {
         const long long g0 = ONE ? (targets ? (long long)targets[g] : g) : grp_ptr[g];
         const int m = ONE ? 1 : (int)(grp_ptr[g + 1] - g0);
         const long long b0 = cand_ptr[g];
@@ -309,6 +316,7 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
         // ---- the steps ----
         double vt = diag;  // columns: the target's variance (thread 0, gains only)
         int t = 0;
+        bool again = false;
         if (!s_fail) {
             for (; t < k; ++t) {
                 int* cnt = &s_cnt[t & 1];
@@ -370,6 +378,10 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
                     if (!s_go) break;
                     q = s_q;
                 }
+                if (ONE && !rows64 && exponent_of(VB[q]) < 2 * e - FX_COV_BITS) {
+                    again = true;
+                    break;
+                }
                 // ---- stage the pivot: its rows, and 1/sqrt of its variances by the last warp ----
                 if (warp == NW - 1) {
                     const double v = (!ONE && lane == 1) ? VB[q] : VA[q];
@@ -398,39 +410,56 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
                 fx_factor(s_r[0], e, M1, h1);
                 if (!ONE) fx_factor(s_r[1], e, M2, h2);
                 const double ut = ONE ? vbq * s_r[0] : 0.0;
-                for (int r = tid; r < C; r += NT) {
-                    const double va = VA[r];
-                    if (!(va >= -1e300)) continue;  // picked, invalid (-inf) or NaN
-                    // half of each scheduler's warps evaluate Theta (FP64 pipe) before the sums (integer
-                    // pipes and loads), the other half after them
-                    double th = 0.0;
-                    long long s1 = 0, s2 = 0;
+                if (ONE && rows64) {
+                    const double2* p = reinterpret_cast<const double2*>(p1);
+                    for (int r = tid; r < C; r += NT) {
+                        const double va = VA[r];
+                        if (!(va >= -1e300)) continue;
+                        double num = theta(r, q);
+                        if (r == q) num += kp.nugget;
+                        const double2* F = reinterpret_cast<const double2*>(S) + r;
+                        for (int c = 0; c < t >> 1; ++c) num = fma(-F[c * Cm].y, p[c].y, fma(-F[c * Cm].x, p[c].x, num));
+                        if (t & 1) num = fma(-F[(t >> 1) * Cm].x, p[t >> 1].x, num);
+                        const double u = num * s_r[0];
+                        *reinterpret_cast<double*>(entry(t, r)) = u;
+                        VA[r] = r == q ? NEG : fma(-u, u, va);  // (NaN: never a candidate again)
+                        VB[r] = fma(-u, ut, VB[r]);
+                    }
+                } else {
+                    for (int r = tid; r < C; r += NT) {
+                        const double va = VA[r];
+                        if (!(va >= -1e300)) continue;  // picked, invalid (-inf) or NaN
+                        // half of each scheduler's warps evaluate Theta (FP64 pipe) before the sums (integer
+                        // pipes and loads), the other half after them
+                        double th = 0.0;
+                        long long s1 = 0, s2 = 0;
 #pragma unroll 1
-                    for (int ph = 0; ph < 2; ++ph) {
-                        if (ph == ((warp >> 2) & 1)) {
-                            th = theta(r, q);
-                        } else {
-                            if constexpr (!ONE) s2 = dot(0, mt + t, r, p2);
-                            s1 = dot(fb, t, r, p1);
+                        for (int ph = 0; ph < 2; ++ph) {
+                            if (ph == ((warp >> 2) & 1)) {
+                                th = theta(r, q);
+                            } else {
+                                if constexpr (!ONE) s2 = dot(0, mt + t, r, p2);
+                                s1 = dot(fb, t, r, p1);
+                            }
                         }
+                        if (r == q) th += kp.nugget;
+                        if (not_finite(th)) {  // never a candidate again
+                            VA[r] = VB[r] = NAN;
+                            continue;
+                        }
+                        const long long tx = fx_of_positive(th, FXS - 2 * e);
+                        if constexpr (!ONE) {
+                            const long long u2 = fx_mul(tx - s2, M2, h2);
+                            *entry(mt + t, r) = fx_split(u2);
+                            const double d2 = fx_to_double(u2, e - FXS);
+                            VB[r] = r == q ? NEG : fma(-d2, d2, VB[r]);
+                        }
+                        const long long u1 = fx_mul(tx - s1, M1, h1);
+                        *entry(fb + t, r) = fx_split(u1);
+                        const double d1 = fx_to_double(u1, e - FXS);
+                        VA[r] = r == q ? NEG : fma(-d1, d1, va);
+                        if constexpr (ONE) VB[r] = fma(-d1, ut, VB[r]);
                     }
-                    if (r == q) th += kp.nugget;
-                    if (not_finite(th)) {  // never a candidate again
-                        VA[r] = VB[r] = NAN;
-                        continue;
-                    }
-                    const long long tx = fx_of_positive(th, FXS - 2 * e);
-                    if constexpr (!ONE) {
-                        const long long u2 = fx_mul(tx - s2, M2, h2);
-                        *entry(mt + t, r) = fx_split(u2);
-                        const double d2 = fx_to_double(u2, e - FXS);
-                        VB[r] = r == q ? NEG : fma(-d2, d2, VB[r]);
-                    }
-                    const long long u1 = fx_mul(tx - s1, M1, h1);
-                    *entry(fb + t, r) = fx_split(u1);
-                    const double d1 = fx_to_double(u1, e - FXS);
-                    VA[r] = r == q ? NEG : fma(-d1, d1, va);
-                    if constexpr (ONE) VB[r] = fma(-d1, ut, VB[r]);
                 }
                 if (ONE && gain && tid == 0) {
                     vt = fmax(vt - ut * ut, vfloor);
@@ -441,6 +470,11 @@ __global__ void __launch_bounds__(NT, FX_THREADS / NT) k_select_fx(
         // the picks' global indices and (with gain) the decreases of 2 KL per nonzero (Section 5.4), off the
         // step chain
         __syncthreads();
+        if (ONE && again) {
+            rows64 = true;
+            continue;
+        }
+        rows64 = false;
         for (int q = tid; q < t; q += NT) {
             sel_idx[g * k + q] = cand_idx[b0 + qs[q]];
             if (gain) gain[g * k + q] = ONE ? log(gv1[q] / gv1[q + 1]) : log(gv1[q] / gv2[q]) / m;

@@ -18,6 +18,8 @@
 // In FP64 the factor is held in fixed point (fx.cuh, select_fx.cu): exact integer dot products instead of FP64
 // multiply-adds, and scores in FP32 first, the FP64 quotient only where a row is within 2^-18 of its block's largest.
 //
+// (A best covariance below 2^-30 of the variance starts over with the rows in FP64, as in select_fx.cu.)
+//
 // Bound: a barrier and four dependent L2 round trips per step, then the factor's L2 traffic (4 n k^2 bytes) and the FP64
 // pipe.  One block on one SM was the whole kernel: 98.3 ms for n = 65,536, k = 64 in FP64 (3-D, Matern 5/2); over
 // the grid with FP64 multiply-adds and divisions 1.16 ms, in fixed point 0.85 ms.
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
     __shared__ Best<T> wbest[NW_MAX];
     __shared__ long long s_q;
     __shared__ T s_rs, s_ut;
-    __shared__ int s_ok;
+    __shared__ int s_ok, s_small;
     __shared__ double tab[F64 ? EXP_TAB : 1];  // s2 2^(j/256): the FP64 Matern's exp
     T* F = ws;
     T* var = F + (long long)k * n;
@@ -116,15 +118,18 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
         exp_table_fill(tab, kp.s2);
         __syncthreads();
     }
-    for (long long j = j0; j < n; j += jstep) {
-        T d2 = (T)0;
-        for (int d = 0; d < dim; ++d) {
-            T df = (T)(xtr[j * dim + d] - org[d]);
-            d2 += df * df;
+    auto unconditional = [&]() {
+        for (long long j = j0; j < n; j += jstep) {
+            T d2 = (T)0;
+            for (int d = 0; d < dim; ++d) {
+                T df = (T)(xtr[j * dim + d] - org[d]);
+                d2 += df * df;
+            }
+            var[j] = kp.s2 + kp.nugget;
+            cov[j] = theta(d2);
         }
-        var[j] = kp.s2 + kp.nugget;
-        cov[j] = theta(d2);
-    }
+    };
+    unconditional();
     double vt = (double)(kp.s2 + kp.nugget);
     if (j0 == 0) out_var[0] = vt;
     // FP32 score key of a row (0: not a candidate)
@@ -149,8 +154,9 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
         const int src = __ffs(__ballot_sync(FULL, b.idx == i)) - 1;
         b = Best<T>{s, __shfl_sync(FULL, b.var, src), __shfl_sync(FULL, b.cov, src), i};
     };
-    int t = 0;
-    for (; t < k; ++t) {
+    bool rows64 = false;  // (FP64) from the start once more, the factor's rows in FP64
+    int t = 0, round = 0;
+    for (; t < k; ++t, ++round) {
         Best<T> b{NEG, (T)0, (T)0, NONE};
         unsigned lim = 1u, mine = 0u;
         if constexpr (F64) {
@@ -183,10 +189,10 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
             warp_best(b);
             int ok = 1;
             if (gridDim.x > 1) {
-                Best<T>* all = bests + (t & 1) * gridDim.x;
+                Best<T>* all = bests + (round & 1) * gridDim.x;
                 if (lane == 0) {
                     all[blockIdx.x] = b;
-                    ok = grid_wait(count, (unsigned)gridDim.x * (unsigned)(t + 1));
+                    ok = grid_wait(count, (unsigned)gridDim.x * (unsigned)(round + 1));
                 }
                 ok = __shfl_sync(FULL, ok, 0);
                 b = Best<T>{NEG, (T)0, (T)0, NONE};
@@ -200,6 +206,7 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
                 s_ok = ok;
                 const bool go = ok && b.idx != NONE && b.score > (T)0;
                 s_q = go ? b.idx : NONE;
+                s_small = F64 && go && !rows64 && exponent_of((double)b.cov) < 2 * e - FX_COV_BITS;
                 if (go) {
                     if constexpr (F64)
                         s_rs = rsqrt_newton(b.var);
@@ -216,6 +223,13 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
         }
         const long long q = s_q;
         if (q == NONE) break;
+        if (F64 && s_small) {  // every block decides the same from the same best
+            rows64 = true;
+            unconditional();
+            vt = (double)(kp.s2 + kp.nugget);
+            t = -1;
+            continue;
+        }
         const T rs = s_rs, ut = s_ut;
         T qx[3] = {(T)0, (T)0, (T)0};
         for (int d = 0; d < dim; ++d) qx[d] = coord(q, d);
@@ -235,7 +249,11 @@ __global__ void __launch_bounds__(NT_MAX) k_select_single(const double* __restri
             T num = theta(d2);
             if (j == q) num += kp.nugget;
             T u;
-            if constexpr (F64) {
+            if (F64 && rows64) {
+                for (int tau = 0; tau < t; ++tau) num = fma(-F[(long long)tau * n + j], piv[tau], num);
+                u = num * rs;
+                if (t + 1 < k) F[(long long)t * n + j] = u;
+            } else if constexpr (F64) {
                 long long sum = 0, ux = 0;
                 for (int c0 = 0; c0 < t; c0 += 256) {  // (the cross sums stay in 64 bits over 256 columns)
                     const int c1 = min(t, c0 + 256);
