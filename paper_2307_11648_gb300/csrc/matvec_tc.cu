@@ -4,20 +4,26 @@
 // kernel for few right-hand sides); what cost most was summing their products to far below FP32, 11
 // operations per entry and right-hand side.  Here both factors are cut into 8-bit digits, which BF16
 // holds exactly, and the digits' products are summed exactly (after Ozaki et al., Numer. Algorithms 59 (2012)):
-//   Theta_ij / 2^E = sum_a A_a 2^-(7 + 8a), a = 0..5 (2^E >= variance),
-//   x_jr / 2^X_r   = sum_b B_b 2^-(7 + 8b), b = 0..5 (2^X_r > max_j |x_jr|), |A_a|, |B_b| <= 128,
+//   Theta_ij / 2^E = sum_a A_a 2^-(7 + 8a), a = 0..7 (2^E >= variance),
+//   x_jr / 2^X_r   = sum_b B_b 2^-(7 + 8b), b = 0..7 (2^X_r > max_j |x_jr|), |A_a|, |B_b| <= 128,
 // with A_0 = round(128 Theta / 2^E), the remainder times 256, and so on (exact FP32 operations).  Products of
-// level a + b = l <= 5 go to one accumulator: 128 sources x 6 pairs x 2^14 < 2^24, so FP32 holds every partial
-// sum exactly; after 128 sources the levels are added to two 64-bit integers per row and right-hand
-// side.  What is left out (digits below 2^-47 of the variance and of max|x|, levels from 6 on) is below 2^-46 max|x|
-// per term, of random sign: about 2^-38 max|x| over 50,000 sources, 1e-12 of a typical result.  The integers do
-// not depend on the order of the sum.
+// level a + b = l <= 8 go to one accumulator: 128 sources x 8 pairs x 2^14 <= 2^24, so FP32 holds every partial
+// sum exactly; after 128 sources the levels are added to three 64-bit integers per row and right-hand
+// side.  The integers do not depend on the order of the sum.
+//
+// Accuracy.  An FP32 entry is held exactly from 2^-40 of the variance on, an x from 2^-10 of max|x| on; the digits cut off
+// below that and the levels left out come to about sqrt(n) 2^-68 variance max|x| in a row (their signs are random).
+// A row must be as good as its own sum S_i = sum_j |Theta_ij x_j|, not as max|x|: a row far from a large x_j, or one
+// with a wide range of x, has a small S_i.  So one more MMA per step sums A_0 times the leading 15 bits of |x|, a
+// lower bound of S_i (to its rounding), and where it stays below sqrt(n) 2^-20 variance max|x| the entry of y is marked (a
+// NaN with a payload of its own) and k_matvec_rows, launched behind, forms it in double-FP32.  The others are within
+// 2^-48 of S_i, as far as such sums go.  (With six digits and no check, rows beside a spike of 1e12 were off by 1e-3 S_i,
+// and rows of a unit vector's product lost entries below 2^-47.)
 //
 // A CTA takes 128 rows (TMEM lanes) and, in a cluster, a share of the sources; 256 threads = row and half of a step's
-// 16 sources.  Per step the threads write the six digit tiles of Theta (128 x 16 BF16, K-major core matrices) into
-// one of two buffers and one thread issues six MMAs (digit a against B_0 .. B_(5-a), N = 48, 48, 32, 32, 16, 16 into
-// the columns from level a on; where that is one digit more than needed it lands in level 6, which is not
-// read).  The MMAs run under the next step's evaluation; the accumulators (two sets) are read one chunk late.
+// 16 sources.  Per step the threads write the eight digit tiles of Theta (128 x 16 BF16, K-major core matrices) into
+// one of two buffers and one thread issues the MMAs, digit a against B_0 .. B_(8-a) into the columns from level a on (N a
+// multiple of 16; where that is one digit more than needed it lands in level 9, which is not read).  The MMAs run under the next step's evaluation; the accumulators (two sets) are read one chunk late.
 //
 // Bound: FP32 issue of the kernel evaluation and the digits, about 45 operations per entry whatever the
 // number of right-hand sides.  N = 50,001 with 8 of them: 16.6 ms with double-FP32 sums on the CUDA cores, 6.8 ms
@@ -28,19 +34,30 @@
 namespace {
 
 constexpr int ROWS = 128, CH = 128, SUB = 16, NT = 256;
-constexpr int KD = 6, XD = 6;  // digits of Theta and of x
+constexpr int KD = 8, XD = 8;    // digits of Theta and of x
+constexpr int BR = XD * 8 + 16;  // rows of an x tile: the digits, then the leading 7 and the next 8 bits of |x|
 constexpr int A_TILE = ROWS * SUB * 2;       // one digit tile
 constexpr int SA = 0;                        // [2 buffers][KD] tiles
-constexpr int SB = SA + 2 * KD * A_TILE;     // [2 chunks] digits of x: XD * 8 rows x CH, K-major
-constexpr int B_TILE = XD * 8 * CH * 2;
+constexpr int SB = SA + 2 * KD * A_TILE;     // [2 chunks] x: BR rows x CH, K-major
+constexpr int B_TILE = BR * CH * 2;
+constexpr int B_GROUP = (CH / 8) * 128;      // 8 rows of it
 constexpr int SC = SB + 2 * B_TILE;          // [2 chunks][3][CH] negated coordinates
 constexpr int SX = SC + 2 * 3 * CH * 4;      // largest biased exponent per right-hand side, a flag
 constexpr int SBAR = SX + 16 * 4;            // two mbarriers, TMEM address
 constexpr int SMEM_MV = SBAR + 32;
-constexpr int SACC = SA;                     // [ROWS][8][2] 64-bit sums for the cluster (after the last MMA)
-static_assert(ROWS * 8 * 2 * 8 <= SB, "the sums fit in the digit tiles");
-// two CTAs per SM: 256 of the 512 TMEM columns, none waits for them
-constexpr unsigned TMEM_COLS = 128;
+constexpr int SACC = SA;                     // [ROWS][8][4] 64-bit sums for the cluster (after the last MMA)
+static_assert(ROWS * 8 * 4 * 8 <= SB, "the sums fit in the digit tiles");
+// two CTAs per SM: all 512 TMEM columns, none waits for them
+constexpr unsigned TMEM_COLS = 256;
+constexpr uint32_t T_SET = 128;              // columns of an accumulator set: 8 per level 0 .. 9, then S
+constexpr uint32_t T_S = 80;
+constexpr int S_BITS = 20;                   // marked below sqrt(n) 2^-S_BITS
+
+// an entry of y that k_matvec_rows has to form; the low bits hold the biased exponent of max|x|
+constexpr unsigned long long MARK = 0x7ff85ac000000000ULL;
+__device__ __forceinline__ bool is_marked(double v) {
+    return ((unsigned long long)__double_as_longlong(v) & ~0x7ffULL) == MARK;
+}
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
     uint32_t r[4];
@@ -111,7 +128,7 @@ template <int NU>
 __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ pts, long long n, int dim, KP<float> kp,
                                                      float to_unit, int E, double diag_extra,
                                                      const double* __restrict__ x, double* __restrict__ y, int nrhs,
-                                                     int parts, DevStatus* st) {
+                                                     int parts, float least, DevStatus* st) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int row = (warp & 3) * 32 + lane, half = warp >> 2;
@@ -165,22 +182,34 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     const long long chunks = (n + CH - 1) / CH;
     const long long c_lo = chunks * rank / parts, c_hi = chunks * (rank + 1) / parts;
 
-    long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+    long long hi[4] = {0, 0, 0, 0}, mid[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
     float chk = 0.f;  // NaN once a kernel entry is
     bool failed = false;
     uint32_t par[2] = {0u, 0u};
     bool used[2] = {false, false};
     // adds the levels of accumulator set `set` to the sums
     auto take = [&](int set) {
-        float v[6][4];
+        const uint32_t at = lane_addr + set * T_SET + 4 * half;
+        auto three = [&](int l, long long(&sum)[4]) {
+            float v[3][4];
 #pragma unroll
-        for (int l = 0; l < 6; ++l) tmem_ld4(lane_addr + set * 64 + 8 * l + 4 * half, v[l]);
+            for (int i = 0; i < 3; ++i) tmem_ld4(at + 8 * (l + i), v[i]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                sum[r] += ((long long)__float2int_rn(v[0][r]) << 16) + (__float2int_rn(v[1][r]) * 256LL) +
+                          __float2int_rn(v[2][r]);
+        };
+        three(0, hi);
+        three(3, mid);
+        three(6, lo);
+        float v[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) tmem_ld4(at + T_S + 8 * i, v[i]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            hi[r] += ((long long)__float2int_rn(v[0][r]) << 16) + (__float2int_rn(v[1][r]) * 256LL) + __float2int_rn(v[2][r]);
-            lo[r] += ((long long)__float2int_rn(v[3][r]) << 16) + (__float2int_rn(v[4][r]) * 256LL) + __float2int_rn(v[5][r]);
-        }
+        for (int r = 0; r < 4; ++r) S[r] -= fmaf(v[0][r], 256.f, v[1][r]);  // (Theta's digits have the minus sign)
     };
     __syncthreads();
     if (parts > 1) {
@@ -207,13 +236,15 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
         for (int q = 0; q < CH * 8 / NT; ++q) {
             const int t = (tid >> 3) + q * (NT / 8), r = tid & 7;
             const long long j = c * CH + t;
-            long long I = 0;  // round(x 2^(47 - X)), |I| <= 2^47
+            long long I = 0;    // round(x 2^(63 - X)), |I| < 2^63
+            unsigned top = 0u;  // the leading 15 bits of |x| 2^-X
             if (j < n && r < nrhs) {
                 const long long u = __double_as_longlong(x[j * nrhs + r]);
                 const int e = (int)((u >> 52) & 0x7ff);
                 const long long mant = (u & 0xfffffffffffffLL) | 0x10000000000000LL;
-                const int sh = sx[r] - e + 6;  // X = sx[r] - 1022
-                if (e > 0 && sh < 55) I = ((mant >> (sh - 1)) + 1) >> 1;
+                const int sh = sx[r] - e - 10;  // X = sx[r] - 1022
+                if (e > 0) I = sh <= 0 ? mant << -sh : (sh < 55 ? ((mant >> (sh - 1)) + 1) >> 1 : 0LL);
+                top = (unsigned)(I >> 48);
                 if (u < 0) I = -I;
             }
             unsigned char* Bt = sm + SB + set * B_TILE;
@@ -223,6 +254,9 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
                 I = (I - dgt) >> 8;
                 *reinterpret_cast<__nv_bfloat16*>(Bt + core_off(b * 8 + r, t, CH)) = __float2bfloat16_rn((float)dgt);
             }
+            *reinterpret_cast<__nv_bfloat16*>(Bt + core_off(XD * 8 + r, t, CH)) = __float2bfloat16_rn((float)(top >> 8));
+            *reinterpret_cast<__nv_bfloat16*>(Bt + core_off(XD * 8 + 8 + r, t, CH)) =
+                __float2bfloat16_rn((float)(top & 255u));
         }
         __syncthreads();
         for (int s = 0; s < CH / SUB; ++s) {
@@ -273,11 +307,21 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
             }
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // `digits` digits of x from b on, against digit a, into the columns from `col` on
+                auto mma = [&](int a, int b, int digits, uint32_t col, uint32_t acc) {
+                    mma_f16(tmem + set * T_SET + col, smem_desc(aA + (buf * KD + a) * A_TILE, 128, 256),
+                            smem_desc(aB + set * B_TILE + b * B_GROUP + s * (SUB / 8) * 128, 128, B_GROUP), acc,
+                            idesc_bf16(8 * digits, 0, 0));
+                };
+                // a chunk's first MMAs set the columns: 16 .. 79 by digit 2, 0 .. 15 by digit 0, then S
+                const uint32_t acc = s > 0 ? 1u : 0u;
+                mma(2, 0, 8, 16, acc);
+                mma(0, 0, 2, 0, acc);
+                mma(0, 2, 6, 16, 1u);
+                mma(0, XD, 2, T_S, acc);
+                mma(1, 0, 8, 8, 1u);
 #pragma unroll
-                for (int a = 0; a < KD; ++a)
-                    mma_f16(tmem + set * 64 + 8 * a, smem_desc(aA + (buf * KD + a) * A_TILE, 128, 256),
-                            smem_desc(aB + set * B_TILE + s * (SUB / 8) * 128, 128, (CH / 8) * 128),
-                            (s > 0 || a > 0) ? 1u : 0u, idesc_bf16(48 - 16 * (a / 2), 0, 0));
+                for (int a = 3; a < KD; ++a) mma(a, 0, (10 - a) / 2 * 2, 8 * a, 1u);
                 mma_commit(bar[buf]);
             }
             // the previous chunk's last MMAs were waited for in this chunk's first two steps
@@ -308,19 +352,24 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     if (parts > 1) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            acc[(row * 8 + 4 * half + r) * 2] = nan_row ? NOT_A_NUMBER : hi[r];
-            acc[(row * 8 + 4 * half + r) * 2 + 1] = lo[r];
+            long long* at = acc + (row * 8 + 4 * half + r) * 4;
+            at[0] = nan_row ? NOT_A_NUMBER : hi[r];
+            at[1] = mid[r];
+            at[2] = lo[r];
+            at[3] = (long long)S[r];
         }
         cluster_sync_all();
         if (rank == 0) {
             for (int q = 1; q < parts; ++q) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const uint32_t at = smem_u32(acc + (row * 8 + 4 * half + r) * 2);
+                    const uint32_t at = smem_u32(acc + (row * 8 + 4 * half + r) * 4);
                     const long long h = ld_cluster_s64(at, q);
                     if (h == NOT_A_NUMBER) nan_row = true;
                     hi[r] += h;
-                    lo[r] += ld_cluster_s64(at + 8, q);
+                    mid[r] += ld_cluster_s64(at + 8, q);
+                    lo[r] += ld_cluster_s64(at + 16, q);
+                    S[r] += (float)ld_cluster_s64(at + 24, q);
                 }
             }
         }
@@ -332,10 +381,14 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
             const int r = 4 * half + r0;
             if (r >= nrhs) continue;
             // (the sums have the minus sign of Theta's digits)
-            double v = -(ldexp((double)hi[r0], -30) + ldexp((double)lo[r0], -54));
+            double v = -(ldexp((double)hi[r0], -30) + (ldexp((double)mid[r0], -54) + ldexp((double)lo[r0], -78)));
             v = ldexp(v, E + sx[r] - 1022);
             if (nan_row || sx[r] == 0x7ff) v = NAN;
-            y[i * nrhs + r] = v + diag_extra * x[i * nrhs + r];
+            v += diag_extra * x[i * nrhs + r];
+            // (S in units of 2^-22; sx 0: the right-hand side is zero)
+            if (!nan_row && sx[r] != 0x7ff && sx[r] > 0 && !(S[r0] >= least))
+                v = __longlong_as_double((long long)(MARK | (unsigned)sx[r]));
+            y[i * nrhs + r] = v;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -343,6 +396,133 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+// The marked entries of y in double-FP32: products and sums with their errors (TwoProduct, TwoSum) in FP32 pairs, x
+// as two FP32 numbers, added to FP64 every ROW_FLUSH terms.  A CTA looks through 64 rows and takes the marked ones two at a
+// time, thread = every 256th source.  Right-hand sides beyond FP32's range are scaled by a power of two.
+constexpr int ROW_TILE = 64, ROW_FLUSH = 64;
+
+template <int NU>
+__global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict__ pts, long long n, int dim, KP<float> kp,
+                                                       double diag_extra, const double* __restrict__ x,
+                                                       double* __restrict__ y, int nrhs) {
+    __shared__ unsigned mask[ROW_TILE];  // marked right-hand sides of a row
+    __shared__ int list[ROW_TILE], expo[8];
+    __shared__ int count;
+    __shared__ double red[NT / 32][16];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long row0 = blockIdx.x * (long long)ROW_TILE;
+    if (tid < ROW_TILE) mask[tid] = 0u;
+    if (tid < 8) expo[tid] = 1022;
+    if (tid == 0) count = 0;
+    __syncthreads();
+    bool any = false;
+    for (int e = tid; e < ROW_TILE * nrhs; e += NT) {
+        const int row = e / nrhs, r = e - row * nrhs;
+        if (row0 + row >= n) break;
+        const double v = y[(row0 + row) * nrhs + r];
+        if (is_marked(v)) {
+            atomicOr(&mask[row], 1u << r);
+            expo[r] = (int)(__double_as_longlong(v) & 0x7ffLL);
+            any = true;
+        }
+    }
+    if (!__syncthreads_or(any)) return;
+    if (tid < ROW_TILE && mask[tid]) list[atomicAdd(&count, 1)] = tid;
+    __syncthreads();
+    const int rows = count;
+    double up[8];  // scale of a right-hand side
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const int X = expo[r] - 1022;
+        up[r] = X > 120 || X < -100 ? ldexp(1.0, min(max(-X, -1000), 1000)) : 1.0;
+    }
+    const float2 neg1 = make_float2(-1.f, -1.f);
+    auto coord = [&](long long i, int d) { return d < dim ? (float)pts[i * dim + d] : 0.f; };
+    for (int p = 0; p < rows; p += 2) {
+        const int ra = list[p], rb = list[min(p + 1, rows - 1)];
+        const long long ia = row0 + ra, ib = row0 + rb;
+        const float2 rx = make_float2(coord(ia, 0), coord(ib, 0)), ry = make_float2(coord(ia, 1), coord(ib, 1)),
+                     rz = make_float2(coord(ia, 2), coord(ib, 2));
+        float2 S[2][4], lo[2][4];
+        double acc[2][8];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
+                acc[q][2 * r] = acc[q][2 * r + 1] = 0.0;
+            }
+        auto flush = [&]() {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    acc[q][2 * r] += (double)S[q][r].x + (double)lo[q][r].x;
+                    acc[q][2 * r + 1] += (double)S[q][r].y + (double)lo[q][r].y;
+                    S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
+                }
+        };
+        int terms = 0;
+        for (long long j = tid; j < n; j += NT) {
+            const float cx = coord(j, 0), cy = coord(j, 1);
+            const float2 dx = __fadd2_rn(rx, make_float2(-cx, -cx)), dy = __fadd2_rn(ry, make_float2(-cy, -cy));
+            float2 d2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+            if (dim > 2) {
+                const float cz = coord(j, 2);
+                const float2 dz = __fadd2_rn(rz, make_float2(-cz, -cz));
+                d2 = __ffma2_rn(dz, dz, d2);
+            }
+            const float2 dist = sqrt_f2(d2);
+            const float ka = matern_nu<NU>(kp, dist.x), kb = matern_nu<NU>(kp, dist.y);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float2 xh = make_float2(0.f, 0.f), xl = xh;
+                if (2 * r < nrhs) split_f64(x[j * nrhs + 2 * r] * up[2 * r], xh.x, xl.x);
+                if (2 * r + 1 < nrhs) split_f64(x[j * nrhs + 2 * r + 1] * up[2 * r + 1], xh.y, xl.y);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float2 k = q == 0 ? make_float2(ka, ka) : make_float2(kb, kb);
+                    const float2 pr = __fmul2_rn(k, xh);
+                    const float2 pe = __ffma2_rn(k, xl, __ffma2_rn(k, xh, __fmul2_rn(pr, neg1)));
+                    const float2 s = __fadd2_rn(S[q][r], pr);
+                    const float2 nb = __ffma2_rn(s, neg1, S[q][r]);                  // -(s - S)
+                    const float2 ea = __ffma2_rn(__fadd2_rn(s, nb), neg1, S[q][r]);  // S - (s - (s - S))
+                    lo[q][r] = __fadd2_rn(lo[q][r], __fadd2_rn(__fadd2_rn(ea, __fadd2_rn(pr, nb)), pe));
+                    S[q][r] = s;
+                }
+            }
+            if (++terms == ROW_FLUSH) {
+                flush();
+                terms = 0;
+            }
+        }
+        flush();
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                double a = acc[q][r];
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+                if (lane == 0) red[warp][8 * q + r] = a;
+            }
+        __syncthreads();
+        if (tid < 16) {
+            const int row = tid < 8 ? ra : rb, r = tid & 7;
+            const long long i = row0 + row;
+            if (mask[row] >> r & 1u) {
+                double a = red[0][tid];
+#pragma unroll
+                for (int w = 1; w < NT / 32; ++w) a += red[w][tid];
+                const int X = expo[r] - 1022;
+                const double s = X > 120 || X < -100 ? ldexp(1.0, min(max(-X, -1000), 1000)) : 1.0;
+                y[i * nrhs + r] = a / s + diag_extra * x[i * nrhs + r];
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -381,7 +561,11 @@ static sic_status launch_matvec_tc(sic_handle* h, const double* pts, long long n
     cfg.attrs = at;
     cfg.numAttrs = parts > 1 ? 1 : 0;
     SIC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, pts, n, (int)kp->dim, make_kp<float>(*kp), ldexpf(1.f, -E), E,
-                                    kp->nugget + shift, x, y, nrhs, parts, h->d_status));
+                                    kp->nugget + shift, x, y, nrhs, parts,
+                                    (float)(sqrt((double)n) * ldexp(1.0, 22 - S_BITS)), h->d_status));
+    k_matvec_rows<NU><<<(unsigned)((n + ROW_TILE - 1) / ROW_TILE), NT, 0, s>>>(
+        pts, n, kp->dim, make_kp<float>(*kp), kp->nugget + shift, x, y, nrhs);
+    SIC_CUDA_TRY(cudaGetLastError());
     return SIC_OK;
 }
 

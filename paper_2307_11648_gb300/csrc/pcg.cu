@@ -31,24 +31,6 @@ constexpr int RED_TILE = 4096;
 // with a thread per row, 5.2 ms now (two: 8.0 and 5.2).
 constexpr int MVF_WARPS = 8, MVF_ROWS = 64, MVF_FLUSH = 32;  // (tiles between FP64 additions)
 
-// v as hi + lo, hi = v rounded to FP32, lo = the rest rounded to FP32: by integer operations where 2^-99 <= |v| <
-// 2^115 (conversions run on the FP64 pipe), else by conversions
-__device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-    const int e = (int)((u >> 52) & 0x7ff);
-    if (e > 923 && e < 1138) {
-        const unsigned long long mant = (u & 0xfffffffffffffULL) | 0x10000000000000ULL;
-        const unsigned h = (unsigned)((mant + (1ULL << 28)) >> 29);  // 24 bits, or 2^24
-        const int l = (int)(mant - ((unsigned long long)h << 29));  // |l| <= 2^28
-        const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
-        hi = __fmul_rn(__uint2float_rn(h), __uint_as_float(sg | ((unsigned)(e - 919) << 23)));
-        lo = __fmul_rn(__fmul_rn(__int2float_rn(l), __uint_as_float(sg | ((unsigned)(e - 884) << 23))), 0x1p-64f);
-    } else {
-        hi = (float)v;
-        lo = (float)(v - (double)hi);
-    }
-}
-
 template <int NR>
 __global__ void __launch_bounds__(32 * MVF_WARPS, 2) k_matvec_f32(const double* __restrict__ pts, long long n, int dim,
                                                                   KP<float> kp, double diag_extra,

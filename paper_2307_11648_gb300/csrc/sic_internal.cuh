@@ -171,6 +171,24 @@ __device__ __forceinline__ void f64_split(double x, float& hi, float& lo) {
     lo = e >= 949u ? __fmul_rn(m, __uint_as_float(sg | ((e - 948u) << 23))) : 0.f;
 }
 
+// v as hi + lo, hi = v rounded to FP32, lo = the rest rounded to FP32: by integer operations where 2^-99 <= |v| <
+// 2^115 (conversions run on the FP64 pipe), else by conversions
+__device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)((u >> 52) & 0x7ff);
+    if (e > 923 && e < 1138) {
+        const unsigned long long mant = (u & 0xfffffffffffffULL) | 0x10000000000000ULL;
+        const unsigned h = (unsigned)((mant + (1ULL << 28)) >> 29);  // 24 bits, or 2^24
+        const int l = (int)(mant - ((unsigned long long)h << 29));  // |l| <= 2^28
+        const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
+        hi = __fmul_rn(__uint2float_rn(h), __uint_as_float(sg | ((unsigned)(e - 919) << 23)));
+        lo = __fmul_rn(__fmul_rn(__int2float_rn(l), __uint_as_float(sg | ((unsigned)(e - 884) << 23))), 0x1p-64f);
+    } else {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    }
+}
+
 // exp(x), -700 <= x <= 700: table-driven reduction after Tang (ACM TOMS 15(2), 1989).  With
 // k = round(256 x / ln 2) = 256 q + j (from an FP32 product: off by at most one from the
 // nearest integer, which only widens |r| to ~1.6e-3), x = k ln2/256 + r and
