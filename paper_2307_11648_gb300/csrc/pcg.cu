@@ -5,7 +5,7 @@
 // forming Theta.  The kernel entries are FP32 (a fixed, symmetric rounding of Theta: K(|x_i - x_j|) is evaluated
 // identically for (i, j) and (j, i)); x is carried as an unevaluated sum of two FP32 numbers (hi + lo) and the
 // products are summed as a double-FP32 pair with the error-free transformations TwoProduct (by fma) and
-// TwoSum (Knuth), 1024 terms at a time, then in FP64 -- so the product is accurate to ~1e-13 of sum |K x| and
+// TwoSum (Knuth), 256 terms at a time, then in FP64 -- so the product is accurate to a few 1e-15 of sum |K x| (typically) and
 // CG can reach small residuals.  k_matvec_f64 is FP64 throughout (reference mode; the kernel entries by the fill's table-driven exp
 // and Newton square root, about 2 ulp).  The diagonal adds the nugget and the shift in FP64.
 // The CG vector updates and dot products are fused kernels with fixed-order reductions
@@ -29,7 +29,8 @@ constexpr int RED_TILE = 4096;
 // ten warps.  Bound: FP32 lanes (11 operations per source, row and right-hand side, about 22 per entry).
 // N = 50,001, one right-hand side: 6.0 ms
 // with a thread per row, 5.2 ms now (two: 8.0 and 5.2).
-constexpr int MVF_WARPS = 8, MVF_ROWS = 64, MVF_FLUSH = 32;  // (tiles between FP64 additions)
+constexpr int MVF_WARPS = 8, MVF_ROWS = 64;
+constexpr int MVF_FLUSH = 8;  // tiles between FP64 additions: 256 terms (1024 left three times the error)
 
 template <int NR>
 __global__ void __launch_bounds__(32 * MVF_WARPS, 2) k_matvec_f32(const double* __restrict__ pts, long long n, int dim,

@@ -81,3 +81,28 @@ def test_the_recomputed_rows_use_the_same_theta(env):  # noqa: F811
         x[299, 1] = 1e18
         y = _product(env, pts, kp, x)
         assert np.array_equal(y[:299, 0], y[:299, 1]) and y[299, 1] == 1e18 * np.float64(np.float32(1.3))
+
+
+@pytest.mark.parametrize("dim,nu_x2,ell", [(2, 3, 0.02), (3, 5, 0.2), (2, 1, 0.05)])
+def test_one_right_hand_side_of_many_points(env, dim, nu_x2, ell):  # noqa: F811
+    """The CUDA-core sums: the errors of m terms' double-FP32 sum of random signs come to about sqrt(m) 2^-52 of the sum of
+    their magnitudes, 2^-48 on average over the rows at m = 256."""
+    torch, sic, _, h = env
+    n = 12800
+    kp = sic.kernel(dim, nu_x2, ell, 1.0, 0.0)
+    pts = torch.from_numpy(synthetic.points(n, dim, 8)).cuda()
+    K = torch.zeros(n, n, dtype=torch.float32, device="cuda")
+    y8 = torch.zeros(n, 8, dtype=torch.float64, device="cuda")
+    rows = slice(0, n, 16)
+    for j in range(0, n, 8):
+        e = torch.zeros(n, 8, dtype=torch.float64, device="cuda")
+        e[torch.arange(j, j + 8), torch.arange(8)] = 1.0
+        sic.matern_matvec(h, pts, kp, 0.0, sic.SIC_FP32_MIXED, e, y8)
+        K[:, j:j + 8] = y8.float()
+    x = torch.from_numpy(synthetic.normal(3, n)).cuda()
+    y = torch.zeros_like(x)
+    sic.matern_matvec(h, pts, kp, 0.0, sic.SIC_FP32_MIXED, x, y)
+    h.sync()
+    Ks, xl = K[rows].cpu().numpy().astype(np.longdouble), x.cpu().numpy().astype(np.longdouble)
+    err = np.abs(y[rows].cpu().numpy().astype(np.longdouble) - Ks @ xl) / (Ks @ np.abs(xl))
+    assert err.mean() <= 2.0 ** -48 and err.max() <= 2.0 ** -43
