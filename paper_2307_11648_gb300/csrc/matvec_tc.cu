@@ -29,6 +29,7 @@
 // number of right-hand sides.  N = 50,001 with 8 of them: 16.6 ms with double-FP32 sums on the CUDA cores, 6.8 ms
 // now (N = 4096: 1.04 -> 0.086 ms); with sqrtf and a run-time smoothness, whose branches keep the evaluations from
 // overlapping, 11.2 ms.
+#include "matvec_f32.cuh"
 #include "tc_common.cuh"
 
 namespace {
@@ -399,27 +400,29 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     }
 }
 
-// The marked entries of y in double-FP32: products and sums with their errors (TwoProduct, TwoSum) in FP32 pairs, x
-// as two FP32 numbers, added to FP64 every ROW_FLUSH terms.  A CTA looks through 64 rows and takes the marked ones two at a
-// time, thread = every 256th source.  Right-hand sides beyond FP32's range are scaled by a power of two.
-constexpr int ROW_TILE = 64, ROW_FLUSH = 64;
+// The marked entries of y in double-FP32 (matvec_f32.cuh), a CTA per 64 rows.  Up to ROW_FEW marked rows go two at a time,
+// thread = every 256th source (a tile's chain over all sources takes far longer than that); more of them by
+// the whole tile.  Right-hand sides beyond FP32's range are scaled by a power of two.
+constexpr int ROW_FEW = 6;
 
 template <int NU>
 __global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict__ pts, long long n, int dim, KP<float> kp,
                                                        double diag_extra, const double* __restrict__ x,
                                                        double* __restrict__ y, int nrhs) {
-    __shared__ unsigned mask[ROW_TILE];  // marked right-hand sides of a row
-    __shared__ int list[ROW_TILE], expo[8];
+    static_assert(NT == 32 * MVF_WARPS, "the tile's threads");
+    __shared__ MvfSmem<8> sm;
+    __shared__ unsigned mask[MVF_ROWS];  // marked right-hand sides of a row
+    __shared__ int list[MVF_ROWS], expo[8];
     __shared__ int count;
-    __shared__ double red[NT / 32][16];
+    __shared__ double up[8];  // scale of a right-hand side
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long row0 = blockIdx.x * (long long)ROW_TILE;
-    if (tid < ROW_TILE) mask[tid] = 0u;
+    const long long row0 = blockIdx.x * (long long)MVF_ROWS;
+    if (tid < MVF_ROWS) mask[tid] = 0u;
     if (tid < 8) expo[tid] = 1022;
     if (tid == 0) count = 0;
     __syncthreads();
     bool any = false;
-    for (int e = tid; e < ROW_TILE * nrhs; e += NT) {
+    for (int e = tid; e < MVF_ROWS * nrhs; e += NT) {
         const int row = e / nrhs, r = e - row * nrhs;
         if (row0 + row >= n) break;
         const double v = y[(row0 + row) * nrhs + r];
@@ -430,16 +433,26 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict_
         }
     }
     if (!__syncthreads_or(any)) return;
-    if (tid < ROW_TILE && mask[tid]) list[atomicAdd(&count, 1)] = tid;
+    if (tid < MVF_ROWS && mask[tid]) list[atomicAdd(&count, 1)] = tid;
+    if (tid < 8) {
+        const int X = expo[tid] - 1022;
+        up[tid] = X > 120 || X < -100 ? ldexp(1.0, min(max(-X, -1000), 1000)) : 1.0;
+    }
     __syncthreads();
     const int rows = count;
-    double up[8];  // scale of a right-hand side
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int X = expo[r] - 1022;
-        up[r] = X > 120 || X < -100 ? ldexp(1.0, min(max(-X, -1000), 1000)) : 1.0;
+    auto entry = [&](float2 d2) {
+        const float2 r = sqrt_f2(d2);
+        return make_float2(matern_nu<NU>(kp, r.x), matern_nu<NU>(kp, r.y));
+    };
+    auto put = [&](int row, int r, double sum) {
+        const long long i = row0 + row;
+        if (mask[row] >> r & 1u) y[i * nrhs + r] = sum / up[r] + diag_extra * x[i * nrhs + r];
+    };
+    if (rows > ROW_FEW) {
+        mvf_tile<8>(sm, pts, n, dim, x, nrhs, row0, entry, [&](int r) { return up[r]; });
+        for (int e = tid; e < MVF_ROWS * 8; e += NT) put(e >> 3, e & 7, sm.sum(e >> 3, e & 7));
+        return;
     }
-    const float2 neg1 = make_float2(-1.f, -1.f);
     auto coord = [&](long long i, int d) { return d < dim ? (float)pts[i * dim + d] : 0.f; };
     for (int p = 0; p < rows; p += 2) {
         const int ra = list[p], rb = list[min(p + 1, rows - 1)];
@@ -455,51 +468,26 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict_
                 S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
                 acc[q][2 * r] = acc[q][2 * r + 1] = 0.0;
             }
-        auto flush = [&]() {
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    acc[q][2 * r] += (double)S[q][r].x + (double)lo[q][r].x;
-                    acc[q][2 * r + 1] += (double)S[q][r].y + (double)lo[q][r].y;
-                    S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
-                }
-        };
         int terms = 0;
         for (long long j = tid; j < n; j += NT) {
-            const float cx = coord(j, 0), cy = coord(j, 1);
-            const float2 dx = __fadd2_rn(rx, make_float2(-cx, -cx)), dy = __fadd2_rn(ry, make_float2(-cy, -cy));
-            float2 d2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-            if (dim > 2) {
-                const float cz = coord(j, 2);
-                const float2 dz = __fadd2_rn(rz, make_float2(-cz, -cz));
-                d2 = __ffma2_rn(dz, dz, d2);
-            }
-            const float2 dist = sqrt_f2(d2);
-            const float ka = matern_nu<NU>(kp, dist.x), kb = matern_nu<NU>(kp, dist.y);
+            const float cx = coord(j, 0), cy = coord(j, 1), cz = coord(j, 2);
+            const float2 dx = __fadd2_rn(rx, make_float2(-cx, -cx)), dy = __fadd2_rn(ry, make_float2(-cy, -cy)),
+                         dz = __fadd2_rn(rz, make_float2(-cz, -cz));
+            const float2 k = entry(__ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy))));
+            float2 xh[4], xl[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                float2 xh = make_float2(0.f, 0.f), xl = xh;
-                if (2 * r < nrhs) split_f64(x[j * nrhs + 2 * r] * up[2 * r], xh.x, xl.x);
-                if (2 * r + 1 < nrhs) split_f64(x[j * nrhs + 2 * r + 1] * up[2 * r + 1], xh.y, xl.y);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const float2 k = q == 0 ? make_float2(ka, ka) : make_float2(kb, kb);
-                    const float2 pr = __fmul2_rn(k, xh);
-                    const float2 pe = __ffma2_rn(k, xl, __ffma2_rn(k, xh, __fmul2_rn(pr, neg1)));
-                    const float2 s = __fadd2_rn(S[q][r], pr);
-                    const float2 nb = __ffma2_rn(s, neg1, S[q][r]);                  // -(s - S)
-                    const float2 ea = __ffma2_rn(__fadd2_rn(s, nb), neg1, S[q][r]);  // S - (s - (s - S))
-                    lo[q][r] = __fadd2_rn(lo[q][r], __fadd2_rn(__fadd2_rn(ea, __fadd2_rn(pr, nb)), pe));
-                    S[q][r] = s;
-                }
+                xh[r] = xl[r] = make_float2(0.f, 0.f);
+                if (2 * r < nrhs) split_f64(x[j * nrhs + 2 * r] * up[2 * r], xh[r].x, xl[r].x);
+                if (2 * r + 1 < nrhs) split_f64(x[j * nrhs + 2 * r + 1] * up[2 * r + 1], xh[r].y, xl[r].y);
             }
-            if (++terms == ROW_FLUSH) {
-                flush();
+            mvf_add<4>(k.x, k.y, xh, xl, S, lo);
+            if (++terms == 32 * MVF_FLUSH) {
+                mvf_flush<4>(S, lo, acc);
                 terms = 0;
             }
         }
-        flush();
+        mvf_flush<4>(S, lo, acc);
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -507,21 +495,10 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict_
                 double a = acc[q][r];
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                if (lane == 0) red[warp][8 * q + r] = a;
+                if (lane == 0) sm.acc[warp][r][q] = a;
             }
         __syncthreads();
-        if (tid < 16) {
-            const int row = tid < 8 ? ra : rb, r = tid & 7;
-            const long long i = row0 + row;
-            if (mask[row] >> r & 1u) {
-                double a = red[0][tid];
-#pragma unroll
-                for (int w = 1; w < NT / 32; ++w) a += red[w][tid];
-                const int X = expo[r] - 1022;
-                const double s = X > 120 || X < -100 ? ldexp(1.0, min(max(-X, -1000), 1000)) : 1.0;
-                y[i * nrhs + r] = a / s + diag_extra * x[i * nrhs + r];
-            }
-        }
+        if (tid < 16) put(tid < 8 ? ra : rb, tid & 7, sm.sum(tid >> 3, tid & 7));
         __syncthreads();
     }
 }
@@ -563,7 +540,7 @@ static sic_status launch_matvec_tc(sic_handle* h, const double* pts, long long n
     SIC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, pts, n, (int)kp->dim, make_kp<float>(*kp), ldexpf(1.f, -E), E,
                                     kp->nugget + shift, x, y, nrhs, parts,
                                     (float)(sqrt((double)n) * ldexp(1.0, 22 - S_BITS)), h->d_status));
-    k_matvec_rows<NU><<<(unsigned)((n + ROW_TILE - 1) / ROW_TILE), NT, 0, s>>>(
+    k_matvec_rows<NU><<<(unsigned)((n + MVF_ROWS - 1) / MVF_ROWS), NT, 0, s>>>(
         pts, n, kp->dim, make_kp<float>(*kp), kp->nugget + shift, x, y, nrhs);
     SIC_CUDA_TRY(cudaGetLastError());
     return SIC_OK;

@@ -15,129 +15,29 @@
 
 #include <vector>
 
-#include "sic_internal.cuh"
+#include "matvec_f32.cuh"
 
 namespace {
 
 constexpr int MV_NT = 128;   // FP64: target rows per CTA
-constexpr int MV_TILE = 256; // source points per shared-memory tile
 constexpr int RED_TILE = 4096;
 
-// A CTA of 8 warps takes 64 target rows (two per lane, so that a source's values are read once for both and the
-// kernel evaluation runs in packed FP32 pairs); the warps share the staged source tile, 32 sources each, and
-// their sums are added in order at the end.  With one thread per row over all sources, N = 50,001 left an SM
-// ten warps.  Bound: FP32 lanes (11 operations per source, row and right-hand side, about 22 per entry).
-// N = 50,001, one right-hand side: 6.0 ms
-// with a thread per row, 5.2 ms now (two: 8.0 and 5.2).
-constexpr int MVF_WARPS = 8, MVF_ROWS = 64;
-constexpr int MVF_FLUSH = 8;  // tiles between FP64 additions: 256 terms (1024 left three times the error)
-
+// One or two right-hand sides (matvec_f32.cuh)
 template <int NR>
 __global__ void __launch_bounds__(32 * MVF_WARPS, 2) k_matvec_f32(const double* __restrict__ pts, long long n, int dim,
                                                                   KP<float> kp, double diag_extra,
                                                                   const double* __restrict__ x, double* __restrict__ y,
                                                                   int nrhs) {
-    constexpr int NP = (NR + 1) / 2;  // right-hand sides in pairs
-    constexpr int NT = 32 * MVF_WARPS;
-    __shared__ union Sm {
-        struct {
-            float4 c[MV_TILE];        // coordinates
-            float2 h[MV_TILE][NP];    // high parts of x
-            float2 l[MV_TILE][NP];    // low parts
-        } t;
-        double acc[MVF_WARPS][2 * NP][MVF_ROWS];
-    } sm;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long i0 = blockIdx.x * (long long)MVF_ROWS + lane, i1 = i0 + 32;
-    float2 rx = make_float2(0.f, 0.f), ry = rx, rz = rx;  // the lane's two rows
-    auto coord = [&](long long i, int d) { return i < n && d < dim ? (float)pts[i * dim + d] : 0.f; };
-    rx = make_float2(coord(i0, 0), coord(i1, 0));
-    ry = make_float2(coord(i0, 1), coord(i1, 1));
-    rz = make_float2(coord(i0, 2), coord(i1, 2));
-    const float2 neg1 = make_float2(-1.f, -1.f);
-    float2 S[2][NP], lo[2][NP];
-    double acc[2][2 * NP];
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int r = 0; r < NP; ++r) {
-            S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
-            acc[q][2 * r] = acc[q][2 * r + 1] = 0.0;
-        }
-    auto flush = [&]() {
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int r = 0; r < NP; ++r) {
-                acc[q][2 * r] += (double)S[q][r].x + (double)lo[q][r].x;
-                acc[q][2 * r + 1] += (double)S[q][r].y + (double)lo[q][r].y;
-                S[q][r] = lo[q][r] = make_float2(0.f, 0.f);
-            }
-    };
-    int tiles = 0;
-    for (long long j0 = 0; j0 < n; j0 += MV_TILE) {
-        __syncthreads();
-        for (int t = tid; t < MV_TILE; t += NT) {
-            const long long j = j0 + t;
-            sm.t.c[t] = make_float4(coord(j, 0), coord(j, 1), coord(j, 2), 0.f);
-#pragma unroll
-            for (int r = 0; r < NP; ++r) {
-                float2 h = make_float2(0.f, 0.f), l = h;
-                if (j < n) {
-                    if (2 * r < nrhs) split_f64(x[j * nrhs + 2 * r], h.x, l.x);
-                    if (2 * r + 1 < nrhs) split_f64(x[j * nrhs + 2 * r + 1], h.y, l.y);
-                }
-                sm.t.h[t][r] = h;
-                sm.t.l[t][r] = l;
-            }
-        }
-        __syncthreads();
-        const int t0 = warp * (MV_TILE / MVF_WARPS);
-        const int t1 = (int)min((long long)(t0 + MV_TILE / MVF_WARPS), n - j0);
-        for (int t = t0; t < t1; ++t) {
-            const float4 c = sm.t.c[t];
-            const float2 dx = __fadd2_rn(rx, make_float2(-c.x, -c.x)), dy = __fadd2_rn(ry, make_float2(-c.y, -c.y)),
-                         dz = __fadd2_rn(rz, make_float2(-c.z, -c.z));
-            const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
-            const float k0 = matern<float>(kp, sqrtf(d2.x)), k1 = matern<float>(kp, sqrtf(d2.y));
-#pragma unroll
-            for (int r = 0; r < NP; ++r) {
-                const float2 xh = sm.t.h[t][r], xl = sm.t.l[t][r];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const float2 k = q == 0 ? make_float2(k0, k0) : make_float2(k1, k1);
-                    // TwoProduct, TwoSum (packed operations: lane-wise the scalar roundings)
-                    const float2 p = __fmul2_rn(k, xh);
-                    const float2 pe = __ffma2_rn(k, xl, __ffma2_rn(k, xh, __fmul2_rn(p, neg1)));
-                    const float2 s = __fadd2_rn(S[q][r], p);
-                    const float2 nb = __ffma2_rn(s, neg1, S[q][r]);                       // -(s - S)
-                    const float2 ea = __ffma2_rn(__fadd2_rn(s, nb), neg1, S[q][r]);       // S - (s - (s - S))
-                    lo[q][r] = __fadd2_rn(lo[q][r], __fadd2_rn(__fadd2_rn(ea, __fadd2_rn(p, nb)), pe));
-                    S[q][r] = s;
-                }
-            }
-        }
-        if (++tiles == MVF_FLUSH) {
-            flush();
-            tiles = 0;
-        }
-    }
-    flush();
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 2 * NP; ++r) {
-        sm.acc[warp][r][lane] = acc[0][r];
-        sm.acc[warp][r][lane + 32] = acc[1][r];
-    }
-    __syncthreads();
-    for (int e = tid; e < MVF_ROWS * nrhs; e += NT) {
+    __shared__ MvfSmem<NR> sm;
+    const long long row0 = blockIdx.x * (long long)MVF_ROWS;
+    mvf_tile<NR>(
+        sm, pts, n, dim, x, nrhs, row0,
+        [&](float2 d2) { return make_float2(matern<float>(kp, sqrtf(d2.x)), matern<float>(kp, sqrtf(d2.y))); },
+        [](int) { return 1.0; });
+    for (int e = threadIdx.x; e < MVF_ROWS * nrhs; e += 32 * MVF_WARPS) {
         const int row = e / nrhs, r = e - row * nrhs;
-        const long long i = blockIdx.x * (long long)MVF_ROWS + row;
-        if (i >= n) continue;
-        double a = sm.acc[0][r][row];
-#pragma unroll
-        for (int w = 1; w < MVF_WARPS; ++w) a += sm.acc[w][r][row];
-        y[i * nrhs + r] = a + diag_extra * x[i * nrhs + r];
+        const long long i = row0 + row;
+        if (i < n) y[i * nrhs + r] = sm.sum(row, r) + diag_extra * x[i * nrhs + r];
     }
 }
 
