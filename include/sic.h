@@ -465,9 +465,12 @@ sic_status sic_apply_factor(sic_handle* h, int64_t n, const int64_t* col_ptr, co
 
 /* y = (Theta + shift I) x without forming Theta (O(n^2) kernel evaluations), x, y
  * n x nrhs row-major FP64, 1 <= nrhs <= 8.  SIC_FP32_MIXED evaluates the kernel entries
- * in FP32 (a fixed symmetric rounding of Theta) and sums the products exactly from BF16
- * digits of the entries and of x (one or two right-hand sides at n >= 12288: with double-FP32
- * compensated arithmetic, x split into two FP32 parts, tiles added in FP64); SIC_FP64
+ * in FP32 (a fixed symmetric rounding of Theta).  Row i of the product is within about 1e-14 of
+ * its own sum_j |Theta_ij x_j| (typically 5e-15 or less), whatever the range of x: the products are
+ * summed from 8-bit digits of the entries and of x, exactly down to 2^-64 of the largest x and of
+ * the variance; rows too small for that, and all of one or two right-hand sides at n >= 12288,
+ * are summed with double-FP32 compensated arithmetic (x split into two FP32 parts, FP64 additions
+ * every 256 terms; FP32's range bounds |x| there at n >= 12288).  SIC_FP64
  * is FP64 throughout (reference for small n).  x and y must not overlap. */
 sic_status sic_matern_matvec(sic_handle* h, const double* pts, int64_t n, const sic_kernel* kp, double shift,
                              sic_precision prec, const double* x, double* y, int32_t nrhs, void* stream);

@@ -165,9 +165,10 @@ sic_status matvec_any(sic_handle* h, cudaStream_t s, const double* pts, long lon
         else matvec_f64<8>(s, pts, n, dim, kp, shift, x, y, nrhs);
         return SIC_OK;
     }
-    // The tensor-core kernel's time does not depend on the right-hand sides (N = 50,001: 6.6 ms for 3, 6.8 for 8),
-    // this one's does (5.2 ms for 1 or 2); below 2^14 rows the former also spreads a row tile over more CTAs
-    // (N = 8192, one right-hand side: 0.21 against 0.27 ms; N = 16,384: 0.78 against 0.68 ms).
+    // The tensor-core kernel's time does not depend on the right-hand sides (N = 50,001: 7.8 ms for 3, 8.0 for 8),
+    // this one's does (5.2 ms for 1 or 2); at few rows the former also spreads a row tile over more CTAs (one right-hand
+    // side: N = 4096 0.116 against 0.138 ms, 8192 0.260 against 0.268, 10,000 0.476 against 0.417) and takes any
+    // scale of x.
     if (nrhs > 2 || n < 12288) return matvec_tc(h, pts, n, kp, shift, x, y, nrhs, s);
     k_matvec_f32<2><<<(unsigned)((n + MVF_ROWS - 1) / MVF_ROWS), 32 * MVF_WARPS, 0, s>>>(
         pts, n, dim, make_kp<float>(*kp), kp->nugget + shift, x, y, nrhs);

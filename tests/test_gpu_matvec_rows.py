@@ -106,3 +106,26 @@ def test_one_right_hand_side_of_many_points(env, dim, nu_x2, ell):  # noqa: F811
     Ks, xl = K[rows].cpu().numpy().astype(np.longdouble), x.cpu().numpy().astype(np.longdouble)
     err = np.abs(y[rows].cpu().numpy().astype(np.longdouble) - Ks @ xl) / (Ks @ np.abs(xl))
     assert err.mean() <= 2.0 ** -48 and err.max() <= 2.0 ** -43
+
+
+def test_sparse_right_hand_sides_of_many_points(env):  # noqa: F811
+    """From 2048 points on no digits are formed for these; zeros, a unit vector, scales beyond FP32."""
+    torch, sic, _, h = env
+    n = 2100
+    kp = sic.kernel(2, 3, 0.1, 0.7, 0.0)
+    pts = synthetic.points(n, 2, 8)
+    at = np.arange(0, n, 300)
+    K = np.zeros((n, len(at)))
+    for j in range(0, len(at), 8):
+        e = np.zeros((n, min(8, len(at) - j)))
+        e[at[j:j + 8], np.arange(e.shape[1])] = 1.0
+        K[:, j:j + 8] = _product(env, pts, kp, e)
+    x = np.zeros((n, 4))
+    x[at[3], 1] = 1.0
+    x[at, 2] = 1e-210 * synthetic.normal(3, len(at))
+    x[at, 3] = 1e210 * synthetic.normal(4, len(at))
+    y = _product(env, pts, kp, x)
+    L = np.longdouble
+    ref, S = K.astype(L) @ x[at].astype(L), K.astype(L) @ np.abs(x[at]).astype(L)
+    assert np.all(y[:, 0] == 0.0) and np.array_equal(y[:, 1], K[:, 3])
+    assert np.all(np.abs(y.astype(L) - ref) <= 2.0 ** -41 * S)
