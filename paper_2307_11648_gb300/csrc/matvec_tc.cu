@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int row = (warp & 3) * 32 + lane, half = warp >> 2;
-    int* sx = reinterpret_cast<int*>(sm + SX);  // [0..7] exponents, [8] non-finite source coordinate
+    int* sx = reinterpret_cast<int*>(sm + SX);  // [0..7] exponents, [9] whether digits are formed
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + SBAR);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + SBAR + 16);
     const uint32_t bar[2] = {smem_u32(bars), smem_u32(bars + 1)};
@@ -244,7 +244,6 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
             const int d = e / CH, t = e % CH;
             const long long j = c * CH + t;
             const float v = (j < n && d < dim) ? (float)pts[j * dim + d] : 0.f;
-            if (!(fabsf(v) < INFINITY)) sx[8] = 1;
             nc[d * CH + t] = -v;
         }
 #pragma unroll
@@ -354,9 +353,9 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_tc(const double* __restrict__ 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!failed && c_hi > c_lo && sx[9]) take((int)((c_hi - 1 - c_lo) & 1));
     if (failed && tid == 0) record_error(st, SIC_ERR_TIMEOUT, blockIdx.x);
-    // a non-finite kernel entry in either half of the row, or a non-finite source: the row's result is NaN
+    // a kernel entry that is not a number in either half of the row: the row's result is NaN
     int* flag = reinterpret_cast<int*>(sm + SC);
-    if (half == 0) flag[row] = sx[8];
+    if (half == 0) flag[row] = 0;
     __syncthreads();
     if (!(fabsf(chk) < INFINITY)) flag[row] = 1;
     __syncthreads();

@@ -129,3 +129,19 @@ def test_sparse_right_hand_sides_of_many_points(env):  # noqa: F811
     ref, S = K.astype(L) @ x[at].astype(L), K.astype(L) @ np.abs(x[at]).astype(L)
     assert np.all(y[:, 0] == 0.0) and np.array_equal(y[:, 1], K[:, 3])
     assert np.all(np.abs(y.astype(L) - ref) <= 2.0 ** -41 * S)
+
+
+def test_a_point_at_infinity(env):  # noqa: F811
+    """The exponential kernel is zero at infinite distance: such a point leaves the other rows as they are without it."""
+    torch, sic, _, h = env
+    kp = sic.kernel(2, 1, 0.2, 1.0, 1e-4)
+    pts = synthetic.points(300, 2, 8)
+    x = synthetic.normal(3, 900).reshape(300, 3)
+    x[5] *= 1e-2
+    pts[5, 0] = np.inf
+    y = _product(env, pts, kp, x)
+    x[5] = 0.0
+    pts[5, 0] = 0.5
+    ref = _product(env, pts, kp, x)
+    rest = np.arange(300) != 5
+    assert np.array_equal(y[rest], ref[rest]) and np.all(np.isnan(y[5]))
