@@ -607,6 +607,10 @@ sic_status sic_selftest_fixed_point(sic_handle* h, const double* pa, const doubl
 sic_status sic_selftest_matern_df(sic_handle* h, const sic_kernel* kp, const double* pa, const double* pb, int64_t n,
                                   double* out, void* stream);
 
+/* The FP32 square root of the kernel-matrix product (not part of the paper) on n inputs x[i] >= 0:
+ * root[i] by its own fused operations, ref[i] by the library's sqrtf.  [device], n floats each. */
+sic_status sic_selftest_sqrt_f32(sic_handle* h, const float* x, int64_t n, float* root, float* ref, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -87,11 +87,11 @@ __device__ __forceinline__ long long ld_cluster_s64(uint32_t addr, uint32_t rank
     return v;
 }
 
-// The correctly rounded square roots of a pair (sqrtf without its special-case branches, so that the evaluations
-// overlap): from the hardware's reciprocal square root y, g = x y and h = y / 2 by one coupled Newton step, then the
-// residual step g + h (x - g^2) with fused operations (Markstein, IBM J. Res. Dev. 34 (1990)).  Checked over
-// every significand with y off by up to 2.5 ulp.  Below 2^-100 (distances that leave every kernel at its value at 0)
-// the last bits may differ; infinity stays infinite.
+// The square roots of a pair by fused operations after Markstein (IBM J. Res. Dev. 34 (1990)), without branches, so that
+// the evaluations overlap.  From an approximate reciprocal root y: g = x y and h = y / 2, both brought on by their
+// common error e = 1/2 - g h (g += g e, h += h e), then g += h (x - g^2) with the residual exact: correctly rounded,
+// equal to sqrtf for every significand (sic_selftest_sqrt_f32).  Below 2^-100 (distances that leave every kernel at
+// its value at 0) the last bits may differ; infinity stays infinite.
 __device__ __forceinline__ float2 sqrt_f2(float2 x) {
     float ya, yb;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ya) : "f"(fmaxf(x.x, 1.2e-38f)));
@@ -517,6 +517,32 @@ __global__ void __launch_bounds__(NT, 2) k_matvec_rows(const double* __restrict_
 }
 
 }  // namespace
+
+__global__ void k_sqrt_f32(const float* __restrict__ x, long long n, float* __restrict__ root, float* __restrict__ ref) {
+    const long long step = 2LL * gridDim.x * blockDim.x;
+    for (long long i = 2 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < n; i += step) {
+        const bool two = i + 1 < n;
+        const float2 v = make_float2(x[i], two ? x[i + 1] : 1.f), r = sqrt_f2(v);
+        root[i] = r.x;
+        ref[i] = sqrtf(v.x);
+        if (two) {
+            root[i + 1] = r.y;
+            ref[i + 1] = sqrtf(v.y);
+        }
+    }
+}
+
+extern "C" sic_status sic_selftest_sqrt_f32(sic_handle* h, const float* x, int64_t n, float* root, float* ref,
+                                            void* stream) {
+    if (!h || n < 0 || (n > 0 && (!x || !root || !ref))) return SIC_ERR_INVALID;
+    if (n == 0) return SIC_OK;
+    SIC_CUDA_TRY(cudaSetDevice(h->device));
+    long long blocks = (n + 511) / 512;
+    if (blocks > 8LL * h->num_sms) blocks = 8LL * h->num_sms;
+    k_sqrt_f32<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(x, n, root, ref);
+    SIC_CUDA_TRY(cudaGetLastError());
+    return SIC_OK;
+}
 
 template <int NU>
 static sic_status launch_matvec_tc(sic_handle* h, const double* pts, long long n, const sic_kernel* kp, double shift,

@@ -35,7 +35,7 @@ EXPORTS = [
     "sic_build_factor", "sic_prep_partition", "sic_factor_nnz_range", "sic_build_factor_range", "sic_sum_fixed",
     "sic_apply_factor_workspace", "sic_apply_factor",
     "sic_matern_matvec", "sic_pcg_workspace", "sic_pcg_solve", "sic_selftest_wait_timeout",
-    "sic_selftest_fp64_math", "sic_selftest_matern_df", "sic_selftest_fixed_point",
+    "sic_selftest_fp64_math", "sic_selftest_matern_df", "sic_selftest_fixed_point", "sic_selftest_sqrt_f32",
     "sic_mlp_param_count", "sic_proposal_features", "sic_proposal_score",
     "sic_proposal_topk", "sic_proposal_labels", "sic_mlp_train_workspace", "sic_mlp_grads", "sic_adamw_step",
 ]
@@ -126,6 +126,7 @@ def lib():
             "sic_selftest_wait_timeout": (st, [vp, i64, vp, vp]),
             "sic_selftest_fp64_math": (st, [vp, pk, vp, i64, vp, vp, vp, vp, vp]),
             "sic_selftest_matern_df": (st, [vp, pk, vp, vp, i64, vp, vp]),
+            "sic_selftest_sqrt_f32": (st, [vp, vp, i64, vp, vp, vp]),
             "sic_selftest_fixed_point": (st, [vp, vp, vp, i64, i32, vp, vp, vp, vp, vp]),
             "sic_pcg_workspace": (st, [i64, i32, C.POINTER(sz)]),
             "sic_pcg_solve": (st, [vp, vp, i64, pk, d, st, vp, vp, vp, vp, vp, i32, d, i32, vp, vp, vp, sz, vp]),
@@ -729,6 +730,15 @@ def selftest_matern_df(h: Handle, kp: Kernel, pa, pb, stream=None):
                                         _dptr(out, torch.float64, "out"), _stream(stream)),
            "sic_selftest_matern_df", h)
     return out
+
+
+def selftest_sqrt_f32(h: Handle, x, stream=None):
+    """The kernel-matrix product's FP32 square root of x (CUDA float32), and the library's."""
+    import torch
+    root, ref = torch.empty_like(x), torch.empty_like(x)
+    _check(lib().sic_selftest_sqrt_f32(h.ptr, _dptr(x, torch.float32, "x"), x.numel(), _dptr(root, torch.float32, "root"),
+                                       _dptr(ref, torch.float32, "ref"), _stream(stream)), "sic_selftest_sqrt_f32", h)
+    return root, ref
 
 
 def gp_predict(h: Handle, pts, kp: Kernel, targets, sel_idx, sel_count, k: int, y, mean, var, stream=None):
