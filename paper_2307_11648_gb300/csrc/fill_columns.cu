@@ -10,6 +10,9 @@
 // added by warp reductions (three redux of 26-bit limbs).  The column is x = F^-T e_last: a back substitution in
 // FP64, b_i -= F_li x_l, lane = entry; log v = log of the target's pivot, 32 columns' logarithms at a time.
 //
+// The fixed point is absolute: a kernel entry below 2^-36 of the variance would keep fewer than 24 bits, one below 2^-60
+// none (points many length scales apart).  A column with such an entry is formed in FP64 by the same steps.
+//
 // The CTA-wide fill (k_fill) spends 5 warps and two barriers per panel on a 33 x 33 block: 65,536 columns of 32 picks
 // 4.19 ms; here 2.2 ms (2.3 with the pivots' reciprocal square roots in FP64).  Bound: the FP64 pipe (Theta's 8
 // operations per entry, the substitution: about 300 warp instructions per column of 32 picks).
@@ -41,7 +44,7 @@ __device__ __forceinline__ long long warp_sum(long long v) {
 
 // S sets of 32 picks
 template <int S>
-__global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
+__global__ void __launch_bounds__(32 * WARPS, S == 1 ? 9 : 5) k_fill_columns(
     const double* __restrict__ pts, int dim, KP<double> kp, int e, const int32_t* __restrict__ sel_idx,
     const int32_t* __restrict__ sel_count, int k, long long n, long long col0, long long n_cols,
     const long long* __restrict__ col_ptr, long long base, int32_t* __restrict__ row_idx, double* __restrict__ val,
@@ -117,9 +120,14 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
             for (int i = lane; i <= cnt; i += 32) xf[d * (k + 1) + i] = fx_coord(pts[(long long)pos[i] * dim + d], E[d]);
         }
         __syncwarp();
+        bool small_ = false;  // an entry that the fixed point holds to fewer than 24 bits
+        auto theta64 = [&](int i, int j) -> double {
+            return matern_d2_fast(kp, fx_dist2(xf, k + 1, dim, i, j, E[0], E[1], E[2]), tab);
+        };
         auto theta = [&](int i, int j) -> long long {
             const double d2 = fx_dist2(xf, k + 1, dim, i, j, E[0], E[1], E[2]);
             const double th = matern_d2_fast(kp, d2, tab);
+            small_ = small_ || (exponent_of(th) < 2 * e - 36 && __double_as_longlong(th) != 0LL);
             // (without a nugget coincident points make Theta singular, whatever the factorisation's rounding)
             return not_finite(th) || (d2 == 0.0 && !(kp.nugget > 0.0)) ? LLONG_MIN : fx_of_positive(th, FCS - 2 * e);
         };
@@ -150,9 +158,71 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
             rsd[s] = 0.0;
         }
         bool npd = __any_sync(FULL, nan_);
+        const bool wide = __any_sync(FULL, small_);
+        double b[S];  // the target's row in FP64, then the column
+        double d = 0.0;
+        if (wide) {
+            // ---- the same in FP64 (points many length scales apart): factor entries as doubles in the same words ----
+            auto at = [&](int j, int i) -> double& { return *reinterpret_cast<double*>(entry(j, i)); };
+            __syncwarp();
+            int i = (int)((sqrtf(8.0f * (float)lane + 1.0f) - 1.0f) * 0.5f);
+            while (i * (i + 1) / 2 > lane) --i;
+            while ((i + 1) * (i + 2) / 2 <= lane) ++i;
+            int j = lane - i * (i + 1) / 2;
+            while (i < cnt) {
+                at(j, i) = i == j ? kp.s2 + kp.nugget : theta64(i, j);
+                j += 32;
+                while (j > i) {
+                    j -= i + 1;
+                    ++i;
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < S; ++s) b[s] = lane + 32 * s < cnt ? theta64(cnt, lane + 32 * s) : 0.0;
+            __syncwarp();
+            auto sum64 = [&](double v) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+                return v;
+            };
+            for (int c = 0; c < cnt && !npd; ++c) {
+                double num[S], part = 0.0;
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    const int r = lane + 32 * s;
+                    const bool own = r >= c && r < cnt;
+                    num[s] = own ? at(c, r) : 0.0;
+                    for (int p = 0; p < c; ++p) num[s] = fma(-at(p, own ? r : c), at(p, c), num[s]);
+                    if (r < c) part = fma(b[s], at(r, c), part);
+                }
+                const double dot = sum64(part);
+                double dc = num[0];
+#pragma unroll
+                for (int s = 1; s < S; ++s) dc = (c >> 5) == s ? num[s] : dc;
+                dc = __shfl_sync(FULL, dc, c & 31);
+                npd = !(dc > 0.0);
+                const double rs = rsqrt_newton(npd ? 1.0 : dc);
+                __syncwarp();
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    const int r = lane + 32 * s;
+                    if (r >= c && r < cnt) at(c, r) = num[s] * rs;
+                    if (r == c) {
+                        rsd[s] = rs;
+                        b[s] = (b[s] - dot) * rs;
+                    }
+                }
+                __syncwarp();
+            }
+            double part = 0.0;
+#pragma unroll
+            for (int s = 0; s < S; ++s) part = fma(b[s], b[s], part);
+            d = kp.s2 + kp.nugget - sum64(part);
+            npd = npd || !(d > 0.0);
+        }
         __syncwarp();
         // ---- left-looking Cholesky ----
-        for (int j = 0; j < cnt && !npd; ++j) {
+        for (int j = 0; j < cnt && !npd && !wide; ++j) {
             const int pairs = j >> 1;
             FcSum a[S];
 #pragma unroll
@@ -229,16 +299,19 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
             part += b.hh * 2 + ((b.c1 + b.c2) >> 29);
         }
         const long long dt = diag_x - ((warp_sum(part) + 1) >> 1);
-        if (npd || dt <= 0) {
+        if (npd || (!wide && dt <= 0)) {
             if (lane == 0) record_error(st, SIC_ERR_NOT_PD, c);
             continue;
         }
         // ---- x = F^-T e_last ----
-        const double d = fx_to_double(dt, 2 * e - FCS);
-        const double xt = rsqrt_newton(d);
-        double b[S];
+        if (!wide) {
+            d = fx_to_double(dt, 2 * e - FCS);
 #pragma unroll
-        for (int s = 0; s < S; ++s) b[s] = lane + 32 * s < cnt ? -fx_to_double(tr[s], e - FCS) * xt : 0.0;
+            for (int s = 0; s < S; ++s) b[s] = lane + 32 * s < cnt ? fx_to_double(tr[s], e - FCS) : 0.0;
+        }
+        const double xt = rsqrt_newton(d);
+#pragma unroll
+        for (int s = 0; s < S; ++s) b[s] *= -xt;
 #pragma unroll
         for (int q = S - 1; q >= 0; --q)
             for (int l = min(31, cnt - 1 - 32 * q); l >= 0; --l) {
@@ -250,7 +323,9 @@ __global__ void __launch_bounds__(32 * WARPS) k_fill_columns(
                     const int i = lane + 32 * s;
                     if (i < r) {
                         const int2 f = *entry(i, r);
-                        b[s] = fma(-fx_to_double(((long long)f.x << 30) + f.y, e - FCS), x, b[s]);
+                        const double v = wide ? *reinterpret_cast<const double*>(&f)
+                                              : fx_to_double(((long long)f.x << 30) + f.y, e - FCS);
+                        b[s] = fma(-v, x, b[s]);
                     }
                 }
             }
