@@ -117,12 +117,14 @@ __global__ void __launch_bounds__(NT + 32, side_min_ctas(NT)) k_side(
     }
 }
 
-// ---- few units ----
+// ---- few or small units ----
 //
 // Both factorisations of a unit at once, right-looking over all 256 threads, two barriers per pivot.  It takes more
-// work than the panels, but a unit's chain is shorter and there is one launch of one class: while there are
-// few units per SM, that is the time.  N = 5,641 (262 units, k = 55) 260 us against 451 by the panels, 19,528 (857) 589
-// against 636; 48,858 (1,996) 1,400 against 1,225, 65,536 (2,796) 1,980 against 1,750.
+// work than the panels, but a unit's chain is shorter and there is one launch of one class: with few units per SM, or
+// few picks, that is the time.  Few units, k = 55: 262 260 us against 451 by the panels, 857 589 against 636; 1,121 with k = 64
+// 910 against 949, 1,410 1,177 against 1,042.  2,816 units of up to 64 members: k = 16 377 us against 442, 32 694 against 722,
+// 40 971 against 915, 64 1,994 against 1,884; of up to 24: 40 745 against 772, 48 990 each, 64 1,730 against 1,569;
+// 32,768 columns: k = 32 2.47 ms against 3.31, 64 9.98 against 10.12.
 constexpr int FLAT_NT = 256;
 
 struct FlatLayout {
@@ -214,6 +216,14 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
         if (!s_bad && cnt > 0) {
             // Theta over [P; S] (packed lower) and a copy of its S block
             const int tri = nn * (nn + 1) / 2;
+            if (singular)  // coincident points without a nugget, whatever rounding would leave of the pivot
+                for (int e = tid; e < tri; e += FLAT_NT) {
+                    int a, b;
+                    decode(e, a, b);
+                    const double dx = xyz[a] - xyz[b], dy = xyz[NMAX + a] - xyz[NMAX + b],
+                                 dz = xyz[2 * NMAX + a] - xyz[2 * NMAX + b];
+                    if (a != b && __double_as_longlong(fma(dz, dz, fma(dy, dy, dx * dx))) == 0LL) s_bad = 2;
+                }
             for (int e = tid; e < tri; e += FLAT_NT) {
                 int a, b;
                 decode(e, a, b);
@@ -221,10 +231,7 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
                 if (a != b) {
                     const double dx = xyz[a] - xyz[b], dy = xyz[NMAX + a] - xyz[NMAX + b],
                                  dz = xyz[2 * NMAX + a] - xyz[2 * NMAX + b];
-                    const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-                    // coincident points without a nugget: singular, whatever rounding leaves of the pivot
-                    if (singular && __double_as_longlong(d2) == 0LL) s_bad = 2;
-                    v = matern_d2_fast(kp, d2, tab);
+                    v = matern_d2_fast(kp, fma(dz, dz, fma(dy, dy, dx * dx)), tab);
                 }
                 A[e] = v;
                 if (b >= m) B[pk(a - m, b - m)] = v;
@@ -279,7 +286,8 @@ __global__ void __launch_bounds__(FLAT_NT) k_side_flat(const double* __restrict_
     }
 }
 
-constexpr int FLAT_UNITS_PER_SM = 7;
+constexpr int FLAT_UNITS_PER_SM = 8;
+constexpr int PANELS_K = 40, PANELS_ROWS = 72;  // least picks, and least rows of the largest unit, for the panels
 
 }  // namespace
 
@@ -300,7 +308,8 @@ extern "C" sic_status sic_side_state_fp64(sic_handle* h, const double* pts, int6
     F.k = k;
     F.dec = 1;
     if (F.bytes() > 227 * 1024 - 1024) F.dec = 0;
-    if (n_units <= (int64_t)FLAT_UNITS_PER_SM * h->num_sms && F.bytes() <= 227 * 1024 - 1024) {
+    const bool panels = n_units > (int64_t)FLAT_UNITS_PER_SM * h->num_sms && k >= PANELS_K && max_m + k >= PANELS_ROWS;
+    if (!panels && F.bytes() <= 227 * 1024 - 1024) {
         const size_t smem = F.bytes();
         SIC_CUDA_TRY(cudaFuncSetAttribute(k_side_flat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const int grid = persistent_grid(h, k_side_flat, FLAT_NT, smem, n_units);
