@@ -571,10 +571,13 @@ extern "C" sic_status sic_select_partial(sic_handle* h, const double* pts, int64
     cudaStream_t s = (cudaStream_t)stream;
     // Two size classes: a step's time is its chain of dependent operations, so two groups on an SM take little longer than
     // one.  Up to `two` members the state fits twice (256 candidates, k = 64 in FP32: 25 members).  N = 2^16, 2,811
-    // groups: 9.0 ms as one class, 7.1 as two.
+    // groups: 9.0 ms as one class, 7.1 as two.  But the two launches follow one another, so with few groups per SM one launch
+    // of one group per SM is shorter.  FP32, 256 candidates, k = 64: 88 groups 0.81 ms against 1.29, 173 1.42
+    // against 1.33, 342 1.87 against 1.42.  FP64, where two groups share the pipe they are bound by, 100 candidates, k = 20: 117 groups
+    // 3.1 ms against 5.6, 747 7.0 against 8.1, 989 9.7 against 9.0.
     int two = max_m;
     while (two > 0 && layout(two).bytes(tsz) > 227 * 1024 / 2 - PT_STATIC) --two;
-    if (two < PT_MIN_CLASS && two < max_m) two = 0;  // a few small groups are not worth a launch
+    if (two < max_m && (two < PT_MIN_CLASS || n_grp <= (prec == SIC_FP64 ? 5LL : 1LL) * h->num_sms)) two = 0;
     for (int c = 0; c < 2; ++c) {
         const int lo = c == 0 ? 1 : two + 1, hi = c == 0 ? two : max_m;
         if (lo > hi) continue;
