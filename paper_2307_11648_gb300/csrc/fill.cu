@@ -148,8 +148,9 @@ constexpr int fill_min_ctas(int nt) { return nt == 128 ? 5 : (nt == 256 ? 3 : 2)
 // PARTIAL: the units are nonadjacent groups, members[grp_ptr[u] ..) at any positions, whose picks condition only the
 // members before them (Section 5.1.1, Appendix A.4).  With the union of members and picks from the latest position to
 // the earliest, a member's set is a leading block of the same factorisation, so it is the same kernel with another
-// order and each member's own index jm in it (N = 2^16, 2,811 groups, k = 64: 1.4 ms; 4.2 ms by a
-// flat right-looking factorisation in FP64).
+// order and each member's own index jm in it.  It keeps FP64 throughout (ldl.cuh's F64 form, the substitution below):
+// N = 2^16, 2,811 groups, k = 64 2.0 ms; 4.2 ms by a flat right-looking factorisation in FP64 of lesser accuracy; 1.4 ms with the
+// consecutive groups' cut rows, 48-bit factor and double-float substitution, nine times the error.
 template <int FILL_NT, bool PARTIAL>
 __global__ void __launch_bounds__(FILL_NT + 32, fill_min_ctas(FILL_NT)) k_fill(const double* __restrict__ pts, int dim, KP<double> kp,
                                                   const long long* __restrict__ grp_ptr,

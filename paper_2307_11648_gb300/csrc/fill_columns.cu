@@ -14,7 +14,7 @@
 // none (points many length scales apart).  A column with such an entry is formed in FP64 by the same steps.
 //
 // The CTA-wide fill (k_fill) spends 5 warps and two barriers per panel on a 33 x 33 block: 65,536 columns of 32 picks
-// 4.19 ms; here 2.2 ms (2.3 with the pivots' reciprocal square roots in FP64).  Bound: the FP64 pipe (Theta's 8
+// 4.19 ms; here 2.3 ms.  Bound: the FP64 pipe (Theta's 8
 // operations per entry, the substitution: about 300 warp instructions per column of 32 picks).
 #include <limits.h>
 
@@ -369,7 +369,7 @@ sic_status launch(sic_handle* h, const double* pts, long long n, const sic_kerne
 
 }  // namespace
 
-// 16,384 columns: k = 32 0.62 against 1.07 ms, k = 48 1.52 against 1.76, k = 64 3.6 against 2.8 (few warps fit an SM then)
+// 16,384 columns: k = 32 0.66 against 1.07 ms, k = 48 1.57 against 1.76, k = 64 3.6 against 2.8 (few warps fit an SM then)
 bool fill_columns_applies(int k) { return k >= 1 && k <= 48; }
 
 sic_status launch_fill_columns(sic_handle* h, const double* pts, long long n, const sic_kernel* kp,

@@ -25,10 +25,10 @@
 // one of two buffers and one thread issues the MMAs, digit a against B_0 .. B_(8-a) into the columns from level a on (N a
 // multiple of 16; where that is one digit more than needed it lands in level 9, which is not read).  The MMAs run under the next step's evaluation; the accumulators (two sets) are read one chunk late.
 //
-// Bound: FP32 issue of the kernel evaluation and the digits, about 45 operations per entry whatever the
-// number of right-hand sides.  N = 50,001 with 8 of them: 16.6 ms with double-FP32 sums on the CUDA cores, 6.8 ms
-// now (N = 4096: 1.04 -> 0.086 ms); with sqrtf and a run-time smoothness, whose branches keep the evaluations from
-// overlapping, 11.2 ms.
+// Bound: FP32 issue of the kernel evaluation and the digits, about 50 operations per entry whatever the
+// number of right-hand sides.  N = 50,001 with 8 of them: 16.6 ms with double-FP32 sums on the CUDA cores, 8.0 ms
+// now (N = 4096: 1.04 -> 0.125 ms); 6.8 ms with six digits and no check; with sqrtf and a run-time smoothness, whose branches
+// keep the evaluations from overlapping, half as much again.
 #include "matvec_f32.cuh"
 #include "tc_common.cuh"
 

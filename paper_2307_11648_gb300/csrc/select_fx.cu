@@ -35,7 +35,7 @@
 // Bound: latency of the step's phases (with 1024 candidates per supernode 44 % of the issue slots and
 // 35 % of the FP64 pipe are busy, L2 delivers 30 bytes per clock and SM); half of each scheduler's warps therefore
 // evaluate Theta while the others sum.  N = 2^16 with 1024 candidates, k = 64 (2,811 supernodes): 61.3 ms with FP64
-// multiply-adds over FP64 rows, 19.2 ms now; 4096 columns of 256 candidates, k = 16: 2.30 -> 0.82 ms.  One row per thread
+// multiply-adds over FP64 rows, 19.2 ms now; 4096 columns of 256 candidates, k = 16: 2.30 -> 0.83 ms.  One row per thread
 // at 64 registers (1024 threads per SM) is faster than two rows per thread at 128 (26.2 ms).
 #include "fx.cuh"
 

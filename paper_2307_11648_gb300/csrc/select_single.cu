@@ -20,11 +20,12 @@
 //
 // (A best covariance below 2^-30 of the variance starts over with the rows in FP64, as in select_fx.cu.)
 //
-// Bound: a barrier and four dependent L2 round trips per step, then the factor's L2 traffic (4 n k^2 bytes) and the FP64
-// pipe.  One block on one SM was the whole kernel: 98.3 ms for n = 65,536, k = 64 in FP64 (3-D, Matern 5/2); over
-// the grid with FP64 multiply-adds and divisions 1.16 ms, in fixed point 0.85 ms.
-// Error of out_var against 128-bit arithmetic over six problems (n 300 .. 4000, k 30 .. 64): 2.0e-15 on average, 2.2e-15
-// with the library exponential and FP64 sums.
+// Bound: a barrier and three dependent L2 round trips per step (slots; the pivot's coordinates and row), then the factor's L2
+// traffic (4 n k^2 bytes) and the FP64 pipe.  One block on one SM was the whole kernel: 98.3 ms for n = 65,536, k = 64 in FP64 (3-D, Matern 5/2); over
+// the grid with FP64 multiply-adds and divisions 1.16 ms, in fixed point 0.86 ms.
+// Error of out_var against 128-bit arithmetic over 48 problems (n 700 .. 65,536, k 30 .. 64, nugget 1e-8 .. 1e-2; variance 1):
+// 1.7e-16 on average, 9e-16 at most; with the library exponential and FP64 sums 2.0e-16 and 1.5e-15.  Either is a
+// few roundings of out_var itself; single problems go either way.
 #include "fx.cuh"
 
 namespace {
