@@ -62,7 +62,8 @@ typedef struct {
 
 /* Arithmetic of the selection kernels.  The fill and the KL sum are always FP64.
  * SIC_FP64 evaluates the kernel with a table-driven exp and Newton square roots (about
- * 2 ulp) and holds factor entries in 58-bit fixed point, their products summed exactly;
+ * 2 ulp) and holds factor entries in 58-bit fixed point, their products summed exactly (in
+ * FP64 for a column whose covariances fall below 2^-30 of the variance);
  * SIC_FP32_MIXED uses the hardware's approximate reciprocal, reciprocal square
  * root and exp (a few ulp of FP32), far below the FP32 state's own resolution. */
 typedef enum {
